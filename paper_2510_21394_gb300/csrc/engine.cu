@@ -12,12 +12,14 @@
 // Lam o U^_n + G^_n with U^_n = Q^T u_n carried from step to step
 // (U^_{n+1} = U^_n + S when u_{n+1} = u_n + bwd(S)), which replaces the
 // paper's explicit K u_n (Eq. krogstad-m) and saves a Tucker operator.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <cstdint>
 
 #include "adjoint.h"
 #include "engine.h"
+#include "sliced.h"
 
 namespace fcgle {
 
@@ -137,6 +139,33 @@ class Engine : public EngineBase {
       mf64_[mu][1].reset(new DevBuf<double>(Mb.size()));
       FCGLE_CUDA(cudaMemcpy(mf64_[mu][0]->ptr, Mf.data(), Mf.size() * 8, cudaMemcpyHostToDevice));
       FCGLE_CUDA(cudaMemcpy(mf64_[mu][1]->ptr, Mb.data(), Mb.size() * 8, cudaMemcpyHostToDevice));
+    }
+    // ---- sliced products: digits of the matrices, workspace for those of the data
+    size_t xbytes = 0;
+    long long xrows = 0;
+    for (int mu = 0; mu < prm.d; ++mu)
+      for (int cx = 0; cx < 2; ++cx) {
+        Sliced& x = xs_[mu][cx];
+        x.rows = (long long)(s_.P / s_.p[mu]) * (cx ? 1 : 2);
+        x.K = s_.p[mu] * (cx ? 2 : 1);
+        if (!sliceable(x.K, x.rows)) continue;
+        xbytes = std::max(xbytes, slice_bytes<double>(x.rows, x.K));
+        xrows = std::max(xrows, x.rows);
+      }
+    if (xbytes) {
+      xdig_.reset(new DevBuf<uint8_t>(xbytes));
+      xex_.reset(new DevBuf<int>((size_t)xrows));
+    }
+    for (int mu = 0; mu < prm.d; ++mu) {
+      for (int cx = 0; cx < 2; ++cx) {
+        Sliced& x = xs_[mu][cx];
+        if (!sliceable(x.K, x.rows)) continue;
+        x.dig = reinterpret_cast<__nv_bfloat16*>(xdig_->ptr);
+        x.ex = xex_->ptr;
+        slice_map<double>(x, false);
+      }
+      if (sliceable(xs_[mu][0].K, xs_[mu][0].rows))
+        for (int f = 0; f < 2; ++f) ms_[mu][f].build(mf64_[mu][f]->ptr, s_.p[mu], st_, launches);
     }
     lv_.c_re = prm.nu;
     lv_.c_im = prm.eta;
@@ -339,9 +368,40 @@ class Engine : public EngineBase {
   static bool needs_uhat(int scheme) { return scheme == FCGLE_ETD2RK || scheme == FCGLE_KROGSTAD; }
 
   // ---- building blocks
+  // digits of a square matrix of order K (row-major, on the device)
+  struct SlicedMat {
+    Sliced s;
+    std::unique_ptr<DevBuf<uint8_t>> dig;
+    std::unique_ptr<DevBuf<int>> ex;
+    void build(const double* M, int K, cudaStream_t st, long long& nl) {
+      s.rows = s.K = K;
+      dig.reset(new DevBuf<uint8_t>(slice_bytes<double>(K, K)));
+      ex.reset(new DevBuf<int>((size_t)K));
+      s.dig = reinterpret_cast<__nv_bfloat16*>(dig->ptr);
+      s.ex = ex->ptr;
+      slice_map<double>(s, true);
+      slice_rows<double>(M, s, 1, K, 0, st, nl);
+    }
+  };
+  // The sliced product (two launches) against the CUDA cores, us: 12.6 / 21.0 at
+  // K = 16 with 32 rows, 15.0 / 70 at 64 x 64, 18 / 150 at K = 132 with 8 rows;
+  // shorter contractions are one k-step of the CUDA-core tile and stay there.
+  static bool sliceable(int K, long long rows) { return kF64 && K >= 16 && rows < (1ll << 31); }
+  // one mode product: cx = 0 with the real matrix m of order p, cx = 1 with the
+  // real block form (order 2 p) of a complex one.  M: its FP64 elements.
+  void product(const T* X, T* Y, int mu, int cx, const double* M, const SlicedMat& m) {
+    const long long R = (long long)(s_.P / s_.p[mu]);
+    const Sliced& x = xs_[mu][cx];
+    if (m.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
+      const long long plane = R * s_.p[mu];
+      slice_rows<double>(X, x, cx ? 2 : 1, s_.p[mu], plane, st_, launches);
+      sliced_gemm<double>(x, m.s, Y, R, plane, err_->ptr, st_, launches);
+      return;
+    }
+    mp_f64(X, Y, M, s_.p[mu], (size_t)R, cx != 0, st_, launches);
+  }
   void mp(const T* X, T* Y, int mu, bool fwd) {
-    const size_t R = s_.P / s_.p[mu];
-    mp_f64(X, Y, mf64_[mu][fwd ? 0 : 1]->ptr, s_.p[mu], R, false, st_, launches);
+    product(X, Y, mu, 0, mf64_[mu][fwd ? 0 : 1]->ptr, ms_[mu][fwd ? 0 : 1]);
   }
 
   // Tucker operator over directions 1..d in the rotating order; Y may equal X.
@@ -373,7 +433,7 @@ class Engine : public EngineBase {
       for (int mu = 0; mu < s_.d; ++mu) {
         T* out = (mu == s_.d - 1) ? Y : B(mu % 2 == 0 ? kT0 : kT1);
         if (out == in) out = B(kW);
-        mp_f64(in, out, E[mu]->ptr, s_.p[mu], s_.P / s_.p[mu], true, st_, launches);
+        product(in, out, mu, 1, E[mu].f64->ptr, E[mu].sl);
         in = out;
       }
       if (in != Y) FCGLE_CUDA(cudaMemcpyAsync(Y, in, 2 * s_.P * sizeof(T), cudaMemcpyDeviceToDevice, st_));
@@ -426,7 +486,11 @@ class Engine : public EngineBase {
   }
 
   // E_mu = Q diag(exp(theta (nu + i eta) lam)) Q^T in real block form, cached
-  std::vector<std::unique_ptr<DevBuf<double>>>& Emat(double theta) {
+  struct EMat {
+    std::unique_ptr<DevBuf<double>> f64;
+    SlicedMat sl;
+  };
+  std::vector<EMat>& Emat(double theta) {
     auto key = dbits(theta);
     auto it = ecache_.find(key);
     if (it != ecache_.end()) return it->second;
@@ -460,8 +524,10 @@ class Engine : public EngineBase {
             Bm[(size_t)(p + a) * K + p + b] = sr; // (im out, im in)
           }
         }
-      v.emplace_back(new DevBuf<double>(Bm.size()));
-      FCGLE_CUDA(cudaMemcpyAsync(v.back()->ptr, Bm.data(), Bm.size() * 8, cudaMemcpyHostToDevice, st_));
+      v.emplace_back();
+      v.back().f64.reset(new DevBuf<double>(Bm.size()));
+      FCGLE_CUDA(cudaMemcpyAsync(v.back().f64->ptr, Bm.data(), Bm.size() * 8, cudaMemcpyHostToDevice, st_));
+      if (sliceable(xs_[mu][1].K, xs_[mu][1].rows)) v.back().sl.build(v.back().f64->ptr, 2 * p, st_, launches);
       FCGLE_CUDA(cudaStreamSynchronize(st_));
     }
     return v;
@@ -667,7 +733,11 @@ class Engine : public EngineBase {
   std::unique_ptr<DevBuf<double>> scratch_;
   std::unique_ptr<DevBuf<int>> err_;
   std::map<std::tuple<int, int, uint64_t>, std::unique_ptr<DevBuf<T>>> fcache_;
-  std::map<uint64_t, std::vector<std::unique_ptr<DevBuf<double>>>> ecache_;
+  std::map<uint64_t, std::vector<EMat>> ecache_;
+  SlicedMat ms_[kMaxDim][2];
+  Sliced xs_[kMaxDim][2];   // digits of the data as direction mu's product reads them (real, complex block form)
+  std::unique_ptr<DevBuf<uint8_t>> xdig_;
+  std::unique_ptr<DevBuf<int>> xex_;
   std::vector<std::unique_ptr<DevBuf<T>>> adj_mem_;
 };
 

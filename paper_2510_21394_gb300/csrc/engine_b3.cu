@@ -15,7 +15,6 @@
 // carried): 4 forward + 4 backward Tucker operators = 24 launches for d = 3.
 #include <cuda.h>
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
 
 #include <cmath>
 #include <cstddef>
@@ -35,6 +34,8 @@
 #include "b3_plain.cuh"
 #include "b3_slab.cuh"
 #include "engine.h"
+#include "sliced.h"
+#include "tma_host.h"
 
 namespace fcgle {
 
@@ -53,33 +54,6 @@ struct DevMem {
   DevMem(const DevMem&) = delete;
   DevMem& operator=(const DevMem&) = delete;
 };
-
-// Programmatic dependent launch of the mode-product kernels (on unless the
-// environment sets FCGLE_PDL=0): the kernel may be scheduled while the previous
-// kernel of the stream drains and runs its prologue meanwhile; it waits for
-// that kernel's completion (griddepcontrol.wait) before any global access.
-bool pdl_enabled() {
-  static const bool on = [] {
-    const char* e = std::getenv("FCGLE_PDL");
-    return !(e && e[0] == '0');
-  }();
-  return on;
-}
-
-template <class... P, class... A>
-void launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl_enabled() ? 1 : 0;
-  FCGLE_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
-}
 
 // ------------------------------------------------ plain-product autotuner
 // Ring configurations of the plain mode product (b3_plain.cuh); which one is
@@ -175,28 +149,6 @@ std::string plain_tune_report() {
 }
 
 namespace {
-
-int num_sms() {
-  static const int sms = [] {   // thread-safe one-time initialisation
-    int dev = 0, m = 0;
-    FCGLE_CUDA(cudaGetDevice(&dev));
-    FCGLE_CUDA(cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev));
-    return m;
-  }();
-  return sms;
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    cudaDriverEntryPointQueryResult q;
-    void* p = nullptr;
-    FCGLE_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q));
-    if (q != cudaDriverEntryPointSuccess || !p) throw std::runtime_error("cuTensorMapEncodeTiled unavailable");
-    fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
 
 // 2D bf16 tensor map, SWIZZLE_128B, box (64 inner, box_rows outer).
 void encode_bf16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
@@ -464,6 +416,30 @@ class EngineB3 : public EngineBase {
       f32_[i].reset(new DevMem<float>(2 * s_.P));
       FCGLE_CUDA(cudaMemsetAsync(f32_[i]->ptr, 0, 2 * s_.P * 4, st_));
     }
+    if (use_sliced()) {
+      // digits [3][2 R][p] bf16 = 12 P bytes of one direction at a time, then 2 R exponents
+      size_t rows = 0;
+      for (int mu = 0; mu < prm.d; ++mu) rows = std::max(rows, 2 * s_.P / (size_t)s_.p[mu]);
+      xdig_.reset(new DevMem<__nv_bfloat16>(6 * s_.P));
+      xex_.reset(new DevMem<int>(rows));
+      for (int mu = 0; mu < prm.d; ++mu) {
+        if (!sliceable(mu)) continue;
+        Sliced& x = xs_[mu];
+        x.dig = xdig_->ptr;
+        x.ex = xex_->ptr;
+        x.rows = 2 * (P_ / s_.p[mu]);
+        x.K = s_.p[mu];
+        slice_map<float>(x, false);
+        for (int f = 0; f < 2; ++f) {
+          Mat& m = mat_[mu][f];
+          m.sl.rows = m.sl.K = m.p;
+          FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<float>(m.p, m.p)));
+          FCGLE_CUDA(cudaMalloc(&m.sl.ex, m.p * sizeof(int)));
+          slice_map<float>(m.sl, true);
+          slice_rows<float>(m.f32, m.sl, 1, m.p, 0, st_, launches);
+        }
+      }
+    }
     for (int i = 0; i < kNumSplit; ++i) {
       sp_[i].reset(new DevMem<__nv_bfloat16>(4 * s_.P));
       FCGLE_CUDA(cudaMemsetAsync(sp_[i]->ptr, 0, 4 * s_.P * 2, st_));
@@ -537,6 +513,8 @@ class EngineB3 : public EngineBase {
         if (mat_[mu][f].f32) cudaFree(mat_[mu][f].f32);
         if (mat_[mu][f].thi) cudaFree(mat_[mu][f].thi);
         if (mat_[mu][f].tlo) cudaFree(mat_[mu][f].tlo);
+        if (mat_[mu][f].sl.dig) cudaFree(mat_[mu][f].sl.dig);
+        if (mat_[mu][f].sl.ex) cudaFree(mat_[mu][f].sl.ex);
       }
   }
 
@@ -621,7 +599,7 @@ class EngineB3 : public EngineBase {
         FCGLE_LAUNCHED(launches);
         launch_tf32(ah, al, mu, fwd, (float*)Y, nullptr);
       } else {
-        mp_f32((const float*)X, (float*)Y, mat_[mu][fwd ? 0 : 1].f32, s_.p[mu], (size_t)R, st_, launches);
+        mp_precise((const float*)X, (float*)Y, mu, fwd);
       }
       return;
     }
@@ -783,7 +761,8 @@ class EngineB3 : public EngineBase {
   struct Mat {
     __nv_bfloat16* hi = nullptr;
     __nv_bfloat16* lo = nullptr;
-    float* f32 = nullptr;   // p x p FP32 (the CUDA-core form of the precise transforms, d == 1)
+    float* f32 = nullptr;   // p x p FP32 (the CUDA-core form of the precise transforms)
+    Sliced sl;              // its digits (the sliced form)
     // split-TF32 hi / lo (m_pad x k_pad32): the tensor-core form of the precise transforms
     float* thi = nullptr;
     float* tlo = nullptr;
@@ -1007,17 +986,18 @@ class EngineB3 : public EngineBase {
   // most kTf32MaxP long: the tensor core's FP32 accumulation of the three
   // products adds an error that grows with the contracted length (measured
   // 2.4e-6 at p = 264; at p = 1024 it lifted the error at T of 500 steps from
-  // 1.6e-6 to 8.5e-6).  FP32 on the CUDA cores otherwise, and always when
-  // tc_ok is false (the adjoint, whose misfit compares nearby states).
+  // 1.6e-6 to 8.5e-6).  Longer contractions: the sliced product (sliced.cu),
+  // whose accumulation is exact (1e-7 at p = 1024, FP32 on the CUDA cores
+  // 8e-7).  FP32 on the CUDA cores for d = 1 and where tc_ok is false (the
+  // adjoint).
   static constexpr int kTf32MaxP = 256;
   void tucker_f32(const float* X, float* Y, bool fwd, bool tc_ok = true) {
-    bool tc = tc_ok && s_.d >= 2;
-    for (int mu = 0; mu < s_.d && tc; ++mu) tc = (P_ / s_.p[mu]) % 8 == 0 && s_.p[mu] <= kTf32MaxP;
-    if (tc) {
+    if (tc_ok && tf32_ok())
       tucker_tf32(X, Y, fwd);
-      return;
-    }
-    tucker_simt(X, Y, fwd);
+    else if (tc_ok && use_sliced())
+      tucker_fp32<true>(X, Y, fwd);
+    else
+      tucker_fp32<false>(X, Y, fwd);
   }
 
   // The split-TF32 intermediates (hi and lo, 2 P floats each) live in four of
@@ -1064,12 +1044,39 @@ class EngineB3 : public EngineBase {
     FCGLE_LAUNCHED(launches);
   }
 
-  void tucker_simt(const float* X, float* Y, bool fwd) {
+  bool tf32_ok() const {
+    bool tc = s_.d >= 2;
+    for (int mu = 0; mu < s_.d && tc; ++mu) tc = (P_ / s_.p[mu]) % 8 == 0 && s_.p[mu] <= kTf32MaxP;
+    return tc;
+  }
+  bool sliceable(int mu) const { return s_.p[mu] >= 16; }
+  bool use_sliced() const {
+    bool any = false;
+    for (int mu = 0; mu < s_.d; ++mu) any = any || sliceable(mu);
+    return s_.d >= 2 && !tf32_ok() && any;
+  }
+  // one precise product, FP32 in and out, without the split-TF32 form
+  void mp_precise(const float* X, float* Y, int mu, bool fwd) {
+    const Mat& m = mat_[mu][fwd ? 0 : 1];
+    const long long R = P_ / s_.p[mu];
+    if (m.sl.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
+      slice_rows<float>(X, xs_[mu], 1, s_.p[mu], 0, st_, launches);
+      sliced_gemm<float>(xs_[mu], m.sl, Y, R, P_, err_->ptr, st_, launches);
+    } else {
+      mp_f32(X, Y, m.f32, s_.p[mu], (size_t)R, st_, launches);
+    }
+  }
+
+  template <bool Sliced>
+  void tucker_fp32(const float* X, float* Y, bool fwd) {
     float* tmp[2] = {F32(kFh), F32(kD2)};
     const float* src = X;
     for (int mu = 0; mu < s_.d; ++mu) {
       float* dst = mu == s_.d - 1 ? Y : tmp[mu % 2];
-      mp_f32(src, dst, mat_[mu][fwd ? 0 : 1].f32, s_.p[mu], (size_t)(P_ / s_.p[mu]), st_, launches);
+      if (Sliced)
+        mp_precise(src, dst, mu, fwd);
+      else
+        mp_f32(src, dst, mat_[mu][fwd ? 0 : 1].f32, s_.p[mu], (size_t)(P_ / s_.p[mu]), st_, launches);
       src = dst;
     }
   }
@@ -1694,6 +1701,10 @@ class EngineB3 : public EngineBase {
   b3::GStatic gs_{};
   double sig_re_[kMaxSrc] = {0, 0, 0, 0}, sig_im_[kMaxSrc] = {0, 0, 0, 0};
   std::unique_ptr<DevMem<float>> f32_[kNumF32];
+  // digits of the data as direction mu's sliced product reads them, and their buffers
+  Sliced xs_[kMaxDim];
+  std::unique_ptr<DevMem<__nv_bfloat16>> xdig_;
+  std::unique_ptr<DevMem<int>> xex_;
   std::unique_ptr<DevMem<__nv_bfloat16>> sp_[kNumSplit];
   std::unique_ptr<DevMem<float>> src_[kMaxSrc];
   std::unique_ptr<DevMem<float>> host_stage_;

@@ -1,0 +1,497 @@
+// Mode products in FP64 and in precise FP32 on the bf16 tensor cores.
+//
+// An FP64 multiply-add on GB300's CUDA cores runs at about 1.1 TFLOP/s per
+// GPU, the bf16 tensor cores at 1.9 PFLOP/s: 28 bf16 products of integer
+// slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59 (2012)) are far cheaper than one FP64 product.  Both operands
+// are written as fixed-point numbers with one exponent per row (per fiber of
+// the contracted index), cut into NS balanced digits of RB bits, which bf16
+// holds exactly, and
+//     Y[i][r] = 2^{E_i + E_r} sum_s 2^{RB (2 NS - 2 - s)} P_s,
+//     P_s = sum_{a + b = s} sum_k m_a[i][k] x_b[r][k],   s < NLEV,
+// where every P_s is a sum of integers that the FP32 accumulator holds exactly
+// (products of the top digits <= 2^14, 2^24 over 1024 of them; longer
+// contractions go in segments).  The levels s >= NLEV are below the rounding of T.  The epilogue
+// adds the levels as 64-bit integers (FP64 arithmetic would cost more than the
+// product) and rounds once.
+//
+// Orientation: the data rows (c, r) are the MMA's M (TMEM lanes), so that a
+// warp stores 32 consecutive r of one output index i; 64 (FP64) or 128 (FP32)
+// output indices are the N of one level.  The digits b of one data row block
+// follow each other in shared memory, and so do those of the matrix: one MMA
+// takes slice a of the data against several slices b of the matrix (N up to
+// 256) and adds into the neighbouring levels a + b, which lie side by side in
+// tensor memory.
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <mutex>
+#include <string>
+
+#include "b3_kernel.cuh"
+#include "sliced.h"
+#include "tma_host.h"
+
+namespace fcgle {
+
+namespace {
+
+using namespace b3;
+
+constexpr int kSliceBad = 0x40000000;   // exponent of a row that holds a NaN or an Inf
+
+// ------------------------------------------------------------ slicing pass
+// HBM-bound (FP64: 8 bytes read and 14 written per element), so one pass: a
+// group of 8, 16 or 32 lanes owns a row, finds its largest exponent, and cuts
+// the elements (read again, from L1 or L2) with integer shifts; no FP64
+// arithmetic.
+template <typename T>
+struct Bits;
+template <>
+struct Bits<double> {
+  using U = unsigned long long;
+  static constexpr int kMant = 52, kExpMask = 0x7ff;
+};
+template <>
+struct Bits<float> {
+  using U = unsigned int;
+  static constexpr int kMant = 23, kExpMask = 0xff;
+};
+
+template <typename T>
+__device__ __forceinline__ void load4(const T* p, typename Bits<T>::U (&u)[4]) {
+  if constexpr (sizeof(T) == 8) {
+    const ulonglong2 a = reinterpret_cast<const ulonglong2*>(p)[0], b = reinterpret_cast<const ulonglong2*>(p)[1];
+    u[0] = a.x; u[1] = a.y; u[2] = b.x; u[3] = b.y;
+  } else {
+    const uint4 a = *reinterpret_cast<const uint4*>(p);
+    u[0] = a.x; u[1] = a.y; u[2] = a.z; u[3] = a.w;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
+                                                    long long seg_stride, int pitch, int group,
+                                                    __nv_bfloat16* __restrict__ dig, int* __restrict__ ex) {
+  using U = typename Bits<T>::U;
+  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant;
+  constexpr U kMantMask = (U(1) << MB) - 1;
+  constexpr int UP = SliceCfg<T>::BITS - MB - 2;   // spare bits below the last one of the largest entry
+  pdl_trigger();
+  pdl_wait();
+  const int per_block = 256 / group;
+  const int lig = threadIdx.x % group;
+  const int quads = seg_len / 4;
+  for (long long row0 = (long long)blockIdx.x * per_block; row0 < rows; row0 += (long long)gridDim.x * per_block) {
+    const long long row = row0 + threadIdx.x / group;
+    const bool live = row < rows;
+    int emax = 1;
+    if (live)
+      for (int c = 0; c < nseg; ++c) {
+        const T* src = X + c * seg_stride + row * seg_len;
+        for (int q = lig; q < quads; q += group) {
+          U u[4];
+          load4<T>(src + 4 * q, u);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) emax = max(emax, (int)((u[v] >> MB) & Bits<T>::kExpMask));
+        }
+      }
+    for (int o = group / 2; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    if (!live) continue;
+    const bool bad = emax == Bits<T>::kExpMask;
+    // x = mant 2^{e - bias - MB}; v = (mant << UP) >> (emax - e): unit 2^{emax - bias - MB - UP}
+    if (lig == 0) ex[row] = bad ? kSliceBad : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
+    for (int c = 0; c < nseg; ++c) {
+      const T* src = X + c * seg_stride + row * seg_len;
+      __nv_bfloat16* dst = dig + row * pitch + c * seg_len;
+      for (int q = lig; q < quads; q += group) {
+        U u[4];
+        load4<T>(src + 4 * q, u);
+        long long w[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int e = (int)((u[v] >> MB) & Bits<T>::kExpMask);
+          const unsigned long long mant = ((unsigned long long)(u[v] & kMantMask) | (e ? 1ull << MB : 0ull)) << UP;
+          const int s = emax - max(e, 1);
+          const unsigned long long m = s < 62 ? (mant + ((1ull << s) >> 1)) >> s : 0ull;
+          long long x = (u[v] >> (8 * sizeof(U) - 1)) ? -(long long)m : (long long)m;
+          if (bad) x = 0;
+          // balanced digits: add half a digit at every place but the top one
+          long long off = 0;
+#pragma unroll
+          for (int j = 0; j + 1 < NS; ++j) off += 1ll << (RB * j + RB - 1);
+          w[v] = x + off;
+        }
+#pragma unroll
+        for (int a = 0; a < NS; ++a) {
+          uint32_t h[4];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            // digit as a small integer, exact in bf16 (at most 8 significant bits)
+            const int d = a == 0 ? (int)(w[v] >> (RB * (NS - 1)))
+                                 : ((int)(w[v] >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
+            h[v] = __float_as_uint((float)d);
+          }
+          uint2 o;
+          o.x = (h[0] >> 16) | (h[1] & 0xFFFF0000u);
+          o.y = (h[2] >> 16) | (h[3] & 0xFFFF0000u);
+          *reinterpret_cast<uint2*>(dst + (size_t)a * rows * pitch + 4 * q) = o;
+        }
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------ product
+// Measured with the slicing pass (one real product, GB300): FP64 128 x 120 x 136
+// 73 us (900 us on the CUDA cores, whose FP64 rate is 1.1 TFLOP/s), 400 x 400 30
+// (414), 1023 x 1024 107 (4090), 432 x 432 x 100 926 (27010); relative error
+// 1.0e-16 .. 1.4e-16 (2.5e-16 .. 1.1e-15).  FP32 1023 x 1024 48 us (150), 432 x
+// 432 x 100 399 (1080); error 5e-8 (4e-7 .. 6e-7).
+// What bounds it: the bf16 tensor cores and, close behind, the operand bytes
+// an SM pulls from L2 (FP64: 84 KB per 32 k against 1792 MMA clocks, 47 bytes
+// per clock).  All levels of a tile share tensor memory (FP64 7 x 64, FP32
+// 4 x 128 columns), so the accumulators are single-buffered and the MMAs of
+// the next tile wait while the epilogue reads them; the stores overlap.
+template <typename T>
+struct GemmCfg;
+template <>
+struct GemmCfg<double> {
+  static constexpr int NLEV = 7, NT = 64, NSTAGE = 2;
+};
+template <>
+struct GemmCfg<float> {
+  static constexpr int NLEV = 4, NT = 128, NSTAGE = 4;
+};
+
+constexpr int kSegK = 1024;     // longest contraction whose digit sums stay exact (below 2^24)
+constexpr int kGK = 32;         // k per stage: 64-byte bf16 rows, 64-byte swizzle
+constexpr int kGM = 128;        // data rows per tile
+constexpr int kGEpi = 8;        // epilogue warps
+constexpr int kGThreads = 32 * (2 + kGEpi);
+
+template <typename T>
+struct GemmLayout {
+  static constexpr int NS = SliceCfg<T>::NS;
+  static constexpr uint32_t kA = kGM * 64, kB = GemmCfg<T>::NT * 64;   // bytes of one slice of a chunk
+  static constexpr uint32_t kStage = NS * (kA + kB);
+  static constexpr uint32_t kOffBar = GemmCfg<T>::NSTAGE * kStage;
+  static constexpr uint32_t kSmem = kOffBar + 256 + 1024;
+  static_assert(kSmem <= 232448, "shared memory budget");
+  static_assert(GemmCfg<T>::NLEV * GemmCfg<T>::NT <= 512, "tensor memory columns");
+  static_assert(kStage % 1024 == 0 && kA % 1024 == 0 && kB % 1024 == 0, "slices start on swizzle atoms");
+};
+
+struct GemmParams {
+  long long rows;    // data rows
+  long long R;       // rows per plane of the output
+  long long plane;   // elements between the planes of Y
+  int m;             // output indices
+  int m_tiles, k_chunks;
+  long long units;
+  int kb;            // bits of the contraction length (FP64 epilogue)
+  int* err;
+};
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
+}
+// K-major, SWIZZLE_64B: rows of 64 bytes, 8-row groups 512 bytes apart
+__device__ __forceinline__ uint64_t desc64(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+}
+
+// The levels of one output, added up exactly: FP64 as V = 2^24 hi + lo, FP32
+// from the smallest level up.  add() takes the levels of one segment of the
+// contraction, get() gives the sum times 2^e.
+template <typename T>
+struct Sum;
+template <>
+struct Sum<double> {
+  long long hi = 0, lo = 0;
+  __device__ __forceinline__ void add(const float (&P)[7]) {
+    hi += ((long long)__float2int_rn(P[0]) << 24) + ((long long)__float2int_rn(P[1]) << 16) +
+          ((long long)__float2int_rn(P[2]) << 8) + (long long)__float2int_rn(P[3]);
+    lo += ((long long)__float2int_rn(P[4]) << 16) + ((long long)__float2int_rn(P[5]) << 8) +
+          (long long)__float2int_rn(P[6]);
+  }
+  // |hi| < 2^{39 + kb}: rounded to 53 bits through a 63-bit integer, V itself
+  // where it fits, else V / 2^kb, which then still has at least 62 - kb >= 52 bits
+  __device__ __forceinline__ double get(int e, int kb) const {
+    const int s = (hi + (1ll << 38)) >> 39 == 0 ? 0 : kb;
+    const long long t = (hi << (24 - s)) + ((lo + ((1ll << s) >> 1)) >> s);
+    if (t == 0) return 0.0;
+    const double d = (double)t;
+    const int k = e + 48 + s;
+    // d has an exponent in [0, 63]: scale by adding to its exponent field while the result is normal
+    if (k > -1000 && k < 900) return __longlong_as_double(__double_as_longlong(d) + ((long long)k << 52));
+    return ldexp(d, k);
+  }
+};
+template <>
+struct Sum<float> {
+  float t = 0.f;
+  __device__ __forceinline__ void add(const float (&P)[4]) {
+    t += fmaf(fmaf(fmaf(P[3], 1.f / 512.f, P[2]), 1.f / 512.f, P[1]), 1.f / 512.f, P[0]);
+  }
+  __device__ __forceinline__ float get(int e, int) const {
+    const int k = e + 36;
+    if (k >= -126 && k <= 127) return t * __int_as_float((k + 127) << 23);
+    return ldexpf(t, k);
+  }
+};
+
+template <typename T>
+__device__ __forceinline__ T finish(const Sum<T>& s, int er, int i, const int* em, const GemmParams& gp) {
+  const int ei = i < gp.m ? __ldg(em + i) : 0;
+  return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei, gp.kb);
+}
+
+// SEG: contractions longer than kSegK go in segments, each drained from tensor
+// memory into the integer sums before the next begins.
+template <typename T, bool SEG>
+__global__ void __launch_bounds__(kGThreads, 1)
+    sliced_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_m,
+                       const int* __restrict__ ex, const int* __restrict__ em, T* __restrict__ Y,
+                       const GemmParams gp) {
+  using L = GemmLayout<T>;
+  constexpr int NS = SliceCfg<T>::NS, NLEV = GemmCfg<T>::NLEV, NT = GemmCfg<T>::NT, NSTAGE = GemmCfg<T>::NSTAGE;
+  extern __shared__ uint8_t smem_raw[];
+  pdl_trigger();
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t sbase = smem_u32(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kOffBar);
+  auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+  auto empty_bar = [&](int s) { return smem_u32(&bars[NSTAGE + s]); };
+  const uint32_t acc_full = smem_u32(&bars[2 * NSTAGE]);
+  const uint32_t acc_empty = smem_u32(&bars[2 * NSTAGE + 1]);
+  const uint32_t fin_bar = smem_u32(&bars[2 * NSTAGE + 2]);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kOffBar + 192);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kOffBar + 200);
+  static_assert((2 * NSTAGE + 3) * 8 <= 192, "barrier area");
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NSTAGE; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, kGEpi);
+    mbar_init(fin_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    if (lane == 0) {
+      uint32_t g = 0;
+      bool ok = true;
+      for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
+        const int row0 = (int)(u / gp.m_tiles) * kGM;
+        const int i0 = (int)(u % gp.m_tiles) * NT;
+        for (int kc = 0; kc < gp.k_chunks; ++kc, ++g) {
+          const int s = (int)(g % NSTAGE);
+          if (!mbar_wait(empty_bar(s), ((g / NSTAGE) & 1) ^ 1, abort_flag, gp.err, 51)) { ok = false; break; }
+          const uint32_t st = sbase + s * L::kStage;
+          mbar_arrive_tx(full_bar(s), L::kStage);
+#pragma unroll
+          for (int a = 0; a < NS; ++a) {
+            tma_load_3d(st + a * L::kA, &tm_x, kc * kGK, row0, a, full_bar(s));
+            tma_load_3d(st + NS * L::kA + a * L::kB, &tm_m, kc * kGK, i0, a, full_bar(s));
+          }
+        }
+      }
+      // drain: every issued stage must have landed before the CTA may exit
+      const uint32_t issued = g;
+      for (uint32_t q = issued >= (uint32_t)NSTAGE ? issued - NSTAGE : 0; q < issued; ++q)
+        mbar_wait(full_bar(q % NSTAGE), (q / NSTAGE) & 1, abort_flag, gp.err, 57, true);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer
+    if (lane == 0) {
+      constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGM >> 4) << 24);
+      uint32_t g = 0, t = 0;
+      bool ok = true;
+      for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
+        for (int kc = 0; kc < gp.k_chunks; ++kc, ++g) {
+          const bool begin = SEG ? kc % (kSegK / kGK) == 0 : kc == 0;
+          if (begin) {
+            if (!mbar_wait(acc_empty, (t & 1) ^ 1, abort_flag, gp.err, 52)) { ok = false; break; }
+            tc_fence_after();
+          }
+          const int s = (int)(g % NSTAGE);
+          if (!mbar_wait(full_bar(s), (g / NSTAGE) & 1, abort_flag, gp.err, 53)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t sa = sbase + s * L::kStage, sb = sa + NS * L::kA;
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            const uint32_t off = ks * 32;
+            const bool first = begin && ks == 0;
+#pragma unroll
+            for (int a = 0; a < NS; ++a) {
+              // slice a against slices 0 .. nb - 1, at most 256 columns per MMA; a piece
+              // starts its levels where no earlier piece of the tile has added to them
+              constexpr int kPer = 256 / NT;
+              const int nb = NS < NLEV - a ? NS : NLEV - a;
+#pragma unroll
+              for (int b = 0; b < nb; b += kPer) {
+                const int w = nb - b < kPer ? nb - b : kPer;
+                const int seen = a == 0 ? b : (NS < NLEV - a + 1 ? NS : NLEV - a + 1) + a - 1;   // levels begun so far
+                const uint32_t acc = (first && a + b >= seen) ? 0u : 1u;
+                mma_bf16(tmem_base + (a + b) * NT, desc64(sa + a * L::kA + off), desc64(sb + b * L::kB + off),
+                         idesc0 | ((uint32_t)(w * NT >> 3) << 17), acc);
+              }
+            }
+          }
+          mma_commit(empty_bar(s));
+          if (kc + 1 == gp.k_chunks || (SEG && (kc + 1) % (kSegK / kGK) == 0)) {
+            mma_commit(acc_full);
+            ++t;
+          }
+        }
+      }
+      // drain: all issued MMAs complete before TMEM is released
+      mma_commit(fin_bar);
+      mbar_wait(fin_bar, 0, abort_flag, gp.err, 58, true);
+    }
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    constexpr int NC = NT / 2;   // columns of this warp
+    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    uint32_t t = 0;
+    bool ok = true;
+    const int segs = SEG ? (gp.k_chunks + kSegK / kGK - 1) / (kSegK / kGK) : 1;
+    for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
+      const long long row = (u / gp.m_tiles) * kGM + q * 32 + lane;
+      const int i0 = (int)(u % gp.m_tiles) * NT + half * NC;
+      const bool live = row < gp.rows;
+      const int er = live ? ex[row] : 0;
+      T y[NC];
+      Sum<T> sum[SEG ? NC : 1];
+      for (int sg = 0; sg < segs; ++sg, ++t) {
+        if (!mbar_wait(acc_full, t & 1, abort_flag, gp.err, 59)) { ok = false; break; }
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < NC; c0 += 8) {
+          uint32_t v[NLEV][8];
+#pragma unroll
+          for (int l = 0; l < NLEV; ++l) tmem_ld8(tmem_base + lane_off + l * NT + half * NC + c0, v[l]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float P[NLEV];
+#pragma unroll
+            for (int l = 0; l < NLEV; ++l) P[l] = __uint_as_float(v[l][j]);
+            if constexpr (SEG) {
+              sum[c0 + j].add(P);
+            } else {
+              Sum<T> one;
+              one.add(P);
+              y[c0 + j] = finish(one, er, i0 + c0 + j, em, gp);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+      }
+      if (!ok) break;
+      if constexpr (SEG) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) y[j] = finish(sum[j], er, i0 + j, em, gp);
+      }
+      if (live) {
+        const long long c = row / gp.R;
+        T* dst = Y + c * gp.plane + (row - c * gp.R);
+#pragma unroll
+        for (int j = 0; j < NC; ++j)
+          if (i0 + j < gp.m) dst[(long long)(i0 + j) * gp.R] = y[j];
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
+}
+
+}  // namespace
+
+template <typename T>
+void slice_map(Sliced& s, bool matrix) {
+  const cuuint64_t pitch = (cuuint64_t)slice_pitch(s.K);
+  cuuint64_t dims[3] = {(cuuint64_t)s.K, (cuuint64_t)s.rows, (cuuint64_t)SliceCfg<T>::NS};
+  cuuint64_t strides[2] = {pitch * 2, pitch * 2 * (cuuint64_t)s.rows};
+  cuuint32_t box[3] = {kGK, (cuuint32_t)(matrix ? GemmCfg<T>::NT : kGM), 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = encode_fn()(&s.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, s.dig, dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) throw std::runtime_error("cuTensorMapEncodeTiled (slices) failed (" + std::to_string((int)r) + ")");
+}
+
+template <typename T>
+void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, cudaStream_t st,
+                long long& nl) {
+  const int quads = seg_len / 4;
+  const int group = quads <= 8 ? 8 : (quads <= 16 ? 16 : 32);
+  const long long per_block = 256 / group;
+  const long long blocks = std::min<long long>((s.rows + per_block - 1) / per_block, (long long)num_sms() * 16);
+  launch_pdl(slice_kernel<T>, (int)blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group,
+             s.dig, s.ex);
+  FCGLE_LAUNCHED(nl);
+}
+
+template <typename T>
+void sliced_gemm(const Sliced& x, const Sliced& m, T* Y, long long R, long long plane, int* err, cudaStream_t st,
+                 long long& nl) {
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GemmLayout<T>::kSmem));
+    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GemmLayout<T>::kSmem));
+  });
+  GemmParams gp;
+  gp.rows = x.rows;
+  gp.R = R;
+  gp.plane = plane;
+  gp.m = (int)m.rows;
+  gp.m_tiles = (gp.m + GemmCfg<T>::NT - 1) / GemmCfg<T>::NT;
+  gp.k_chunks = (x.K + kGK - 1) / kGK;
+  gp.units = (x.rows + kGM - 1) / kGM * gp.m_tiles;
+  gp.kb = 0;
+  while ((1 << gp.kb) < x.K) ++gp.kb;
+  gp.err = err;
+  launch_pdl(x.K <= kSegK ? sliced_gemm_kernel<T, false> : sliced_gemm_kernel<T, true>, (int)std::min<long long>(gp.units, num_sms()), kGThreads, GemmLayout<T>::kSmem, st,
+             x.tm, m.tm, (const int*)x.ex, (const int*)m.ex, Y, gp);
+  FCGLE_LAUNCHED(nl);
+}
+
+#define INST(T)                                                                                                  \
+  template void slice_map<T>(Sliced&, bool);                                                                     \
+  template void slice_rows<T>(const T*, const Sliced&, int, int, long long, cudaStream_t, long long&);           \
+  template void sliced_gemm<T>(const Sliced&, const Sliced&, T*, long long, long long, int*, cudaStream_t, long long&);
+INST(float)
+INST(double)
+#undef INST
+
+}  // namespace fcgle
