@@ -10,8 +10,10 @@
 // mp_b3_kernel).  The intermediate U = X_slab M1^T never leaves the SM: two
 // mode products for the HBM bytes of one.
 //
-// Unit of work: (slab j3, block of 128 i1).  For each plane c (real, then
-// imaginary; M1 and M2 are real, so the planes do not mix):
+// Unit of work: (plane c, slab j3, block of 128 i1); M1 and M2 are real, so the
+// planes do not mix, and a plane per unit halves the last wave (256^3: 1024
+// units on 152 SMs, 6.7 of 7 rounds, where both planes of a slab made 3.4 of 4;
+// five Krogstad steps 8.90 -> 8.57 ms):
 //   stage 1  D[i1][j2]  = sum_j1 M1[i1][j1] X[c][j3][j2][j1]
 //            (A = 128 rows of M1, B = the slab's N2 rows j2, both K-major
 //            from shared memory; N2 = p2 rounded up to 16, <= 256)
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();
 
-  const long long units = (long long)sp.p3 * sp.mb1;
+  const long long units = 2LL * sp.p3 * sp.mb1;   // unit u: plane-slab z = u / mb1 (c * p3 + j3), i1-block u % mb1
   int* err = sp.err;
 
   if (warp == 0) {
@@ -151,28 +153,25 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
       const uint32_t xbytes = (uint32_t)sp.n2 * 64;   // one N2 x 32 bf16 box
       const int m2boxes = sp.n2 > 128 ? 2 : 1;
       for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int j3 = (int)(u / sp.mb1), b1 = (int)(u % sp.mb1);
-        for (int c = 0; c < 2 && ok; ++c) {
-          const int z = c * sp.p3 + j3;
-          for (int kc = 0; kc < sp.kc1; ++kc, ++g) {
-            const int s = (int)(g % SL_NS);
-            if (!mbar_wait(empty_bar(s), ((g / SL_NS) & 1) ^ 1, abort_flag, err, 31)) { ok = false; break; }
-            const uint32_t st = sbase + s * kSlStage;
-            mbar_arrive_tx(full_bar(s), 16384 + 2 * xbytes);
-            tma_load_2d(st, &tm_m1hi, kc * SL_K, b1 * BM, full_bar(s));
-            tma_load_2d(st + 8192, &tm_m1lo, kc * SL_K, b1 * BM, full_bar(s));
-            tma_load_3d(st + 16384, &tm_xhi, kc * SL_K, 0, z, full_bar(s));
-            tma_load_3d(st + 32768, &tm_xlo, kc * SL_K, 0, z, full_bar(s));
-          }
-          for (int kc = 0; kc < sp.kc2 && ok; ++kc, ++g) {
-            const int s = (int)(g % SL_NS);
-            if (!mbar_wait(empty_bar(s), ((g / SL_NS) & 1) ^ 1, abort_flag, err, 32)) { ok = false; break; }
-            const uint32_t st = sbase + s * kSlStage;
-            mbar_arrive_tx(full_bar(s), (uint32_t)m2boxes * 16384);
-            for (int b = 0; b < m2boxes; ++b) {
-              tma_load_2d(st + b * 8192, &tm_m2hi, kc * SL_K, b * BM, full_bar(s));
-              tma_load_2d(st + 16384 + b * 8192, &tm_m2lo, kc * SL_K, b * BM, full_bar(s));
-            }
+        const int z = (int)(u / sp.mb1), b1 = (int)(u % sp.mb1);
+        for (int kc = 0; kc < sp.kc1; ++kc, ++g) {
+          const int s = (int)(g % SL_NS);
+          if (!mbar_wait(empty_bar(s), ((g / SL_NS) & 1) ^ 1, abort_flag, err, 31)) { ok = false; break; }
+          const uint32_t st = sbase + s * kSlStage;
+          mbar_arrive_tx(full_bar(s), 16384 + 2 * xbytes);
+          tma_load_2d(st, &tm_m1hi, kc * SL_K, b1 * BM, full_bar(s));
+          tma_load_2d(st + 8192, &tm_m1lo, kc * SL_K, b1 * BM, full_bar(s));
+          tma_load_3d(st + 16384, &tm_xhi, kc * SL_K, 0, z, full_bar(s));
+          tma_load_3d(st + 32768, &tm_xlo, kc * SL_K, 0, z, full_bar(s));
+        }
+        for (int kc = 0; kc < sp.kc2 && ok; ++kc, ++g) {
+          const int s = (int)(g % SL_NS);
+          if (!mbar_wait(empty_bar(s), ((g / SL_NS) & 1) ^ 1, abort_flag, err, 32)) { ok = false; break; }
+          const uint32_t st = sbase + s * kSlStage;
+          mbar_arrive_tx(full_bar(s), (uint32_t)m2boxes * 16384);
+          for (int b = 0; b < m2boxes; ++b) {
+            tma_load_2d(st + b * 8192, &tm_m2hi, kc * SL_K, b * BM, full_bar(s));
+            tma_load_2d(st + 16384 + b * 8192, &tm_m2lo, kc * SL_K, b * BM, full_bar(s));
           }
         }
       }
@@ -190,56 +189,54 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
       const int ksteps2 = sp.n2 / 16;
       uint32_t g = 0, t = 0;
       bool ok = true;
-      for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        for (int c = 0; c < 2 && ok; ++c, ++t) {
-          // D may be overwritten once the previous plane's stage 2 has read U
-          if (t > 0 && !mbar_wait(d2_full, (t - 1) & 1, abort_flag, err, 33)) { ok = false; break; }
+      for (long long u = blockIdx.x; u < units && ok; u += gridDim.x, ++t) {
+        // D may be overwritten once the previous plane's stage 2 has read U
+        if (t > 0 && !mbar_wait(d2_full, (t - 1) & 1, abort_flag, err, 33)) { ok = false; break; }
+        tc_fence_after();
+        // stage 1: D[i1][j2] = sum_j1 M1[i1][j1] X[j2][j1]
+        for (int kc = 0; kc < sp.kc1; ++kc, ++g) {
+          const int s = (int)(g % SL_NS);
+          if (!mbar_wait(full_bar(s), (g / SL_NS) & 1, abort_flag, err, 34)) { ok = false; break; }
           tc_fence_after();
-          // stage 1: D[i1][j2] = sum_j1 M1[i1][j1] X[j2][j1]
-          for (int kc = 0; kc < sp.kc1; ++kc, ++g) {
-            const int s = (int)(g % SL_NS);
-            if (!mbar_wait(full_bar(s), (g / SL_NS) & 1, abort_flag, err, 34)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t ahi = sbase + s * kSlStage, alo = ahi + 8192;
-            const uint32_t bhi = ahi + 16384, blo = ahi + 32768;
+          const uint32_t ahi = sbase + s * kSlStage, alo = ahi + 8192;
+          const uint32_t bhi = ahi + 16384, blo = ahi + 32768;
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-              const uint32_t off = ks * 32;
-              const uint32_t acc0 = (kc > 0 || ks > 0) ? 1u : 0u;
-              mma_bf16(tmem_base, sw64_desc(ahi + off), sw64_desc(bhi + off), idesc, acc0);
-              mma_bf16(tmem_base, sw64_desc(ahi + off), sw64_desc(blo + off), idesc, 1u);
-              mma_bf16(tmem_base, sw64_desc(alo + off), sw64_desc(bhi + off), idesc, 1u);
-            }
-            mma_commit(empty_bar(s));
+          for (int ks = 0; ks < 2; ++ks) {
+            const uint32_t off = ks * 32;
+            const uint32_t acc0 = (kc > 0 || ks > 0) ? 1u : 0u;
+            mma_bf16(tmem_base, sw64_desc(ahi + off), sw64_desc(bhi + off), idesc, acc0);
+            mma_bf16(tmem_base, sw64_desc(ahi + off), sw64_desc(blo + off), idesc, 1u);
+            mma_bf16(tmem_base, sw64_desc(alo + off), sw64_desc(bhi + off), idesc, 1u);
           }
-          if (!ok) break;
-          mma_commit(d1_full);
-          // stage 2: E[i1][i2] = sum_j2 U[i1][j2] M2[i2][j2], U from tensor
-          // memory; E is free once the previous plane's E has been read out,
-          // and k-chunk kc starts as soon as its 64 columns of U are written
-          if (!mbar_wait(d_empty, (t & 1) ^ 1, abort_flag, err, 41)) { ok = false; break; }
-          for (int kc = 0; kc < sp.kc2; ++kc, ++g) {
-            const int s = (int)(g % SL_NS);
-            if (!mbar_wait(u_full(kc >> 1), t & 1, abort_flag, err, 35)) { ok = false; break; }
-            if (!mbar_wait(full_bar(s), (g / SL_NS) & 1, abort_flag, err, 36)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t bhi = sbase + s * kSlStage, blo = bhi + 16384;
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-              const int kk = 2 * kc + ks;   // 16-wide k-step of j2
-              if (kk < ksteps2) {
-                const uint32_t uhi = tmem_base + 16 * kk, ulo = uhi + 8;
-                const uint32_t off = ks * 32, e_tmem = tmem_base + kSlColE;
-                mma_bf16_ts(e_tmem, uhi, sw64_desc(bhi + off), idesc, kk > 0 ? 1u : 0u);
-                mma_bf16_ts(e_tmem, uhi, sw64_desc(blo + off), idesc, 1u);
-                mma_bf16_ts(e_tmem, ulo, sw64_desc(bhi + off), idesc, 1u);
-              }
-            }
-            mma_commit(empty_bar(s));
-          }
-          if (!ok) break;
-          mma_commit(d2_full);
+          mma_commit(empty_bar(s));
         }
+        if (!ok) break;
+        mma_commit(d1_full);
+        // stage 2: E[i1][i2] = sum_j2 U[i1][j2] M2[i2][j2], U from tensor
+        // memory; E is free once the previous plane's E has been read out,
+        // and k-chunk kc starts as soon as its 64 columns of U are written
+        if (!mbar_wait(d_empty, (t & 1) ^ 1, abort_flag, err, 41)) { ok = false; break; }
+        for (int kc = 0; kc < sp.kc2; ++kc, ++g) {
+          const int s = (int)(g % SL_NS);
+          if (!mbar_wait(u_full(kc >> 1), t & 1, abort_flag, err, 35)) { ok = false; break; }
+          if (!mbar_wait(full_bar(s), (g / SL_NS) & 1, abort_flag, err, 36)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t bhi = sbase + s * kSlStage, blo = bhi + 16384;
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            const int kk = 2 * kc + ks;   // 16-wide k-step of j2
+            if (kk < ksteps2) {
+              const uint32_t uhi = tmem_base + 16 * kk, ulo = uhi + 8;
+              const uint32_t off = ks * 32, e_tmem = tmem_base + kSlColE;
+              mma_bf16_ts(e_tmem, uhi, sw64_desc(bhi + off), idesc, kk > 0 ? 1u : 0u);
+              mma_bf16_ts(e_tmem, uhi, sw64_desc(blo + off), idesc, 1u);
+              mma_bf16_ts(e_tmem, ulo, sw64_desc(bhi + off), idesc, 1u);
+            }
+          }
+          mma_commit(empty_bar(s));
+        }
+        if (!ok) break;
+        mma_commit(d2_full);
       }
       // drain: all issued MMAs complete before TMEM is released
       mma_commit(fin_bar);
@@ -256,77 +253,74 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     const int nbox = (sp.n2 + 31) / 32; // 32-column output boxes
     uint32_t t = 0;
     bool ok = true;
-    for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
-      const int j3 = (int)(u / sp.mb1), b1 = (int)(u % sp.mb1);
-      for (int c = 0; c < 2; ++c, ++t) {
-        // ---- convert: D (FP32) -> U_hi, U_lo (bf16 pairs) in tensor memory, one
-        // 64-column k-chunk (4 groups of 16, 2 per warp of a lane quarter) at a time
-        if (!mbar_wait(d1_full, t & 1, abort_flag, err, 39)) { ok = false; break; }
-        tc_fence_after();
-        for (int kc = 0; kc < (sp.n2 + 63) / 64; ++kc) {
-          uint32_t v[2][16];
+    for (long long u = blockIdx.x; u < units && ok; u += gridDim.x, ++t) {
+      const int z = (int)(u / sp.mb1), b1 = (int)(u % sp.mb1);
+      // ---- convert: D (FP32) -> U_hi, U_lo (bf16 pairs) in tensor memory, one
+      // 64-column k-chunk (4 groups of 16, 2 per warp of a lane quarter) at a time
+      if (!mbar_wait(d1_full, t & 1, abort_flag, err, 39)) { ok = false; break; }
+      tc_fence_after();
+      for (int kc = 0; kc < (sp.n2 + 63) / 64; ++kc) {
+        uint32_t v[2][16];
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int grp = 4 * kc + par + 2 * e;
-            if (grp < ngrp) tmem_ld16(tmem_base + lane_off + 16 * grp, v[e]);
+        for (int e = 0; e < 2; ++e) {
+          const int grp = 4 * kc + par + 2 * e;
+          if (grp < ngrp) tmem_ld16(tmem_base + lane_off + 16 * grp, v[e]);
+        }
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int grp = 4 * kc + par + 2 * e;
+          if (grp < ngrp) {
+            uint32_t h[8], l[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              h[j] = split_pair(__uint_as_float(v[e][2 * j]), __uint_as_float(v[e][2 * j + 1]), l[j]);
+            tmem_st8(tmem_base + lane_off + 16 * grp, h);
+            tmem_st8(tmem_base + lane_off + 16 * grp + 8, l);
           }
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int grp = 4 * kc + par + 2 * e;
-            if (grp < ngrp) {
-              uint32_t h[8], l[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                h[j] = split_pair(__uint_as_float(v[e][2 * j]), __uint_as_float(v[e][2 * j + 1]), l[j]);
-              tmem_st8(tmem_base + lane_off + 16 * grp, h);
-              tmem_st8(tmem_base + lane_off + 16 * grp + 8, l);
-            }
-          }
-          tmem_wait_st();
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(u_full(kc));
+      }
+      // ---- store: E (FP32) -> Y[c][j3][i2][i1], split, one 32-column box at a time
+      if (!mbar_wait(d2_full, t & 1, abort_flag, err, 40)) { ok = false; break; }
+      tc_fence_after();
+      if (par >= nbox && lane == 0) mbar_arrive(d_empty);   // no box of E for this warp
+      const int x = b1 * BM + q * 32;   // first i1 of this warp's rows
+      for (int bx = par; bx < nbox; bx += 2) {
+        uint32_t v[32];
+        tmem_ld16(tmem_base + lane_off + kSlColE + 32 * bx, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
+        tmem_ld16(tmem_base + lane_off + kSlColE + 32 * bx + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
+        tmem_wait_ld();
+        if (bx + 2 >= nbox) {   // this warp's last read of E
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(u_full(kc));
+          if (lane == 0) mbar_arrive(d_empty);
         }
-        // ---- store: E (FP32) -> Y[c][j3][i2][i1], split, one 32-column box at a time
-        if (!mbar_wait(d2_full, t & 1, abort_flag, err, 40)) { ok = false; break; }
-        tc_fence_after();
-        if (par >= nbox && lane == 0) mbar_arrive(d_empty);   // no box of E for this warp
-        const int x = b1 * BM + q * 32;   // first i1 of this warp's rows
-        const int z = c * sp.p3 + j3;
-        for (int bx = par; bx < nbox; bx += 2) {
-          uint32_t v[32];
-          tmem_ld16(tmem_base + lane_off + kSlColE + 32 * bx, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
-          tmem_ld16(tmem_base + lane_off + kSlColE + 32 * bx + 16, *reinterpret_cast<uint32_t(*)[16]>(&v[16]));
-          tmem_wait_ld();
-          if (bx + 2 >= nbox) {   // this warp's last read of E
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(d_empty);
-          }
-          if (lane == 0) bulk_wait_read0();
-          __syncwarp();
-          // box row j = i2 - 32 bx (64 bytes: 32 i1), this lane's i1 at byte 2 lane
+        if (lane == 0) bulk_wait_read0();
+        __syncwarp();
+        // box row j = i2 - 32 bx (64 bytes: 32 i1), this lane's i1 at byte 2 lane
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            uint32_t lo;
-            const uint32_t hi = split_pair(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), lo);
-            const uint32_t a0 = box_u32 + j * 64 + lane * 2;
-            asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0), "h"((unsigned short)(hi & 0xFFFFu)) : "memory");
-            asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 64), "h"((unsigned short)(hi >> 16)) : "memory");
-            asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 2048), "h"((unsigned short)(lo & 0xFFFFu)) : "memory");
-            asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 2048 + 64), "h"((unsigned short)(lo >> 16))
-                         : "memory");
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0 && x < sp.p1 && 32 * bx < sp.p2) {
-            tma_store_3d(&tm_yhi, box_u32, x, 32 * bx, z);
-            tma_store_3d(&tm_ylo, box_u32 + 2048, x, 32 * bx, z);
-            bulk_commit();
-          }
-          __syncwarp();
+        for (int j = 0; j < 32; j += 2) {
+          uint32_t lo;
+          const uint32_t hi = split_pair(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), lo);
+          const uint32_t a0 = box_u32 + j * 64 + lane * 2;
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0), "h"((unsigned short)(hi & 0xFFFFu)) : "memory");
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 64), "h"((unsigned short)(hi >> 16)) : "memory");
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 2048), "h"((unsigned short)(lo & 0xFFFFu)) : "memory");
+          asm volatile("st.shared.b16 [%0], %1;" ::"r"(a0 + 2048 + 64), "h"((unsigned short)(lo >> 16))
+                       : "memory");
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0 && x < sp.p1 && 32 * bx < sp.p2) {
+          tma_store_3d(&tm_yhi, box_u32, x, 32 * bx, z);
+          tma_store_3d(&tm_ylo, box_u32 + 2048, x, 32 * bx, z);
+          bulk_commit();
+        }
+        __syncwarp();
       }
     }
     if (lane == 0) bulk_wait0();

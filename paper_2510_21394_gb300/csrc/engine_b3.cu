@@ -1386,7 +1386,7 @@ class EngineB3 : public EngineBase {
     encode_bf16_3d(&txl, in.lo, (uint64_t)p1, (uint64_t)p2, 2 * (uint64_t)p3, b3::SL_K, (uint32_t)sp.n2, 64);
     encode_bf16_3d(&tyh, out.hi, (uint64_t)p1, (uint64_t)p2, 2 * (uint64_t)p3, 32, 32, 0);
     encode_bf16_3d(&tyl, out.lo, (uint64_t)p1, (uint64_t)p2, 2 * (uint64_t)p3, 32, 32, 0);
-    const long long units = (long long)p3 * sp.mb1;
+    const long long units = 2LL * p3 * sp.mb1;
     const int grid = (int)std::min<long long>(units, num_sms());
     launch_pdl(b3::mp_b3_slab12_kernel, grid, b3::SL_THREADS, b3::kSlSmemBytes, st_, txh, txl, m1.tm_hi64,
                m1.tm_lo64, m2.tm_hi64, m2.tm_lo64, tyh, tyl, sp);
