@@ -9,11 +9,18 @@
 //   * the stage combinations of Eq. krogstad-m and the other schemes,
 // writing FP32 planar tensors and/or split (hi, lo) bf16 tensors that feed
 // the next mode product.  Each functor is a plain struct passed by value with
-//   kIn, kBatch, load<V>(q, i, r, in), store<V>(q, i, r, re, im, in): the
-//              kernel loads the operands of kBatch groups first, then stores.
+//   kIn        real operand planes read per element (two per tensor),
+//   src(k)     operand tensor k (planes at src + q and src + P + q; the kernel
+//              fetches them ahead of the product),
+//   kLam       the functor needs the eigenvalue sums (member L),
+//   kG         the functor evaluates g (member g; its source terms are fetched
+//              like operands),
+//   store<V>(q, sv, re, im, in, src, em): sv = eigenvalue sums of the V elements
+//              (kLam), in[2 k], in[2 k + 1] = operand k, src = source values;
+//              writes its FP32 outputs and leaves the split one in em,
+//   split()    where the split output goes (hi == nullptr: none).
 // (The plain split product without a pointwise stage is b3_plain.cuh.)
-// V = 4 when R % 4 == 0 (16-byte FP32 and 8-byte split accesses, q % 4 == 0),
-// V = 1 otherwise.  Plane indices are 32-bit (the host requires 2 P < 2^32).
+// V = 4 when R % 8 == 0 (d >= 2), V = 1 otherwise.  Plane indices are 32-bit (the host requires 2 P < 2^32).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -90,6 +97,25 @@ __device__ __forceinline__ void put_csplit(const SplitOut& o, uint32_t P, uint32
   put_split<V>(o, P + q, im);
 }
 
+// A functor's split result: V = 4 hands the packed values back to the kernel,
+// which stores them in wider rows (planes hi re, lo re, hi im, lo im; two words
+// of 2 bf16 each); V = 1 stores them at once.
+struct SplitVal {
+  uint2 v[4];
+};
+template <int V>
+__device__ __forceinline__ void emit_csplit(SplitVal& em, const SplitOut& o, uint32_t P, uint32_t q,
+                                            const float (&re)[V], const float (&im)[V]) {
+  if constexpr (V == 4) {
+    em.v[0].x = bf2(re[0], re[1], em.v[1].x);
+    em.v[0].y = bf2(re[2], re[3], em.v[1].y);
+    em.v[2].x = bf2(im[0], im[1], em.v[3].x);
+    em.v[2].y = bf2(im[2], im[3], em.v[3].y);
+  } else {
+    put_csplit<V>(o, P, q, re, im);
+  }
+}
+
 // g(t, u) ingredients: static part and the factors e^{sigma_k t} of one time t.
 struct GStatic {
   float gamma = 0, kappa = 0, zeta = 0;
@@ -100,9 +126,23 @@ struct GTime {
   float e_re[kMaxSrc] = {0, 0, 0, 0}, e_im[kMaxSrc] = {0, 0, 0, 0};
 };
 
+// Source values of 4 elements that the kernel has fetched into shared memory:
+// terms 0 .. n - 1, plane c of term k at addr + 1024 (2 k + c).
+struct SrcIn {
+  uint32_t addr = 0;
+  int n = 0;
+};
+__device__ __forceinline__ void lds16(uint32_t src, float (&v)[4]) {
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "r"(src)
+               : "memory");
+}
+
 template <int V>
 __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_t P, uint32_t q, const float (&ur)[V],
-                                       const float (&ui)[V], float (&gr)[V], float (&gi)[V]) {
+                                       const float (&ui)[V], float (&gr)[V], float (&gi)[V],
+                                       const SrcIn& src = SrcIn{}) {
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     const float m2 = ur[v] * ur[v] + ui[v] * ui[v];
@@ -111,8 +151,18 @@ __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_
   }
   for (int k = 0; k < g.nsrc; ++k) {
     float sr[V], si[V];
-    ldv_ro<V>(g.S[k] + q, sr);
-    ldv_ro<V>(g.S[k] + P + q, si);
+    bool have = false;
+    if constexpr (V == 4) {
+      have = k < src.n;
+      if (have) {
+        lds16(src.addr + 2048 * k, sr);
+        lds16(src.addr + 2048 * k + 1024, si);
+      }
+    }
+    if (!have) {
+      ldv_ro<V>(g.S[k] + q, sr);
+      ldv_ro<V>(g.S[k] + P + q, si);
+    }
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       gr[v] += t.e_re[k] * sr[v] - t.e_im[k] * si[v];
@@ -121,28 +171,43 @@ __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_
   }
 }
 
-// Eigenvalues of K at standard-order indices q + v = i_d * R + r + v (Sec. 3.2):
-// lam = (nu + i eta) (lam_d[i_d] + sum_{mu < d} lam_mu[digits of r + v]).
-// For V = 4, r % 4 == 0 and p_1 % 8 == 0, so only the fastest digit changes.
+// Eigenvalues of K at standard-order indices q = i_d * R + r (Sec. 3.2):
+// lam = (nu + i eta) s, s = lam_d[i_d] + sum_{mu < d} lam_mu[digits of r].
+// The kernel forms s: the part of r is the same for every row of a tile.
 struct LamF {
   const float* lam[kMaxDim] = {nullptr, nullptr, nullptr};
   int p[kMaxDim] = {1, 1, 1};
   int d = 1;
   float c_re = 0, c_im = 0;
 };
+// the terms of r, r + 1, .. (r % V == 0 and p_1 % 8 == 0: only the fastest digit changes)
 template <int V>
-__device__ __forceinline__ void lam_eval(const LamF& L, int i, uint32_t r, float (&lr)[V], float (&li)[V]) {
-  float base = L.lam[L.d - 1][i];
-  uint32_t j1 = r;
+struct LamR {
+  float l2 = 0.f, l1[V];
+};
+template <int V>
+__device__ __forceinline__ void lam_r(const LamF& L, uint32_t r, LamR<V>& o) {
+  const uint32_t j2 = L.d == 3 ? r / (uint32_t)L.p[0] : 0u;
+  if (L.d == 3) o.l2 = __ldg(L.lam[1] + j2);
   if (L.d >= 2) {
-    j1 = r % (uint32_t)L.p[0];
-    if (L.d == 3) base += L.lam[1][r / (uint32_t)L.p[0]];
+    ldv_ro<V>(L.lam[0] + (r - j2 * (uint32_t)L.p[0]), o.l1);
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v) o.l1[v] = 0.f;
   }
+}
+// s at row i, ld = lam_d[i]
+template <int V>
+__device__ __forceinline__ void lam_s(const LamR<V>& o, float ld, float (&sv)[V]) {
+#pragma unroll
+  for (int v = 0; v < V; ++v) sv[v] = (ld + o.l2) + o.l1[v];
+}
+template <int V>
+__device__ __forceinline__ void lam_of(const LamF& L, const float (&sv)[V], float (&lr)[V], float (&li)[V]) {
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    const float s = L.d >= 2 ? base + L.lam[0][j1 + v] : base;
-    lr[v] = L.c_re * s;
-    li[v] = L.c_im * s;
+    lr[v] = L.c_re * sv[v];
+    li[v] = L.c_im * sv[v];
   }
 }
 
@@ -231,19 +296,6 @@ __device__ __forceinline__ void phi123_s(const PhiPoly& P, float s, float (&pr)[
   }
 }
 
-// real eigenvalue sums s (lam = (nu + i eta) s) at the elements of lam_eval
-template <int V>
-__device__ __forceinline__ void lam_sum(const LamF& L, int i, uint32_t r, float (&sv)[V]) {
-  float base = L.lam[L.d - 1][i];
-  uint32_t j1 = r;
-  if (L.d >= 2) {
-    j1 = r % (uint32_t)L.p[0];
-    if (L.d == 3) base += L.lam[1][r / (uint32_t)L.p[0]];
-  }
-#pragma unroll
-  for (int v = 0; v < V; ++v) sv[v] = L.d >= 2 ? base + L.lam[0][j1 + v] : base;
-}
-
 // phi_k(z), any k >= 1: Horner form of the series
 // (1/k!)(1 + z/(k+1)(1 + z/(k+2)(...))) for |z| < 1.5, recurrence otherwise.
 __device__ __forceinline__ void phik(int k, float zr, float zi, float& fr, float& fi) {
@@ -300,34 +352,35 @@ __device__ __forceinline__ void fspec(int kind, float zr, float zi, float& fr, f
 }
 
 // ---------------------------------------------------------------- functors
-#define FCGLE_EPI(IN, BATCH)              \
-  static constexpr int kIn = IN;           \
-  static constexpr int kBatch = BATCH;
+#define FCGLE_EPI(IN, LAM, SRC)          \
+  static constexpr int kIn = IN;          \
+  static constexpr bool kLam = LAM;       \
+  static constexpr bool kG = SRC;
 
 // product -> split, element stores (any R)
 struct EpiStoreSplitGen {
-  FCGLE_EPI(0, 4)
+  FCGLE_EPI(0, false, false)
   uint32_t P;
   SplitOut Y;
+  __device__ SplitOut split() const { return Y; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t, int, uint32_t, float (&)[1][V]) const {}
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&)[1][V]) const {
-    put_csplit<V>(Y, P, q, re, im);
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn&, SplitVal& em) const {
+    emit_csplit<V>(em, Y, P, q, re, im);
   }
 };
 
 // product -> FP32
 struct EpiStoreF32 {
-  FCGLE_EPI(0, 4)
+  FCGLE_EPI(0, false, false)
   uint32_t P;
   float* Y;
+  __device__ SplitOut split() const { return SplitOut{}; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t, int, uint32_t, float (&)[1][V]) const {}
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&)[1][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn&, SplitVal&) const {
     stv<V>(Y + q, re);
     stv<V>(Y + P + q, im);
   }
@@ -335,19 +388,19 @@ struct EpiStoreF32 {
 
 // Y = f(theta lam) o product  (split), f evaluated on the fly (fspec kinds)
 struct EpiScaleF {
-  FCGLE_EPI(0, 4)
+  FCGLE_EPI(0, true, false)
   uint32_t P;
   LamF L;
   int kind;
   float theta;
   SplitOut Y;
+  __device__ SplitOut split() const { return Y; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t, int, uint32_t, float (&)[1][V]) const {}
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&)[1][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], yr[V], yi[V];
-    lam_eval<V>(L, i, r, lr, li);
+    lam_of<V>(L, sv, lr, li);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float fr, fi;
@@ -355,80 +408,71 @@ struct EpiScaleF {
       yr[v] = fr * re[v] - fi * im[v];
       yi[v] = fr * im[v] + fi * re[v];
     }
-    put_csplit<V>(Y, P, q, yr, yi);
+    emit_csplit<V>(em, Y, P, q, yr, yi);
   }
 };
 
-// u = (add ? U : 0) + product -> U (FP32);  V = a u + b g(t', u) -> split
+// u = product -> U (FP32);  V = a u + b g(t', u) -> split
 struct EpiUpdateG {
-  FCGLE_EPI(2, 2)
+  FCGLE_EPI(0, false, true)
   uint32_t P;
   float* U;
-  int add;
   GStatic g;
   GTime t;
   float a, b;
   SplitOut Vout;
+  __device__ SplitOut split() const { return Vout; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    if (add) {
-      ldv<V>(U + q, in[0]);
-      ldv<V>(U + P + q, in[1]);
-    }
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn& src, SplitVal& em) const {
     float ur[V], ui[V], gr[V], gi[V], vr[V], vi[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      ur[v] = add ? re[v] + in[0][v] : re[v];
-      ui[v] = add ? im[v] + in[1][v] : im[v];
+      ur[v] = re[v];
+      ui[v] = im[v];
       gr[v] = gi[v] = 0.f;
     }
     stv<V>(U + q, ur);
     stv<V>(U + P + q, ui);
-    if (b != 0.f) g_eval<V>(g, t, P, q, ur, ui, gr, gi);
+    if (b != 0.f) g_eval<V>(g, t, P, q, ur, ui, gr, gi, src);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       vr[v] = a * ur[v] + b * gr[v];
       vi[v] = a * ui[v] + b * gi[v];
     }
-    put_csplit<V>(Vout, P, q, vr, vi);
+    emit_csplit<V>(em, Vout, P, q, vr, vi);
   }
 };
 
 // u_s = U + product;  D = g(t_s, u_s) - g(t_n, U) -> split;  optionally U_out = u_s
 struct EpiStageD {
-  FCGLE_EPI(2, 2)
+  FCGLE_EPI(2, false, true)
   uint32_t P;
   const float* U;
   float* Uout;
   GStatic g;
   GTime ts, tn;
   SplitOut D;
+  __device__ SplitOut split() const { return D; }
+  __device__ const float* src(int) const { return U; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(U + q, in[0]);
-    ldv<V>(U + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float sr[V], si[V], g1r[V], g1i[V], g0r[V], g0i[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       sr[v] = in[0][v] + re[v];
       si[v] = in[1][v] + im[v];
     }
-    g_eval<V>(g, ts, P, q, sr, si, g1r, g1i);
-    g_eval<V>(g, tn, P, q, in[0], in[1], g0r, g0i);
+    g_eval<V>(g, ts, P, q, sr, si, g1r, g1i, src);
+    g_eval<V>(g, tn, P, q, in[0], in[1], g0r, g0i, src);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       g1r[v] -= g0r[v];
       g1i[v] -= g0i[v];
     }
-    put_csplit<V>(D, P, q, g1r, g1i);
+    emit_csplit<V>(em, D, P, q, g1r, g1i);
     if (Uout) {
       stv<V>(Uout + q, sr);
       stv<V>(Uout + P + q, si);
@@ -439,7 +483,7 @@ struct EpiStageD {
 // G^ = product;  F^ = Lam o U^ + G^ -> Fh (not stored when Fh is null: ETD2RK
 // needs F^ only here);  S = c phi_1(theta Lam) o F^ -> split;  optionally U^ += S
 struct EpiFhat {
-  FCGLE_EPI(2, 2)
+  FCGLE_EPI(2, true, false)
   uint32_t P;
   LamF L;
   float* Uh;
@@ -449,22 +493,13 @@ struct EpiFhat {
   int update_uh;
   SplitOut S;
   PhiPoly ph;   // phi series coefficients of this launch (theta = theta)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return Uh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(Uh + q, in[0]);
-    ldv<V>(Uh + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], fr[V], fi[V], sr[V], si[V];
-    float sv[V];
-    lam_sum<V>(L, i, r, sv);
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      lr[v] = L.c_re * sv[v];
-      li[v] = L.c_im * sv[v];
-    }
+    lam_of<V>(L, sv, lr, li);
     cmulv<V>(lr, li, in[0], in[1], fr, fi);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -479,7 +514,7 @@ struct EpiFhat {
       stv<V>(Fh + q, fr);
       stv<V>(Fh + P + q, fi);
     }
-    put_csplit<V>(S, P, q, sr, si);
+    emit_csplit<V>(em, S, P, q, sr, si);
     if (update_uh) {
 #pragma unroll
       for (int v = 0; v < V; ++v) {
@@ -495,7 +530,7 @@ struct EpiFhat {
 // Krogstad stage 2 (Eq. krogstad-m), zh = tau/2 Lam:
 // D^_2 = product -> D2;  S = tau (1/2 phi_1(zh) F^ + phi_2(zh) D^_2) -> split
 struct EpiKrog2 {
-  FCGLE_EPI(2, 2)
+  FCGLE_EPI(2, true, false)
   uint32_t P;
   LamF L;
   const float* Fh;
@@ -503,19 +538,14 @@ struct EpiKrog2 {
   float tau;
   SplitOut S;
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau / 2)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return Fh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv_ro<V>(Fh + q, in[0]);
-    ldv_ro<V>(Fh + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     stv<V>(D2 + q, re);
     stv<V>(D2 + P + q, im);
     float sr[V], si[V];
-    float sv[V];
-    lam_sum<V>(L, i, r, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
@@ -525,7 +555,7 @@ struct EpiKrog2 {
       sr[v] = tau * ar;
       si[v] = tau * ai;
     }
-    put_csplit<V>(S, P, q, sr, si);
+    emit_csplit<V>(em, S, P, q, sr, si);
   }
 };
 
@@ -535,7 +565,7 @@ struct EpiKrog2 {
 // W = tau phi_1 F^ + (2 tau phi_2 - 4 tau phi_3) (D^_2 + D^_3) -> W (FP32),
 // since P2 (2 D2 + 2 D3 - D4) + P3 (-4 D2 - 4 D3 + 4 D4) = (2 P2 - 4 P3)(D2 + D3) + (4 P3 - P2) D4.
 struct EpiKrog3 {
-  FCGLE_EPI(4, 2)
+  FCGLE_EPI(4, true, false)
   uint32_t P;
   LamF L;
   const float* Fh;
@@ -544,19 +574,12 @@ struct EpiKrog3 {
   float tau;
   SplitOut S;
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int k) const { return k == 0 ? Fh : D2; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[4][V]) const {
-    ldv_ro<V>(Fh + q, in[0]);
-    ldv_ro<V>(Fh + P + q, in[1]);
-    ldv_ro<V>(D2 + q, in[2]);
-    ldv_ro<V>(D2 + P + q, in[3]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[4][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
     float sr[V], si[V], wr[V], wi[V];
-    float sv[V];
-    lam_sum<V>(L, i, r, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
@@ -569,7 +592,7 @@ struct EpiKrog3 {
       wr[v] = tau * (fr + cr * er - ci * ei);
       wi[v] = tau * (fi + cr * ei + ci * er);
     }
-    put_csplit<V>(S, P, q, sr, si);
+    emit_csplit<V>(em, S, P, q, sr, si);
     stv<V>(W + q, wr);
     stv<V>(W + P + q, wi);
   }
@@ -579,7 +602,7 @@ struct EpiKrog3 {
 // S = W + tau (4 phi_3 - phi_2) D^_4;  U^ += S, and U^_{n+1} -> split (the
 // backward Tucker operator then gives u_{n+1} itself)
 struct EpiKrogFinal {
-  FCGLE_EPI(4, 2)
+  FCGLE_EPI(4, true, false)
   uint32_t P;
   LamF L;
   const float* W;
@@ -587,19 +610,12 @@ struct EpiKrogFinal {
   float tau;
   SplitOut S;
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int k) const { return k == 0 ? W : Uh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[4][V]) const {
-    ldv_ro<V>(W + q, in[0]);
-    ldv_ro<V>(W + P + q, in[1]);
-    ldv<V>(Uh + q, in[2]);
-    ldv<V>(Uh + P + q, in[3]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[4][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
     float sr[V], si[V], ur[V], ui[V];
-    float sv[V];
-    lam_sum<V>(L, i, r, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
@@ -610,7 +626,7 @@ struct EpiKrogFinal {
       ur[v] = in[2][v] + sr[v];
       ui[v] = in[3][v] + si[v];
     }
-    put_csplit<V>(S, P, q, ur, ui);
+    emit_csplit<V>(em, S, P, q, ur, ui);
     stv<V>(Uh + q, ur);
     stv<V>(Uh + P + q, ui);
   }
@@ -620,24 +636,19 @@ struct EpiKrogFinal {
 // new spectral state U^_{n+1} -> split (the backward Tucker operator then gives
 // u_{n+1} itself, so the physical state carries the error of one transform)
 struct EpiEtd2 {
-  FCGLE_EPI(2, 4)
+  FCGLE_EPI(2, true, false)
   uint32_t P;
   LamF L;
   float* Uh;
   float tau;
   SplitOut S;
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return Uh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(Uh + q, in[0]);
-    ldv<V>(Uh + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float sr[V], si[V], ur[V], ui[V];
-    float sv[V];
-    lam_sum<V>(L, i, r, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
@@ -647,35 +658,11 @@ struct EpiEtd2 {
       ur[v] = in[0][v] + sr[v];
       ui[v] = in[1][v] + si[v];
     }
-    put_csplit<V>(S, P, q, ur, ui);
+    emit_csplit<V>(em, S, P, q, ur, ui);
     stv<V>(Uh + q, ur);
     stv<V>(Uh + P + q, ui);
   }
 };
-
-// phi_1(z) = (e^z - 1)/z: Horner form of sum_m z^m/(m+1)! for |z| < 1.5 (16 terms),
-// the quotient otherwise.  e^z - 1 = z phi_1(z) then carries no cancellation.
-__device__ __forceinline__ void phi1f(float zr, float zi, float& fr, float& fi) {
-  if (zr * zr + zi * zi < 2.25f) {
-    float ar = 1.f, ai = 0.f;
-    for (int m = 16; m >= 1; --m) {
-      const float w = 1.f / (float)(m + 1);
-      const float tr = 1.f + w * (ar * zr - ai * zi);
-      ai = w * (ar * zi + ai * zr);
-      ar = tr;
-    }
-    fr = ar;
-    fi = ai;
-  } else {
-    float sn, co;
-    sincosf(zi, &sn, &co);
-    const float ex = expf(zr);
-    const float er = ex * co - 1.f, ei = ex * sn;
-    const float inv = 1.f / (zr * zr + zi * zi);
-    fr = (er * zr + ei * zi) * inv;
-    fi = (ei * zr - er * zi) * inv;
-  }
-}
 
 // The schemes below keep the spectral state U^ = Q^T u (FP32) as the primary
 // state: each step updates U^ in spectral space, and the backward Tucker
@@ -688,7 +675,7 @@ __device__ __forceinline__ void phi1f(float zr, float zi, float& fr, float& fi) 
 // f = 1/(1 - z) or e^z:  U^ <- U^ + (f - 1) U^ + c f X^, with f - 1 = z f
 // resp. z phi_1(z) (no cancellation); U^_{n+1} -> Uh and -> split.
 struct EpiSpecStep {
-  FCGLE_EPI(2, 4)
+  FCGLE_EPI(2, true, false)
   uint32_t P;
   LamF L;
   float* Uh;
@@ -696,16 +683,14 @@ struct EpiSpecStep {
   float theta;
   float c;
   SplitOut S;
+  PhiPoly ph;   // phi series coefficients of this launch (kind 1: theta = theta)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return Uh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(Uh + q, in[0]);
-    ldv<V>(Uh + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], ur[V], ui[V];
-    lam_eval<V>(L, i, r, lr, li);
+    lam_of<V>(L, sv, lr, li);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float zr = theta * lr[v], zi = theta * li[v];
@@ -717,10 +702,10 @@ struct EpiSpecStep {
         mr = zr * fr - zi * fi;
         mi = zr * fi + zi * fr;
       } else {
-        float pr, pi;
-        phi1f(zr, zi, pr, pi);
-        mr = zr * pr - zi * pi;
-        mi = zr * pi + zi * pr;
+        float pr[3], pi[3];
+        phi123_s(ph, sv[v], pr, pi);
+        mr = zr * pr[0] - zi * pi[0];
+        mi = zr * pi[0] + zi * pr[0];
         fr = 1.f + mr;
         fi = mi;
       }
@@ -730,7 +715,7 @@ struct EpiSpecStep {
     }
     stv<V>(Uh + q, ur);
     stv<V>(Uh + P + q, ui);
-    put_csplit<V>(S, P, q, ur, ui);
+    emit_csplit<V>(em, S, P, q, ur, ui);
   }
 };
 
@@ -741,7 +726,7 @@ struct EpiSpecStep {
 // third = 0 and theta = tau give the linearly-implicit Euler first step.
 // dU^_{n+1} -> dU, U^_{n+1} -> Uh and -> split.
 struct EpiLBDF2S {
-  FCGLE_EPI(4, 2)
+  FCGLE_EPI(4, true, false)
   uint32_t P;
   LamF L;
   float* Uh;
@@ -749,31 +734,22 @@ struct EpiLBDF2S {
   float theta;
   float third;
   SplitOut S;
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int k) const { return k == 0 ? Uh : dU; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[4][V]) const {
-    ldv<V>(Uh + q, in[0]);
-    ldv<V>(Uh + P + q, in[1]);
-    if (third != 0.f) {
-      ldv<V>(dU + q, in[2]);
-      ldv<V>(dU + P + q, in[3]);
-    } else {
-#pragma unroll
-      for (int v = 0; v < V; ++v) in[2][v] = in[3][v] = 0.f;
-    }
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[4][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], dr[V], di[V], ur[V], ui[V];
-    lam_eval<V>(L, i, r, lr, li);
+    lam_of<V>(L, sv, lr, li);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float zr = theta * lr[v], zi = theta * li[v];
       const float ar = 1.f - zr, ai = -zi, inv = 1.f / (ar * ar + ai * ai);
       const float fr = ar * inv, fi = -ai * inv;   // (1 - z)^{-1}
       const float xr = in[0][v], xi = in[1][v];
-      const float br = third * in[2][v] + (zr * xr - zi * xi) + theta * re[v];
-      const float bi = third * in[3][v] + (zr * xi + zi * xr) + theta * im[v];
+      const float pr = third != 0.f ? in[2][v] : 0.f, pi = third != 0.f ? in[3][v] : 0.f;   // the first step has no dU^
+      const float br = third * pr + (zr * xr - zi * xi) + theta * re[v];
+      const float bi = third * pi + (zr * xi + zi * xr) + theta * im[v];
       dr[v] = fr * br - fi * bi;
       di[v] = fr * bi + fi * br;
       ur[v] = xr + dr[v];
@@ -783,27 +759,24 @@ struct EpiLBDF2S {
     stv<V>(dU + P + q, di);
     stv<V>(Uh + q, ur);
     stv<V>(Uh + P + q, ui);
-    put_csplit<V>(S, P, q, ur, ui);
+    emit_csplit<V>(em, S, P, q, ur, ui);
   }
 };
 
 // LBDF2 backward epilogue: u_{n+1} = product -> U (u_n read from U first);
 // g(t, 2 u_{n+1} - u_n) -> split, the input of the next step's forward operator
 struct EpiExtrapG {
-  FCGLE_EPI(2, 4)
+  FCGLE_EPI(2, false, true)
   uint32_t P;
   float* U;
   GStatic g;
   GTime t;
   SplitOut S;
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return U; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(U + q, in[0]);
-    ldv<V>(U + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float er[V], ei[V], gr[V], gi[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -812,8 +785,8 @@ struct EpiExtrapG {
     }
     stv<V>(U + q, re);
     stv<V>(U + P + q, im);
-    g_eval<V>(g, t, P, q, er, ei, gr, gi);
-    put_csplit<V>(S, P, q, gr, gi);
+    g_eval<V>(g, t, P, q, er, ei, gr, gi, src);
+    emit_csplit<V>(em, S, P, q, gr, gi);
   }
 };
 
@@ -822,29 +795,27 @@ struct EpiExtrapG {
 // V^ = e^z (U^ + tau K^_1) -> split (v = bwd(V^) is the Heun predictor),
 // W^ = e^z (U^ + tau/2 K^_1) -> W (FP32)
 struct EpiLRK2A {
-  FCGLE_EPI(2, 4)
+  FCGLE_EPI(2, true, false)
   uint32_t P;
   LamF L;
   const float* Uh;
   float* W;
   float tau;
   SplitOut S;
+  PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return Uh; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv_ro<V>(Uh + q, in[0]);
-    ldv_ro<V>(Uh + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int i, uint32_t r, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], vr[V], vi[V], wr[V], wi[V];
-    lam_eval<V>(L, i, r, lr, li);
+    lam_of<V>(L, sv, lr, li);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float zr = tau * lr[v], zi = tau * li[v];
-      float pr, pi;
-      phi1f(zr, zi, pr, pi);
-      const float mr = zr * pr - zi * pi, mi = zr * pi + zi * pr;   // e^z - 1
+      float pr[3], pi[3];
+      phi123_s(ph, sv[v], pr, pi);
+      const float mr = zr * pr[0] - zi * pi[0], mi = zr * pi[0] + zi * pr[0];   // e^z - 1
       const float fr = 1.f + mr, fi = mi;                           // e^z
       const float xr = in[0][v], xi = in[1][v];
       const float br = xr + (mr * xr - mi * xi), bi = xi + (mr * xi + mi * xr);   // e^z U^
@@ -854,7 +825,7 @@ struct EpiLRK2A {
       wr[v] = br + 0.5f * tau * kr;
       wi[v] = bi + 0.5f * tau * ki;
     }
-    put_csplit<V>(S, P, q, vr, vi);
+    emit_csplit<V>(em, S, P, q, vr, vi);
     stv<V>(W + q, wr);
     stv<V>(W + P + q, wi);
   }
@@ -863,20 +834,17 @@ struct EpiLRK2A {
 // Lawson-RK2 second forward epilogue: product = fwd(g(t_{n+1}, v)):
 // U^_{n+1} = W^ + tau/2 product -> Uh and -> split
 struct EpiLRK2B {
-  FCGLE_EPI(2, 4)
+  FCGLE_EPI(2, false, false)
   uint32_t P;
   const float* W;
   float* Uh;
   float tau;
   SplitOut S;
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return W; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv_ro<V>(W + q, in[0]);
-    ldv_ro<V>(W + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -885,36 +853,38 @@ struct EpiLRK2B {
     }
     stv<V>(Uh + q, ur);
     stv<V>(Uh + P + q, ui);
-    put_csplit<V>(S, P, q, ur, ui);
+    emit_csplit<V>(em, S, P, q, ur, ui);
   }
 };
 // Exact flow of w' = gamma w - (kappa + i zeta)|w|^2 w over time t (Sec. 4):
 // w(t) = exp(t gamma - (kappa + i zeta)/(2 kappa) log(1 + 2 t phi_1(2 gamma t) kappa |w0|^2)) w0
 struct Flow {
   float gamma_t;   // t gamma
+  float growth;    // e^{t gamma}
   float c2;        // 2 t phi_1(2 gamma t) kappa
   float zk;        // zeta / (2 kappa)
 };
+// The modulus e^{t gamma - L / 2} = e^{t gamma} (1 + c2 |w|^2)^{-1/2}.
 __device__ __forceinline__ void flow_eval(const Flow& f, float wr, float wi, float& yr, float& yi) {
-  const float L = log1pf(f.c2 * (wr * wr + wi * wi));
-  const float m = expf(f.gamma_t - 0.5f * L);
+  const float x = f.c2 * (wr * wr + wi * wi);
+  const float m = f.growth * rsqrtf(1.f + x);
   float s, c;
-  sincosf(-f.zk * L, &s, &c);
+  sincosf(-f.zk * log1pf(x), &s, &c);
   yr = m * (c * wr - s * wi);
   yi = m * (c * wi + s * wr);
 }
 
 // Phi_t(w) - w = (e^E - 1) w with E = t gamma - (1 + i zeta/kappa) L / 2,
 // L = log(1 + c2 |w|^2): e^E - 1 = expm1(Re E) cos(Im E) - 2 sin^2(Im E / 2)
-// + i e^{Re E} sin(Im E), without cancellation for small t.
+// + i e^{Re E} sin(Im E), without cancellation for small t; cos and sin of Im E
+// from those of Im E / 2.
 __device__ __forceinline__ void flow_incr(const Flow& f, float wr, float wi, float& dr, float& di) {
   const float L = log1pf(f.c2 * (wr * wr + wi * wi));
-  const float a = f.gamma_t - 0.5f * L, b = -f.zk * L;
-  float s, c, sh, ch;
-  sincosf(b, &s, &c);
-  sincosf(0.5f * b, &sh, &ch);
-  const float em = expm1f(a);
-  const float er = em * c - 2.f * sh * sh, ei = (1.f + em) * s;
+  float sh, ch;
+  sincosf(-0.5f * f.zk * L, &sh, &ch);
+  const float em = expm1f(f.gamma_t - 0.5f * L);
+  const float v = 2.f * sh * sh;                 // 1 - cos(Im E)
+  const float er = em * (1.f - v) - v, ei = (1.f + em) * (2.f * sh * ch);
   dr = er * wr - ei * wi;
   di = er * wi + ei * wr;
 }
@@ -924,16 +894,16 @@ __device__ __forceinline__ void flow_incr(const Flow& f, float wr, float wi, flo
 // increment Phi_tau(w) - w -> split, which the next step's forward operator
 // turns into e^ <- e^{tau Lam}(e^ + fwd(Phi_tau(w) - w)) (EpiSpecStep, c = 1).
 struct EpiStrangB {
-  FCGLE_EPI(0, 4)
+  FCGLE_EPI(0, false, false)
   uint32_t P;
   float* U;
   Flow half, full;
   SplitOut S;
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t, int, uint32_t, float (&)[1][V]) const {}
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&)[1][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V], dr[V], di[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -942,7 +912,7 @@ struct EpiStrangB {
     }
     stv<V>(U + q, ur);
     stv<V>(U + P + q, ui);
-    put_csplit<V>(S, P, q, dr, di);
+    emit_csplit<V>(em, S, P, q, dr, di);
   }
 };
 
@@ -953,16 +923,16 @@ struct EpiStrangB {
 // and the next step's input Phi_{tau/2}(u_{n+1}) = Phi_tau(w) (the flows of the
 // autonomous nonlinear part compose) -> split
 struct EpiStrangKron {
-  FCGLE_EPI(0, 4)
+  FCGLE_EPI(0, false, false)
   uint32_t P;
   float* U;
   Flow half, full;
   SplitOut S;
+  __device__ SplitOut split() const { return S; }
+  __device__ const float* src(int) const { return nullptr; }
   template <int V>
-  __device__ void load(uint32_t, int, uint32_t, float (&)[1][V]) const {}
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&)[1][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V], sr[V], si[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -971,7 +941,7 @@ struct EpiStrangKron {
     }
     stv<V>(U + q, ur);
     stv<V>(U + P + q, ui);
-    put_csplit<V>(S, P, q, sr, si);
+    emit_csplit<V>(em, S, P, q, sr, si);
   }
 };
 
@@ -980,7 +950,7 @@ struct EpiStrangKron {
 //   u_{n+1} = product + tau/2 g(t_{n+1}, A);
 // the next step's inputs u_{n+1} + tau g(t_{n+1}, u_{n+1}) and u_{n+1} + tau/2 g(...) -> split
 struct EpiLRK2Kron {
-  FCGLE_EPI(2, 2)
+  FCGLE_EPI(2, false, true)
   uint32_t P;
   const float* A;
   float* U;
@@ -988,16 +958,13 @@ struct EpiLRK2Kron {
   GTime t;   // t_{n+1}
   float tau;
   SplitOut V1, V2;
+  __device__ SplitOut split() const { return V1; }
+  __device__ const float* src(int) const { return A; }
   template <int V>
-  __device__ void load(uint32_t q, int, uint32_t, float (&in)[2][V]) const {
-    ldv<V>(A + q, in[0]);
-    ldv<V>(A + P + q, in[1]);
-  }
-  template <int V>
-  __device__ void store(uint32_t q, int, uint32_t, const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V]) const {
+  __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float gr[V], gi[V], ur[V], ui[V];
-    g_eval<V>(g, t, P, q, in[0], in[1], gr, gi);
+    g_eval<V>(g, t, P, q, in[0], in[1], gr, gi, src);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       ur[v] = re[v] + 0.5f * tau * gr[v];
@@ -1005,14 +972,14 @@ struct EpiLRK2Kron {
     }
     stv<V>(U + q, ur);
     stv<V>(U + P + q, ui);
-    g_eval<V>(g, t, P, q, ur, ui, gr, gi);
+    g_eval<V>(g, t, P, q, ur, ui, gr, gi, src);
     float ar[V], ai[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       ar[v] = ur[v] + tau * gr[v];
       ai[v] = ui[v] + tau * gi[v];
     }
-    put_csplit<V>(V1, P, q, ar, ai);
+    emit_csplit<V>(em, V1, P, q, ar, ai);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       ar[v] = ur[v] + 0.5f * tau * gr[v];

@@ -31,6 +31,7 @@
 #include "adjoint.h"
 #include "b3_epilogues.cuh"
 #include "b3_kernel.cuh"
+#include "b3_launch.h"
 #include "b3_plain.cuh"
 #include "b3_slab.cuh"
 #include "engine.h"
@@ -452,45 +453,29 @@ class EngineB3 : public EngineBase {
     // an exception leaves the flag unset, so a later setup retries
     static std::once_flag attrs;
     std::call_once(attrs, [] {
-      set_smem_attr<b3::EpiStoreSplitGen>();
-      set_smem_attr<b3::EpiStoreF32>();
-      set_smem_attr<b3::EpiScaleF>();
-      set_smem_attr<b3::EpiUpdateG>();
-      set_smem_attr<b3::EpiStageD>();
-      set_smem_attr<b3::EpiFhat>();
-      set_smem_attr<b3::EpiKrog2>();
-      set_smem_attr<b3::EpiKrog3>();
-      set_smem_attr<b3::EpiKrogFinal>();
-      set_smem_attr<b3::EpiEtd2>();
-      set_smem_attr<b3::EpiSpecStep>();
-      set_smem_attr<b3::EpiLBDF2S>();
-      set_smem_attr<b3::EpiExtrapG>();
-      set_smem_attr<b3::EpiLRK2A>();
-      set_smem_attr<b3::EpiLRK2B>();
-      set_smem_attr<b3::EpiStrangB>();
-      set_smem_attr_mn<b3::EpiStoreSplitGen>();
-      set_smem_attr_mn<b3::EpiStoreF32>();
-      set_smem_attr_mn<b3::EpiScaleF>();
-      set_smem_attr_mn<b3::EpiUpdateG>();
-      set_smem_attr_mn<b3::EpiStageD>();
-      set_smem_attr_mn<b3::EpiFhat>();
-      set_smem_attr_mn<b3::EpiKrog2>();
-      set_smem_attr_mn<b3::EpiKrog3>();
-      set_smem_attr_mn<b3::EpiKrogFinal>();
-      set_smem_attr_mn<b3::EpiEtd2>();
-      set_smem_attr_mn<b3::EpiSpecStep>();
-      set_smem_attr_mn<b3::EpiLBDF2S>();
-      set_smem_attr_mn<b3::EpiExtrapG>();
-      set_smem_attr_mn<b3::EpiLRK2A>();
-      set_smem_attr_mn<b3::EpiLRK2B>();
-      set_smem_attr_mn<b3::EpiStrangB>();
+      FusedLaunch<b3::EpiStoreSplitGen>::attributes();
+      FusedLaunch<b3::EpiStoreF32>::attributes();
+      FusedLaunch<b3::EpiScaleF>::attributes();
+      FusedLaunch<b3::EpiUpdateG>::attributes();
+      FusedLaunch<b3::EpiStageD>::attributes();
+      FusedLaunch<b3::EpiFhat>::attributes();
+      FusedLaunch<b3::EpiKrog2>::attributes();
+      FusedLaunch<b3::EpiKrog3>::attributes();
+      FusedLaunch<b3::EpiKrogFinal>::attributes();
+      FusedLaunch<b3::EpiEtd2>::attributes();
+      FusedLaunch<b3::EpiSpecStep>::attributes();
+      FusedLaunch<b3::EpiLBDF2S>::attributes();
+      FusedLaunch<b3::EpiExtrapG>::attributes();
+      FusedLaunch<b3::EpiLRK2A>::attributes();
+      FusedLaunch<b3::EpiLRK2B>::attributes();
+      FusedLaunch<b3::EpiStrangB>::attributes();
       FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_slab12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)b3::kSlSmemBytes));
-      set_smem_attr_cx<b3::EpiStoreF32>();
-      set_smem_attr_cx<b3::EpiStoreSplitGen>();
-      set_smem_attr_cx<b3::EpiUpdateG>();
-      set_smem_attr_cx<b3::EpiStrangKron>();
-      set_smem_attr_cx<b3::EpiLRK2Kron>();
+      FusedLaunchCx<b3::EpiStoreF32>::attributes();
+      FusedLaunchCx<b3::EpiStoreSplitGen>::attributes();
+      FusedLaunchCx<b3::EpiUpdateG>::attributes();
+      FusedLaunchCx<b3::EpiStrangKron>::attributes();
+      FusedLaunchCx<b3::EpiLRK2Kron>::attributes();
       FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_plain_kernel<false, b3::kOpBF16, 2, false, true>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b3::kPlSmemBytes));
       FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_plain_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -719,7 +704,7 @@ class EngineB3 : public EngineBase {
     SplitOut V = SP(kV), G = SP(kW);
     to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), Uh, V);
     FCGLE_LAUNCHED(launches);
-    tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t), 0.f, 1.f, G});
+    tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t), 0.f, 1.f, G});
     tucker(G, true, b3::EpiStoreF32{P32(), K});
   }
 
@@ -775,20 +760,15 @@ class EngineB3 : public EngineBase {
   uint32_t P32() const { return (uint32_t)s_.P; }
   SplitOut SP(int i) { return SplitOut{sp_[i]->ptr, sp_[i]->ptr + 2 * s_.P}; }
 
+  // one single-problem fused launch; natural_order: X[c][k][r]
   template <class Epi>
-  static void set_smem_attr() {
-    FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_kernel<Epi, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)b3::Cfg<Epi>::kSmemBytes));
-  }
-  template <class Epi>
-  static void set_smem_attr_mn() {
-    FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_kernel<Epi, false, false, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b3::Cfg<Epi>::kSmemBytes));
-  }
-  template <class Epi>
-  static void set_smem_attr_cx() {
-    FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_kernel<Epi, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)b3::Cfg<Epi, true>::kSmemBytes));
+  void launch_fused(bool natural_order, const CUtensorMap& txh, const CUtensorMap& txl, const Mat& m, b3::KParams kp,
+                    const Epi& epi) {
+    kp.mhi = m.hi;
+    kp.mlo = m.lo;
+    kp.k_pad = m.k_pad;
+    FusedLaunch<Epi>::single(natural_order, FusedMaps{txh, txl, m.tm_hi, m.tm_lo}, kp, epi, st_);
+    FCGLE_LAUNCHED(launches);
   }
 
   // ---- Kronecker-product form of the exponential (Eq. Neudeckerd)
@@ -882,11 +862,7 @@ class EngineB3 : public EngineBase {
     CUtensorMap txh, txl;
     encode_bf16(&txh, xh, (uint64_t)s_.p[mu], 2 * (uint64_t)kp.R, b3::BR);
     encode_bf16(&txl, xl, (uint64_t)s_.p[mu], 2 * (uint64_t)kp.R, b3::BR);
-    const long long units = kp.tiles * kp.m_blocks;
-    const int grid = (int)std::min<long long>(units, num_sms());
-    launch_pdl(b3::mp_b3_kernel<Epi, false, true>, grid, b3::Cfg<Epi, true>::kThreads,
-               b3::Cfg<Epi, true>::kSmemBytes, st_, txh, txl, c.tm_hi, c.tm_lo, kp, epi,
-               (const b3::FusedDesc<Epi>*)nullptr, 0, 0LL);
+    FusedLaunchCx<Epi>::single(FusedMaps{txh, txl, c.tm_hi, c.tm_lo}, kp, epi, st_);
     FCGLE_LAUNCHED(launches);
   }
 
@@ -1308,21 +1284,6 @@ class EngineB3 : public EngineBase {
     launch_pdl(b3::mp_b3_plain_kernel<true, b3::kOpBF16, NXR>, grid, b3::PL_THREADS, b3::kPlSmemBytes, st, z, z, z, z,
                z, z, kp, static_cast<const b3::PlainDesc*>(descs), n, units);
   }
-  template <class Epi>
-  static void launch_fused_grouped(const void* descs, int n, long long units, cudaStream_t st) {
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-      FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_kernel<Epi, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)b3::Cfg<Epi>::kSmemBytes));
-    });
-    CUtensorMap z;
-    std::memset(&z, 0, sizeof(z));
-    b3::KParams kp{};
-    const int grid = (int)std::min<long long>(units, num_sms());
-    launch_pdl(b3::mp_b3_kernel<Epi, true>, grid, b3::Cfg<Epi>::kThreads, b3::Cfg<Epi>::kSmemBytes, st, z, z, z, z,
-               kp, Epi{}, static_cast<const b3::FusedDesc<Epi>*>(descs), n, units);
-  }
-
   // one mode product of direction mu on split input (xh, xl) with epilogue epi
   template <class Epi>
   void launch_mp(const __nv_bfloat16* xh, const __nv_bfloat16* xl, int mu, bool fwd, const Epi& epi) {
@@ -1339,7 +1300,6 @@ class EngineB3 : public EngineBase {
     kp.tiles = (R + b3::BR - 1) / b3::BR;
     kp.err = err_->ptr;
     const long long units = kp.tiles * kp.m_blocks;
-    const int grid = (int)std::min<long long>(units, num_sms());
     if (rec_) {
       b3::FusedDesc<Epi> d;
       std::memset(static_cast<void*>(&d), 0, sizeof(d));
@@ -1349,12 +1309,10 @@ class EngineB3 : public EngineBase {
       d.mlo = m.tm_lo;
       d.kp = kp;
       d.epi = epi;
-      record(last_mp_, &launch_fused_grouped<Epi>, offsetof(b3::FusedDesc<Epi>, ubegin), &d, sizeof(d), units);
+      record(last_mp_, &FusedLaunch<Epi>::grouped, offsetof(b3::FusedDesc<Epi>, ubegin), &d, sizeof(d), units);
       return;
     }
-    launch_pdl(b3::mp_b3_kernel<Epi, false>, grid, b3::Cfg<Epi>::kThreads, b3::Cfg<Epi>::kSmemBytes, st_, txh, txl,
-               m.tm_hi, m.tm_lo, kp, epi, (const b3::FusedDesc<Epi>*)nullptr, 0, 0LL);
-    FCGLE_LAUNCHED(launches);
+    launch_fused(false, txh, txl, m, kp, epi);
   }
 
   // ---- slab-fused modes 1 + 2 and the natural-order mode-3 product (d == 3)
@@ -1409,11 +1367,7 @@ class EngineB3 : public EngineBase {
     kp.k_chunks = m.k_pad / b3::BK;
     kp.tiles = (R + b3::BR - 1) / b3::BR;
     kp.err = err_->ptr;
-    const long long units = kp.tiles * kp.m_blocks;
-    const int grid = (int)std::min<long long>(units, num_sms());
-    launch_pdl(b3::mp_b3_kernel<Epi, false, false, true>, grid, b3::Cfg<Epi>::kThreads, b3::Cfg<Epi>::kSmemBytes, st_,
-               txh, txl, m.tm_hi, m.tm_lo, kp, epi, (const b3::FusedDesc<Epi>*)nullptr, 0, 0LL);
-    FCGLE_LAUNCHED(launches);
+    launch_fused(true, txh, txl, m, kp, epi);
   }
 
   // Tucker operator on the split tensor `in` (consumed); the last mode product
@@ -1475,6 +1429,7 @@ class EngineB3 : public EngineBase {
     const double p1 = std::fabs(z) < 1e-8 ? 1.0 + z / 2.0 : std::expm1(z) / z;
     b3::Flow f;
     f.gamma_t = (float)(t * prm_.gamma);
+    f.growth = (float)std::exp(t * prm_.gamma);
     f.c2 = (float)(2.0 * t * p1 * prm_.kappa);
     f.zk = (float)(prm_.zeta / (2.0 * prm_.kappa));
     return f;
@@ -1583,7 +1538,7 @@ class EngineB3 : public EngineBase {
     if (kron_scheme(scheme)) {
       if (scheme == FCGLE_LAWSON_EULER) {
         // u_{n+1} = e^{tau K}(u_n + tau g_n);  V = u_{n+1} + tau g(t_{n+1}, u_{n+1})
-        exp_kron(V, tau, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t + tau), 1.f, ft, V});
+        exp_kron(V, tau, b3::EpiUpdateG{P32(), U, gs_, gtime(t + tau), 1.f, ft, V});
       } else if (scheme == FCGLE_STRANG) {
         // w = e^{tau K} Phi_{tau/2}(u_n);  u_{n+1} = Phi_{tau/2}(w);  V = Phi_tau(w)
         exp_kron(V, tau, b3::EpiStrangKron{P32(), U, flow(tau / 2), flow(tau), V});
@@ -1600,25 +1555,25 @@ class EngineB3 : public EngineBase {
       case FCGLE_LAWSON_EULER: {
         // U^ <- f(tau Lam)(U^ + tau G^), f = 1/(1 - z) or e^z;  u_{n+1} = bwd(U^);  V = g(t_{n+1}, u_{n+1})
         const int kind = scheme == FCGLE_LIE ? 0 : 1;
-        tucker(V, true, b3::EpiSpecStep{P32(), lf_, F32(kUh), kind, ft, ft, V});
-        tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t + tau), 0.f, 1.f, V});
+        tucker(V, true, b3::EpiSpecStep{P32(), lf_, F32(kUh), kind, ft, ft, V, phipoly(tau)});
+        tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t + tau), 0.f, 1.f, V});
         break;
       }
       case FCGLE_STRANG: {
         // e^ <- e^{tau Lam}(e^ + fwd(increment));  w = bwd(e^);  u_{n+1} = Phi_{tau/2}(w);
         // next increment Phi_tau(w) - w
-        tucker(V, true, b3::EpiSpecStep{P32(), lf_, F32(kUh), 1, ft, 1.f, V});
+        tucker(V, true, b3::EpiSpecStep{P32(), lf_, F32(kUh), 1, ft, 1.f, V, phipoly(tau)});
         tucker(V, false, b3::EpiStrangB{P32(), U, flow(tau / 2), flow(tau), V});
         break;
       }
       case FCGLE_LAWSON_RK2: {
         float *Uh = F32(kUh), *Wh = F32(kEA);
         // V^ = e^z (U^ + tau K^_1) -> v = bwd(V^);  W^ = e^z (U^ + tau/2 K^_1)
-        tucker(V, true, b3::EpiLRK2A{P32(), lf_, Uh, Wh, ft, V});
-        tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t + tau), 0.f, 1.f, V});
+        tucker(V, true, b3::EpiLRK2A{P32(), lf_, Uh, Wh, ft, V, phipoly(tau)});
+        tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t + tau), 0.f, 1.f, V});
         // U^_{n+1} = W^ + tau/2 fwd(g(t_{n+1}, v));  u_{n+1} = bwd(U^_{n+1})
         tucker(V, true, b3::EpiLRK2B{P32(), Wh, Uh, ft, V});
-        tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t + tau), 0.f, 1.f, V});
+        tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t + tau), 0.f, 1.f, V});
         break;
       }
       case FCGLE_LBDF2: {
@@ -1639,7 +1594,7 @@ class EngineB3 : public EngineBase {
         // U^_{n+1} = a^ + tau phi_2(tau Lam) o D^
         tucker(V, true, b3::EpiEtd2{P32(), lf_, Uh, ft, V, phipoly(tau)});
         // u_{n+1} = bwd(U^_{n+1});  next G = g(t + tau, u_{n+1})
-        tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, gtime(t + tau), 0.f, 1.f, V});
+        tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t + tau), 0.f, 1.f, V});
         break;
       }
       case FCGLE_KROGSTAD: {
@@ -1658,7 +1613,7 @@ class EngineB3 : public EngineBase {
         // D^_4;  U^_{n+1} = U^ + W + tau (4 phi_3 - phi_2) D^_4
         tucker(V, true, b3::EpiKrogFinal{P32(), lf_, Wc, Uh, ft, V, phipoly(tau)});
         // u_{n+1} = bwd(U^_{n+1});  next G = g(t + tau, u_{n+1})
-        tucker(V, false, b3::EpiUpdateG{P32(), U, 0, gs_, t1, 0.f, 1.f, V});
+        tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, t1, 0.f, 1.f, V});
         break;
       }
       default: throw InvalidArg("unknown scheme");
