@@ -236,7 +236,8 @@ fcgle_status fcgle_integrate_host(fcgle_handle h, int scheme, double tau, int ns
  * grad_params[5] (host) = dJ/d(nu, eta, gamma, kappa, zeta); *loss (host) = J.
  * States are checkpointed every ckpt_every steps (0: one segment) and each
  * segment is recomputed once, so the cost is about three forward runs and
- * the extra device memory (5 ckpt_every + nsteps / ckpt_every + 9) tensors.
+ * the extra device memory (4 ckpt_every + nsteps / ckpt_every + 8) tensors, of
+ * which up to 2 GiB stay with the handle for the next call.
  * Synchronises the stream and reports device-side failures as fcgle_sync does;
  * a non-finite loss or parameter gradient gives FCGLE_ERR_NUMERIC.  The
  * exponential is applied in the Tucker form (Eq. fKu_diag with f = exp). */

@@ -4,6 +4,8 @@
 #include <cmath>
 #include <type_traits>
 
+#include <cuda_bf16.h>
+
 #include "adjoint.h"
 
 namespace fcgle {
@@ -241,6 +243,24 @@ __device__ __forceinline__ void st4f(float* p, const float (&v)[4]) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// 4 values as bf16 hi + lo at sp.hi[q..], sp.lo[q..] (sp.hi null: nothing)
+__device__ __forceinline__ void split4(const AdjSplit& sp, uint32_t q, const float (&x)[4]) {
+  if (!sp.hi) return;
+  uint2 h, l;
+  uint32_t* hp = &h.x;
+  uint32_t* lp = &l.x;
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(x[2 * v], x[2 * v + 1]);
+    const float2 f = __bfloat1622float2(a);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(x[2 * v] - f.x, x[2 * v + 1] - f.y);
+    hp[v] = *reinterpret_cast<const uint32_t*>(&a);
+    lp[v] = *reinterpret_cast<const uint32_t*>(&b);
+  }
+  *reinterpret_cast<uint2*>(sp.hi + q) = h;
+  *reinterpret_cast<uint2*>(sp.lo + q) = l;
+}
+
 __device__ __forceinline__ void gadj_f(float gam, float kap, float zet, float zr, float zi, float wr, float wi,
                                        float& orr, float& oi) {
   const float m2 = zr * zr + zi * zi;
@@ -252,7 +272,7 @@ __device__ __forceinline__ void gadj_f(float gam, float kap, float zet, float zr
 }
 
 __global__ void gv_kernel_f(uint32_t P, GP g, const float* __restrict__ z, const float* __restrict__ w, float c,
-                            float* __restrict__ mu, double* acc) {
+                            float* __restrict__ mu, AdjSplit sp, double* acc) {
   float f[3] = {0.f, 0.f, 0.f};
   const float gam = (float)g.gamma, kap = (float)g.kappa, zet = (float)g.zeta;
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
@@ -273,8 +293,12 @@ __global__ void gv_kernel_f(uint32_t P, GP g, const float* __restrict__ z, const
       f[1] -= m2 * dd;
       f[2] -= m2 * ee;
     }
-    st4f(mu + q, orr);
-    st4f(mu + P + q, oi);
+    if (mu) {
+      st4f(mu + q, orr);
+      st4f(mu + P + q, oi);
+    }
+    split4(sp, q, orr);
+    split4(sp, P + q, oi);
   }
   double v[3] = {(double)f[0], (double)f[1], (double)f[2]};
   block_acc<3>(v, acc, ADJ_GAMMA);
@@ -302,7 +326,7 @@ __device__ __forceinline__ void expm1_z_f(const Quad& Q, int v, float ar, float 
 // y1 = e^z (x + c1 k), y2 = e^z (x + c2 k) (FP32 form of exp_pair_kernel)
 __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const float* __restrict__ x,
                                   const float* __restrict__ k, float c1, float c2, float* __restrict__ y1,
-                                  float* __restrict__ y2) {
+                                  float* __restrict__ y2, AdjSplit sp) {
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     const Quad Q = quad_lam(L, q);
     float xr[4], xi[4], kr[4], ki[4], pr[4], pi[4], wr[4], wi[4];
@@ -321,8 +345,12 @@ __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const fl
       wr[v] = vr + (mr * vr - mi * vi);
       wi[v] = vi + (mr * vi + mi * vr);
     }
-    st4f(y1 + q, pr);
-    st4f(y1 + P + q, pi);
+    if (y1) {
+      st4f(y1 + q, pr);
+      st4f(y1 + P + q, pi);
+    }
+    split4(sp, q, pr);
+    split4(sp, P + q, pi);
     st4f(y2 + q, wr);
     st4f(y2 + P + q, wi);
   }
@@ -330,7 +358,7 @@ __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const fl
 
 // a = e^z x, b = e^z m; y = ca a + cb b, sum = a + b (FP32 form of exp_combo_kernel; y may alias x)
 __global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const float* x, const float* __restrict__ m,
-                                   float ca, float cb, float* y, float* __restrict__ sum) {
+                                   float ca, float cb, float* y, float* __restrict__ sum, AdjSplit sp) {
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     const Quad Q = quad_lam(L, q);
     float xr[4], xi[4], nr[4], ni[4], yr[4], yi[4], sr[4], si[4];
@@ -349,8 +377,12 @@ __global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const f
       sr[v] = a_r + b_r;
       si[v] = a_i + b_i;
     }
-    st4f(y + q, yr);
-    st4f(y + P + q, yi);
+    if (y) {
+      st4f(y + q, yr);
+      st4f(y + P + q, yi);
+    }
+    split4(sp, q, yr);
+    split4(sp, P + q, yi);
     st4f(sum + q, sr);
     st4f(sum + P + q, si);
   }
@@ -378,7 +410,7 @@ __global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* __restrict__ x,
 }
 
 __global__ void axpby_kernel_f(uint32_t n, float a, const float* __restrict__ x1, float b,
-                               const float* __restrict__ x2, float* __restrict__ y) {
+                               const float* __restrict__ x2, float* __restrict__ y, AdjSplit sp) {
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float u[4], w[4] = {0.f, 0.f, 0.f, 0.f};
     ld4f(x1 + q, u);
@@ -386,6 +418,7 @@ __global__ void axpby_kernel_f(uint32_t n, float a, const float* __restrict__ x1
 #pragma unroll
     for (int v = 0; v < 4; ++v) u[v] = a * u[v] + b * w[v];
     st4f(y + q, u);
+    split4(sp, q, u);
   }
 }
 
@@ -408,11 +441,11 @@ void adj_misfit(const Shape& s, const T* u, const T* target, T* lam, double* acc
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
-void adj_gv(const Shape& s, const GParams& gp, const T* z, const T* w, double c, T* mu, double* acc, cudaStream_t st,
-            long long& nl) {
+void adj_gv(const Shape& s, const GParams& gp, const T* z, const T* w, double c, T* mu, AdjSplit sp, double* acc,
+            cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
     gv_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, (float)c,
-                                                   mu, acc);
+                                                   mu, sp, acc);
   else
     gv_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, c, mu, acc);
   FCGLE_LAUNCHED(nl);
@@ -433,9 +466,11 @@ void adj_spec_dot(const Shape& s, const LamVecs& lv, const T* x, const T* y, dou
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
-void adj_axpby(const Shape& s, double a, const T* x1, double b, const T* x2, T* y, cudaStream_t st, long long& nl) {
+void adj_axpby(const Shape& s, double a, const T* x1, double b, const T* x2, T* y, AdjSplit sp, cudaStream_t st,
+               long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    axpby_kernel_f<<<grid_of(2 * s.P / 4), 256, 0, st>>>((uint32_t)(2 * s.P), (float)a, x1, (float)b, x2, y);
+    axpby_kernel_f<<<grid_of(2 * s.P / 4), 256, 0, st>>>((uint32_t)(2 * s.P), (float)a, x1, (float)b, x2, y,
+                                                         sp);
   else
     axpby_kernel<T><<<grid_of(2 * s.P), 256, 0, st>>>(2 * s.P, a, x1, b, x2, y);
   FCGLE_LAUNCHED(nl);
@@ -443,10 +478,11 @@ void adj_axpby(const Shape& s, double a, const T* x1, double b, const T* x2, T* 
 
 template <typename T>
 void adj_exp_pair(const Shape& s, const LamVecs& lv, double theta, const T* x, const T* k, double c1, double c2,
-                  T* y1, T* y2, cudaStream_t st, long long& nl) {
+                  T* y1, T* y2, AdjSplit sp1, cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
     exp_pair_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
-                                                     (float)(theta * lv.c_im), x, k, (float)c1, (float)c2, y1, y2);
+                                                     (float)(theta * lv.c_im), x, k, (float)c1, (float)c2, y1, y2,
+                                                     sp1);
   else
     exp_pair_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, make_ld(s, lv), theta * lv.c_re, theta * lv.c_im, x, k,
                                                        c1, c2, y1, y2);
@@ -454,10 +490,11 @@ void adj_exp_pair(const Shape& s, const LamVecs& lv, double theta, const T* x, c
 }
 template <typename T>
 void adj_exp_h_combo(const Shape& s, const LamVecs& lv, double theta, const T* x, const T* m, double ca, double cb,
-                     T* y, T* sum, cudaStream_t st, long long& nl) {
+                     T* y, T* sum, AdjSplit spy, cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
     exp_combo_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
-                                                      (float)(-theta * lv.c_im), x, m, (float)ca, (float)cb, y, sum);
+                                                      (float)(-theta * lv.c_im), x, m, (float)ca, (float)cb, y, sum,
+                                                      spy);
   else
     exp_combo_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, make_ld(s, lv), theta * lv.c_re, -theta * lv.c_im, x, m,
                                                         ca, cb, y, sum);
@@ -466,17 +503,18 @@ void adj_exp_h_combo(const Shape& s, const LamVecs& lv, double theta, const T* x
 
 #define INST(T)                                                                                                  \
   template void adj_misfit<T>(const Shape&, const T*, const T*, T*, double*, cudaStream_t, long long&);          \
-  template void adj_gv<T>(const Shape&, const GParams&, const T*, const T*, double, T*, double*, cudaStream_t,  \
-                          long long&);                                                                          \
+  template void adj_gv<T>(const Shape&, const GParams&, const T*, const T*, double, T*, AdjSplit, double*,       \
+                          cudaStream_t, long long&);                                                            \
   template void adj_gu<T>(const Shape&, const GParams&, const T*, const T*, const T*, double, double, T*,       \
                           double*, cudaStream_t, long long&);                                                   \
   template void adj_spec_dot<T>(const Shape&, const LamVecs&, const T*, const T*, double*, cudaStream_t,        \
                                 long long&);                                                                    \
-  template void adj_axpby<T>(const Shape&, double, const T*, double, const T*, T*, cudaStream_t, long long&);    \
+  template void adj_axpby<T>(const Shape&, double, const T*, double, const T*, T*, AdjSplit, cudaStream_t,        \
+                             long long&);                                                                        \
   template void adj_exp_pair<T>(const Shape&, const LamVecs&, double, const T*, const T*, double, double, T*, T*, \
-                                cudaStream_t, long long&);                                                       \
+                                AdjSplit, cudaStream_t, long long&);                                                       \
   template void adj_exp_h_combo<T>(const Shape&, const LamVecs&, double, const T*, const T*, double, double, T*,  \
-                                   T*, cudaStream_t, long long&);
+                                   T*, AdjSplit, cudaStream_t, long long&);
 INST(float)
 INST(double)
 #undef INST

@@ -314,15 +314,33 @@ class Engine : public EngineBase {
   long long& nlaunch() { return launches; }
   GParams gparams() const { return gp_; }
   LamVecs lamvecs() const { return lv_; }
-  T* alloc(size_t n) {
-    adj_mem_.emplace_back(new DevBuf<T>(n));
-    return adj_mem_.back()->ptr;
+  static constexpr bool kSplit = false;
+  static size_t padded(size_t n) { return (n + 63) / 64 * 64; }
+  void reserve(size_t n) {
+    if (adj_size_ < n) {
+      adj_mem_.reset();
+      adj_size_ = 0;
+      adj_mem_.reset(new DevBuf<T>(n));
+      adj_size_ = n;
+    }
+    adj_used_ = 0;
   }
-  void release_all() { adj_mem_.clear(); }
-  void tuckerT(const T* X, T* Y, bool fwd) { tucker(X, Y, fwd); }
+  T* alloc(size_t n) {
+    T* q = adj_mem_->ptr + adj_used_;
+    adj_used_ += padded(n);
+    return q;
+  }
+  // the adjoint's storage stays with the handle for the next gradient while it is small
+  void release_all() {
+    if (adj_size_ * sizeof(T) <= kAdjKeepBytes) return;
+    adj_mem_.reset();
+    adj_size_ = 0;
+  }
+  AdjSplit operand() { return AdjSplit{}; }
+  void tuckerT(const T* X, T* Y, bool fwd, bool) { tucker(X, Y, fwd); }
   void tuckerT_precise(const T* X, T* Y, bool fwd) { tucker(X, Y, fwd); }
   // U = bwd(Uh), K = fwd(g(t, U)); tmp: a work tensor of 2 P
-  void g_roundtrip(const T* Uh, T* U, T* K, T* tmp, double t) {
+  void g_roundtrip(const T* Uh, T* U, T* K, T* tmp, double t, bool) {
     tucker(Uh, U, false);
     gcombo<T>(s_, gp_, t, U, nullptr, nullptr, 1, 0, 0, 0, 1, 0, tmp, st_, launches);
     tucker(tmp, K, true);
@@ -332,9 +350,8 @@ class Engine : public EngineBase {
                void* grad_u0, double* grad_params, double* loss) override {
     if (scheme != FCGLE_LAWSON_RK2) throw Unsupported("the adjoint is implemented for LAWSON_RK2");
     try {
-      T* U0 = alloc(2 * s_.P);
-      T* TG = alloc(2 * s_.P);
-      T* GR = alloc(2 * s_.P);
+      // tensors of the schemes that no Tucker operator uses
+      T *U0 = B(kU), *TG = B(kUh), *GR = B(kG);
       pack<T>(s_, (const T*)u0, U0, st_, launches);
       pack<T>(s_, (const T*)target, TG, st_, launches);
       adjoint_lawson_rk2<T>(*this, tau, nsteps, t0, U0, TG, ckpt, GR, grad_params, loss);
@@ -738,7 +755,8 @@ class Engine : public EngineBase {
   Sliced xs_[kMaxDim][2];   // digits of the data as direction mu's product reads them (real, complex block form)
   std::unique_ptr<DevBuf<uint8_t>> xdig_;
   std::unique_ptr<DevBuf<int>> xex_;
-  std::vector<std::unique_ptr<DevBuf<T>>> adj_mem_;
+  std::unique_ptr<DevBuf<T>> adj_mem_;   // storage of the adjoint, adj_size_ elements
+  size_t adj_size_ = 0, adj_used_ = 0;
 };
 
 Direction spectral_direction(const fcgle_params& prm, int mu) {

@@ -685,25 +685,47 @@ class EngineB3 : public EngineBase {
     for (int mu = 0; mu < kMaxDim; ++mu) lv.lam[mu] = mu < s_.d ? lamd_[mu]->ptr : nullptr;
     return lv;
   }
-  float* alloc(size_t n) {
-    adj_mem_.emplace_back(new DevMem<float>(n));
-    return adj_mem_.back()->ptr;
+  static constexpr bool kSplit = true;
+  static size_t padded(size_t n) { return (n + 63) / 64 * 64; }
+  void reserve(size_t n) {
+    if (adj_size_ < n) {
+      adj_mem_.reset();
+      adj_size_ = 0;
+      adj_mem_.reset(new DevMem<float>(n));
+      adj_size_ = n;
+    }
+    adj_used_ = 0;
   }
-  void release_all() { adj_mem_.clear(); }
-  void tuckerT(const float* X, float* Y, bool fwd) {
+  float* alloc(size_t n) {
+    float* q = adj_mem_->ptr + adj_used_;
+    adj_used_ += padded(n);
+    return q;
+  }
+  // the adjoint's storage stays with the handle for the next gradient while it is small
+  void release_all() {
+    if (adj_size_ * sizeof(float) <= kAdjKeepBytes) return;
+    adj_mem_.reset();
+    adj_size_ = 0;
+  }
+  AdjSplit operand() { return AdjSplit{SP(kV).hi, SP(kV).lo}; }
+  void tuckerT(const float* X, float* Y, bool fwd, bool ready) {
     SplitOut V = SP(kV);
-    to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), X, V);
-    FCGLE_LAUNCHED(launches);
+    if (!ready) {
+      to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), X, V);
+      FCGLE_LAUNCHED(launches);
+    }
     tucker(V, fwd, b3::EpiStoreF32{P32(), Y});
   }
   void tuckerT_precise(const float* X, float* Y, bool fwd) { tucker_f32(X, Y, fwd, false); }
   // U = bwd(Uh) (FP32) and K = fwd(g(t, U)): g is evaluated in the epilogue of
   // the backward operator, which also writes it split for the forward one
   // (no standalone g pass, no split pass); tmp is not needed here
-  void g_roundtrip(const float* Uh, float* U, float* K, float*, double t) {
+  void g_roundtrip(const float* Uh, float* U, float* K, float*, double t, bool ready) {
     SplitOut V = SP(kV), G = SP(kW);
-    to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), Uh, V);
-    FCGLE_LAUNCHED(launches);
+    if (!ready) {
+      to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), Uh, V);
+      FCGLE_LAUNCHED(launches);
+    }
     tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t), 0.f, 1.f, G});
     tucker(G, true, b3::EpiStoreF32{P32(), K});
   }
@@ -712,9 +734,8 @@ class EngineB3 : public EngineBase {
                void* grad_u0, double* grad_params, double* loss) override {
     if (scheme != FCGLE_LAWSON_RK2) throw Unsupported("the adjoint is implemented for LAWSON_RK2");
     try {
-      float* U0 = alloc(2 * s_.P);
-      float* TG = alloc(2 * s_.P);
-      float* GR = alloc(2 * s_.P);
+      // tensors of the schemes that no Tucker operator uses
+      float *U0 = F32(kUh), *TG = F32(kUp), *GR = F32(kWork);
       pack_f32((const float*)u0, U0);
       pack_f32((const float*)target, TG);
       adjoint_lawson_rk2<float>(*this, tau, nsteps, t0, U0, TG, ckpt, GR, grad_params, loss);
@@ -1654,7 +1675,8 @@ class EngineB3 : public EngineBase {
   Mat mat_[kMaxDim][2];
   std::unique_ptr<DevMem<float>> lamf_[kMaxDim];
   std::unique_ptr<DevMem<double>> lamd_[kMaxDim];
-  std::vector<std::unique_ptr<DevMem<float>>> adj_mem_;
+  std::unique_ptr<DevMem<float>> adj_mem_;   // storage of the adjoint, adj_size_ floats
+  size_t adj_size_ = 0, adj_used_ = 0;
   b3::LamF lf_{};
   b3::GStatic gs_{};
   double sig_re_[kMaxSrc] = {0, 0, 0, 0}, sig_im_[kMaxSrc] = {0, 0, 0, 0};
