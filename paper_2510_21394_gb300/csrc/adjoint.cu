@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 
 #include "adjoint.h"
+#include "pdl.cuh"
+#include "tma_host.h"
 
 namespace fcgle {
 
@@ -54,6 +56,7 @@ struct GP {
 template <typename T>
 __global__ void misfit_kernel(size_t P, const T* __restrict__ u, const T* __restrict__ tg, T* __restrict__ lam,
                               double* acc) {
+  pdl_enter();
   double v[1] = {0.0};
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     const double dr = (double)u[q] - (double)tg[q], di = (double)u[P + q] - (double)tg[P + q];
@@ -86,6 +89,7 @@ __device__ __forceinline__ void gpar(double zr, double zi, double wr, double wi,
 template <typename T>
 __global__ void gv_kernel(size_t P, GP g, const T* __restrict__ z, const T* __restrict__ w, double c,
                           T* __restrict__ mu, double* acc) {
+  pdl_enter();
   double v[3] = {0.0, 0.0, 0.0};
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     const double zr = z[q], zi = z[P + q], wr = c * (double)w[q], wi = c * (double)w[P + q];
@@ -136,6 +140,7 @@ __device__ __forceinline__ bool lam_sum(const LD& L, size_t q, double& s) {
 
 template <typename T>
 __global__ void spec_dot_kernel(size_t P, LD L, const T* __restrict__ x, const T* __restrict__ y, double* acc) {
+  pdl_enter();
   double v[2] = {0.0, 0.0};
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     double s;
@@ -150,6 +155,7 @@ __global__ void spec_dot_kernel(size_t P, LD L, const T* __restrict__ x, const T
 template <typename T>
 __global__ void axpby_kernel(size_t n, double a, const T* __restrict__ x1, double b, const T* __restrict__ x2,
                              T* __restrict__ y) {
+  pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x)
     y[q] = (T)(a * (double)x1[q] + (x2 ? b * (double)x2[q] : 0.0));
 }
@@ -172,6 +178,7 @@ __device__ __forceinline__ void exp_z(const LD& L, size_t q, double cre, double 
 template <typename T>
 __global__ void exp_pair_kernel(size_t P, LD L, double cre, double cim, const T* __restrict__ x,
                                 const T* __restrict__ k, double c1, double c2, T* __restrict__ y1, T* __restrict__ y2) {
+  pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     double er, ei;
     exp_z(L, q, cre, cim, er, ei);
@@ -191,6 +198,7 @@ __global__ void exp_pair_kernel(size_t P, LD L, double cre, double cim, const T*
 template <typename T>
 __global__ void exp_combo_kernel(size_t P, LD L, double cre, double cim, const T* x, const T* __restrict__ m,
                                  double ca, double cb, T* y, T* __restrict__ sum) {
+  pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     double er, ei;
     exp_z(L, q, cre, cim, er, ei);
@@ -273,6 +281,7 @@ __device__ __forceinline__ void gadj_f(float gam, float kap, float zet, float zr
 
 __global__ void gv_kernel_f(uint32_t P, GP g, const float* __restrict__ z, const float* __restrict__ w, float c,
                             float* __restrict__ mu, AdjSplit sp, double* acc) {
+  pdl_enter();
   float f[3] = {0.f, 0.f, 0.f};
   const float gam = (float)g.gamma, kap = (float)g.kappa, zet = (float)g.zeta;
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
@@ -327,6 +336,7 @@ __device__ __forceinline__ void expm1_z_f(const Quad& Q, int v, float ar, float 
 __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const float* __restrict__ x,
                                   const float* __restrict__ k, float c1, float c2, float* __restrict__ y1,
                                   float* __restrict__ y2, AdjSplit sp) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     const Quad Q = quad_lam(L, q);
     float xr[4], xi[4], kr[4], ki[4], pr[4], pi[4], wr[4], wi[4];
@@ -359,6 +369,7 @@ __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const fl
 // a = e^z x, b = e^z m; y = ca a + cb b, sum = a + b (FP32 form of exp_combo_kernel; y may alias x)
 __global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const float* x, const float* __restrict__ m,
                                    float ca, float cb, float* y, float* __restrict__ sum, AdjSplit sp) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     const Quad Q = quad_lam(L, q);
     float xr[4], xi[4], nr[4], ni[4], yr[4], yi[4], sr[4], si[4];
@@ -390,6 +401,7 @@ __global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const f
 
 __global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* __restrict__ x, const float* __restrict__ y,
                                   double* acc) {
+  pdl_enter();
   float f[2] = {0.f, 0.f};
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     const Quad Q = quad_lam(L, q);
@@ -411,6 +423,7 @@ __global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* __restrict__ x,
 
 __global__ void axpby_kernel_f(uint32_t n, float a, const float* __restrict__ x1, float b,
                                const float* __restrict__ x2, float* __restrict__ y, AdjSplit sp) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float u[4], w[4] = {0.f, 0.f, 0.f, 0.f};
     ld4f(x1 + q, u);
@@ -437,17 +450,17 @@ LD make_ld(const Shape& s, const LamVecs& lv) {
 
 template <typename T>
 void adj_misfit(const Shape& s, const T* u, const T* target, T* lam, double* acc, cudaStream_t st, long long& nl) {
-  misfit_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, u, target, lam, acc);
+  launch_pdl(misfit_kernel<T>, grid_of(s.P), 256, 0, st, s.P, u, target, lam, acc);
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
 void adj_gv(const Shape& s, const GParams& gp, const T* z, const T* w, double c, T* mu, AdjSplit sp, double* acc,
             cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    gv_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, (float)c,
+    launch_pdl(gv_kernel_f, grid_of(s.P / 4), 256, 0, st, (uint32_t)s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, (float)c,
                                                    mu, sp, acc);
   else
-    gv_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, c, mu, acc);
+    launch_pdl(gv_kernel<T>, grid_of(s.P), 256, 0, st, s.P, GP{gp.gamma, gp.kappa, gp.zeta}, z, w, c, mu, acc);
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
@@ -460,19 +473,19 @@ template <typename T>
 void adj_spec_dot(const Shape& s, const LamVecs& lv, const T* x, const T* y, double* acc, cudaStream_t st,
                   long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    spec_dot_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, make_ld(s, lv), x, y, acc);
+    launch_pdl(spec_dot_kernel_f, grid_of(s.P / 4), 256, 0, st, (uint32_t)s.P, make_ld(s, lv), x, y, acc);
   else
-    spec_dot_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, make_ld(s, lv), x, y, acc);
+    launch_pdl(spec_dot_kernel<T>, grid_of(s.P), 256, 0, st, s.P, make_ld(s, lv), x, y, acc);
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
 void adj_axpby(const Shape& s, double a, const T* x1, double b, const T* x2, T* y, AdjSplit sp, cudaStream_t st,
                long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    axpby_kernel_f<<<grid_of(2 * s.P / 4), 256, 0, st>>>((uint32_t)(2 * s.P), (float)a, x1, (float)b, x2, y,
+    launch_pdl(axpby_kernel_f, grid_of(2 * s.P / 4), 256, 0, st, (uint32_t)(2 * s.P), (float)a, x1, (float)b, x2, y,
                                                          sp);
   else
-    axpby_kernel<T><<<grid_of(2 * s.P), 256, 0, st>>>(2 * s.P, a, x1, b, x2, y);
+    launch_pdl(axpby_kernel<T>, grid_of(2 * s.P), 256, 0, st, 2 * s.P, a, x1, b, x2, y);
   FCGLE_LAUNCHED(nl);
 }
 
@@ -480,11 +493,11 @@ template <typename T>
 void adj_exp_pair(const Shape& s, const LamVecs& lv, double theta, const T* x, const T* k, double c1, double c2,
                   T* y1, T* y2, AdjSplit sp1, cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    exp_pair_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
+    launch_pdl(exp_pair_kernel_f, grid_of(s.P / 4), 256, 0, st, (uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
                                                      (float)(theta * lv.c_im), x, k, (float)c1, (float)c2, y1, y2,
                                                      sp1);
   else
-    exp_pair_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, make_ld(s, lv), theta * lv.c_re, theta * lv.c_im, x, k,
+    launch_pdl(exp_pair_kernel<T>, grid_of(s.P), 256, 0, st, s.P, make_ld(s, lv), theta * lv.c_re, theta * lv.c_im, x, k,
                                                        c1, c2, y1, y2);
   FCGLE_LAUNCHED(nl);
 }
@@ -492,11 +505,11 @@ template <typename T>
 void adj_exp_h_combo(const Shape& s, const LamVecs& lv, double theta, const T* x, const T* m, double ca, double cb,
                      T* y, T* sum, AdjSplit spy, cudaStream_t st, long long& nl) {
   if constexpr (std::is_same<T, float>::value)
-    exp_combo_kernel_f<<<grid_of(s.P / 4), 256, 0, st>>>((uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
+    launch_pdl(exp_combo_kernel_f, grid_of(s.P / 4), 256, 0, st, (uint32_t)s.P, make_ld(s, lv), (float)(theta * lv.c_re),
                                                       (float)(-theta * lv.c_im), x, m, (float)ca, (float)cb, y, sum,
                                                       spy);
   else
-    exp_combo_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, make_ld(s, lv), theta * lv.c_re, -theta * lv.c_im, x, m,
+    launch_pdl(exp_combo_kernel<T>, grid_of(s.P), 256, 0, st, s.P, make_ld(s, lv), theta * lv.c_re, -theta * lv.c_im, x, m,
                                                         ca, cb, y, sum);
   FCGLE_LAUNCHED(nl);
 }

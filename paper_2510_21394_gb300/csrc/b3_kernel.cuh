@@ -36,6 +36,7 @@
 
 #include "b3_epilogues.cuh"
 #include "common.h"
+#include "pdl.cuh"
 
 namespace fcgle {
 namespace b3 {
@@ -132,16 +133,6 @@ struct KParams {
 constexpr uint32_t kNegA = 1u << 13;
 
 // -------------------------------------------------------------- PTX helpers
-// Programmatic dependent launch.  Every mode-product kernel lets the next
-// kernel of its stream be scheduled as soon as all of its own CTAs are running
-// (pdl_trigger at entry) and, after its prologue (mbarrier init, TMEM
-// allocation), waits until the previous kernel of the stream has completed and
-// its writes are visible (pdl_wait) before it touches global memory.  The
-// wait ends when that kernel ends; without the launch attribute both are
-// no-ops.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

@@ -393,7 +393,7 @@ class Engine : public EngineBase {
     void build(const double* M, int K, cudaStream_t st, long long& nl) {
       s.rows = s.K = K;
       dig.reset(new DevBuf<uint8_t>(slice_bytes<double>(K, K)));
-      ex.reset(new DevBuf<int>((size_t)K));
+      ex.reset(new DevBuf<int>(slice_exponents(K)));
       s.dig = reinterpret_cast<__nv_bfloat16*>(dig->ptr);
       s.ex = ex->ptr;
       slice_map<double>(s, true);
@@ -672,7 +672,7 @@ class Engine : public EngineBase {
 
   void krogstad_step(double tau, double t) {
     T *U = B(kU), *Uh = B(kUh), *G = B(kG), *Fh = B(kFh), *S = B(kS), *W = B(kW);
-    T *D2 = B(kD2), *D3 = B(kD3), *D4 = B(kD4), *Us = B(kGh);
+    T *D2 = B(kD2), *D3 = B(kD3), *D4 = B(kD4);
     T* P1h = F(FCGLE_F_PHI, 1, tau / 2);
     T* P2h = F(FCGLE_F_PHI, 2, tau / 2);
     T* P1 = F(FCGLE_F_PHI, 1, tau);
@@ -683,11 +683,10 @@ class Engine : public EngineBase {
     tucker(G, Fh, true);
     form_Fhat(Uh, Fh, Fh);
     auto stage = [&](const SpecArgs<T>& a, double tc, T* Dh) {
-      // S = combination; U_s = u_n + bwd(S); D^ = fwd(g(tc, U_s) - G)
+      // S = combination; D^ = fwd(g(tc, U_s) - G) with U_s = u_n + bwd(S), summed on the fly
       spec_combo<T>(s_, lv_, a, st_, launches);
       tucker(S, W, false);
-      add(U, W, Us);
-      gcombo<T>(s_, gp_, tc, Us, nullptr, G, 1, 0, 0, 0, 1, -1, Dh, st_, launches);
+      gcombo<T>(s_, gp_, tc, U, W, G, 1, 1, 0, 0, 1, -1, Dh, st_, launches);
       tucker(Dh, Dh, true);
     };
     {  // U_n2 = u_n + tau/2 phi_1(tau/2 K) f_n

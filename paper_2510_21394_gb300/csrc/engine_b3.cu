@@ -249,6 +249,7 @@ float tf32_rna_host(float x) {
 // V = a u + b g(t, u) (split); optionally V2 = a2 u + b2 g(t, u) (split)
 __global__ void gsplit_kernel(uint32_t P, b3::GStatic g, b3::GTime t, const float* __restrict__ U, float a, float b,
                               SplitOut V, float a2, float b2, SplitOut V2) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float ur[4], ui[4], gr[4] = {0, 0, 0, 0}, gi[4] = {0, 0, 0, 0}, xr[4], xi[4];
     b3::ldv<4>(U + q, ur);
@@ -274,6 +275,7 @@ __global__ void gsplit_kernel(uint32_t P, b3::GStatic g, b3::GTime t, const floa
 // V = Phi_t(u) (split)
 // U = Phi_t(W)
 __global__ void flow_kernel(uint32_t P, b3::Flow f, const float* __restrict__ W, float* __restrict__ U) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float wr[4], wi[4], ur[4], ui[4];
     b3::ldv<4>(W + q, wr);
@@ -287,6 +289,7 @@ __global__ void flow_kernel(uint32_t P, b3::Flow f, const float* __restrict__ W,
 
 // V = Phi_t(u) -> split (Strang's first half step, Kronecker-product form)
 __global__ void flow_split_kernel(uint32_t P, b3::Flow f, const float* __restrict__ U, SplitOut V) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float ur[4], ui[4], vr[4], vi[4];
     b3::ldv<4>(U + q, ur);
@@ -299,6 +302,7 @@ __global__ void flow_split_kernel(uint32_t P, b3::Flow f, const float* __restric
 
 // V = Phi_t(u) - u -> split (Strang's first half step as an increment)
 __global__ void flow_incr_split_kernel(uint32_t P, b3::Flow f, const float* __restrict__ U, SplitOut V) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float ur[4], ui[4], vr[4], vi[4];
     b3::ldv<4>(U + q, ur);
@@ -312,6 +316,7 @@ __global__ void flow_incr_split_kernel(uint32_t P, b3::Flow f, const float* __re
 // FP32 -> split-TF32: hi = tf32(x), lo = tf32(x - hi); n % 4 == 0
 __global__ void tf32_split_kernel(uint32_t n, const float* __restrict__ X, float* __restrict__ hi,
                                   float* __restrict__ lo) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float x[4], h[4], l[4];
     b3::ldv<4>(X + q, x);
@@ -327,6 +332,7 @@ __global__ void tf32_split_kernel(uint32_t n, const float* __restrict__ X, float
 
 // FP32 -> split (raw mode-product entry point); n % 4 == 0
 __global__ void to_split_kernel(uint32_t n, const float* __restrict__ X, SplitOut Y) {
+  pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float x[4];
     b3::ldv<4>(X + q, x);
@@ -435,7 +441,7 @@ class EngineB3 : public EngineBase {
           Mat& m = mat_[mu][f];
           m.sl.rows = m.sl.K = m.p;
           FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<float>(m.p, m.p)));
-          FCGLE_CUDA(cudaMalloc(&m.sl.ex, m.p * sizeof(int)));
+          FCGLE_CUDA(cudaMalloc(&m.sl.ex, slice_exponents(m.p) * sizeof(int)));
           slice_map<float>(m.sl, true);
           slice_rows<float>(m.f32, m.sl, 1, m.p, 0, st_, launches);
         }
@@ -580,7 +586,7 @@ class EngineB3 : public EngineBase {
       const long long R = P_ / s_.p[mu];
       if (s_.d >= 2 && R % 8 == 0 && s_.p[mu] <= kTf32MaxP) {
         float *ah = F32(kFh), *al = F32(kD2);   // work tensors of the schemes, free here
-        tf32_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), (const float*)X, ah, al);
+        launch_pdl(tf32_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), (const float*)X, ah, al);
         FCGLE_LAUNCHED(launches);
         launch_tf32(ah, al, mu, fwd, (float*)Y, nullptr);
       } else {
@@ -613,7 +619,7 @@ class EngineB3 : public EngineBase {
       store_split(xh, xh + 2 * s_.P, mu, fwd, out);
     } else {
       SplitOut t = SP(kT0);
-      to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), (const float*)X, t);
+      launch_pdl(to_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), (const float*)X, t);
       FCGLE_LAUNCHED(launches);
       launch_mp(t.hi, t.lo, mu, fwd, b3::EpiStoreF32{P32(), (float*)Y});
     }
@@ -711,7 +717,7 @@ class EngineB3 : public EngineBase {
   void tuckerT(const float* X, float* Y, bool fwd, bool ready) {
     SplitOut V = SP(kV);
     if (!ready) {
-      to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), X, V);
+      launch_pdl(to_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), X, V);
       FCGLE_LAUNCHED(launches);
     }
     tucker(V, fwd, b3::EpiStoreF32{P32(), Y});
@@ -723,7 +729,7 @@ class EngineB3 : public EngineBase {
   void g_roundtrip(const float* Uh, float* U, float* K, float*, double t, bool ready) {
     SplitOut V = SP(kV), G = SP(kW);
     if (!ready) {
-      to_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), Uh, V);
+      launch_pdl(to_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), Uh, V);
       FCGLE_LAUNCHED(launches);
     }
     tucker(V, false, b3::EpiUpdateG{P32(), U, gs_, gtime(t), 0.f, 1.f, G});
@@ -1004,7 +1010,7 @@ class EngineB3 : public EngineBase {
   void tucker_tf32(const float* X, float* Y, bool fwd) {
     float* const hi[2] = {F32(kFh), F32(kD3)};
     float* const lo[2] = {F32(kD2), F32(kEA)};
-    tf32_split_kernel<<<grid_for(P_ / 2), 256, 0, st_>>>(2 * P32(), X, hi[0], lo[0]);
+    launch_pdl(tf32_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), X, hi[0], lo[0]);
     FCGLE_LAUNCHED(launches);
     int cur = 0;
     for (int mu = 0; mu < s_.d; ++mu) {
@@ -1444,7 +1450,7 @@ class EngineB3 : public EngineBase {
   // V = a u + b g(t, u) (+ optional V2)
   void gsplit(const float* U, double t, float a, float b, SplitOut V, float a2 = 0.f, float b2 = 0.f,
               SplitOut V2 = SplitOut{}) {
-    gsplit_kernel<<<grid_for(P_ / 4), 256, 0, st_>>>(P32(), gs_, gtime(t), U, a, b, V, a2, b2, V2);
+    launch_pdl(gsplit_kernel, grid_for(P_ / 4), 256, 0, st_, P32(), gs_, gtime(t), U, a, b, V, a2, b2, V2);
     FCGLE_LAUNCHED(launches);
   }
 
@@ -1503,7 +1509,7 @@ class EngineB3 : public EngineBase {
     if (rs_scheme_ == FCGLE_STRANG) {
       float* W = F32(kWork);
       tucker_f32(F32(kUh), W, false);
-      flow_kernel<<<grid_for(P_ / 4), 256, 0, st_>>>(P32(), flow(rs_tau_ / 2), W, F32(kU));
+      launch_pdl(flow_kernel, grid_for(P_ / 4), 256, 0, st_, P32(), flow(rs_tau_ / 2), W, F32(kU));
       FCGLE_LAUNCHED(launches);
     } else {
       tucker_f32(F32(kUh), F32(kU), false);
@@ -1522,7 +1528,7 @@ class EngineB3 : public EngineBase {
       // Kronecker-product form: the state is the physical u; V (and W) = the
       // input of the first e^{tau K} of step 0
       if (scheme == FCGLE_STRANG) {
-        flow_split_kernel<<<grid_for(P_ / 4), 256, 0, st_>>>(P32(), flow(tau / 2), U, V);
+        launch_pdl(flow_split_kernel, grid_for(P_ / 4), 256, 0, st_, P32(), flow(tau / 2), U, V);
         FCGLE_LAUNCHED(launches);
       } else if (scheme == FCGLE_LAWSON_EULER) {
         gsplit(U, t0, 1.f, ft, V);
@@ -1535,7 +1541,7 @@ class EngineB3 : public EngineBase {
       case FCGLE_STRANG:
         // e^_0 = fwd(u_0) (FP32); V = Phi_{tau/2}(u_0) - u_0
         tucker_f32(U, F32(kUh), true);
-        flow_incr_split_kernel<<<grid_for(P_ / 4), 256, 0, st_>>>(P32(), flow(tau / 2), U, V);
+        launch_pdl(flow_incr_split_kernel, grid_for(P_ / 4), 256, 0, st_, P32(), flow(tau / 2), U, V);
         FCGLE_LAUNCHED(launches);
         break;
       case FCGLE_LIE:

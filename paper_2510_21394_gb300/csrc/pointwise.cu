@@ -7,8 +7,11 @@
 // Grid-stride loops; each thread handles 4 consecutive elements so that
 // every global access is a 16-byte (float) or 32-byte (double) vector.
 #include <cmath>
+#include <stdexcept>
 
 #include "common.h"
+#include "pdl.cuh"
+#include "tma_host.h"
 
 namespace fcgle {
 
@@ -82,6 +85,7 @@ __device__ __forceinline__ RowMap row_map(const Shape& s, size_t rho) {
 
 template <typename T>
 __global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__ X) {
+  pdl_enter();
   const size_t P = s.P, quads_per_row = (size_t)s.p[0] / 4, nq = P / 4;
   const int n1 = s.n[0];
   for (size_t q4 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q4 < nq; q4 += (size_t)gridDim.x * blockDim.x) {
@@ -120,6 +124,7 @@ __global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__
 
 template <typename T>
 __global__ void unpack_kernel(Shape s, const T* __restrict__ X, T* __restrict__ user, int* __restrict__ nonfinite) {
+  pdl_enter();
   const size_t P = s.P, quads_per_row = (size_t)s.p[0] / 4, nq = P / 4;
   const int n1 = s.n[0];
   bool bad = false;
@@ -164,45 +169,81 @@ struct GDev {
   const void* S[kMaxSrc];
 };
 
-template <typename T>
+// FP64 arithmetic bound (two FMAs per clock and SM): every term that a call does
+// not have is left out at compile time.  128 x 120 x 136: g(u) alone 102 -> 45 us.
+enum { GC_X1 = 1, GC_UNIT = 2, GC_A = 4, GC_B = 8, GC_X2 = 16 };   // X1; c0 = c1 = 1; a0, a1 terms; b != 1; X2
+template <typename T, int F>
 __global__ void gcombo_kernel(size_t P, GDev g, const T* __restrict__ X0, const T* __restrict__ X1,
                               const T* __restrict__ X2, double c0, double c1, double a0, double a1, double b,
                               double e, T* __restrict__ out) {
+  pdl_enter();
   const size_t nv = P / 4;
   for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nv; v += (size_t)gridDim.x * blockDim.x) {
     const size_t q = v * 4;
-    T x0r[4], x0i[4], x1r[4] = {0, 0, 0, 0}, x1i[4] = {0, 0, 0, 0}, x2r[4] = {0, 0, 0, 0}, x2i[4] = {0, 0, 0, 0};
+    T x0r[4], x0i[4], x1r[4], x1i[4], x2r[4], x2i[4];
     ld4(X0 + q, x0r);
     ld4(X0 + P + q, x0i);
-    if (X1) { ld4(X1 + q, x1r); ld4(X1 + P + q, x1i); }
-    if (X2) { ld4(X2 + q, x2r); ld4(X2 + P + q, x2i); }
-    T src_r[4] = {0, 0, 0, 0}, src_i[4] = {0, 0, 0, 0};
-    for (int k = 0; k < g.nsrc; ++k) {
-      const T* S = reinterpret_cast<const T*>(g.S[k]);
-      T sr[4], si[4];
-      ld4(S + q, sr);
-      ld4(S + P + q, si);
-      const T er = (T)g.e_re[k], ei = (T)g.e_im[k];
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        src_r[l] += er * sr[l] - ei * si[l];
-        src_i[l] += er * si[l] + ei * sr[l];
-      }
-    }
+    if constexpr (F & GC_X1) { ld4(X1 + q, x1r); ld4(X1 + P + q, x1i); }
+    if constexpr (F & GC_X2) { ld4(X2 + q, x2r); ld4(X2 + P + q, x2i); }
     T o_r[4], o_i[4];
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
-      const T ur = (T)c0 * x0r[l] + (T)c1 * x1r[l];
-      const T ui = (T)c0 * x0i[l] + (T)c1 * x1i[l];
+      T ur = x0r[l], ui = x0i[l];
+      if constexpr (F & GC_UNIT) {
+        if constexpr (F & GC_X1) { ur += x1r[l]; ui += x1i[l]; }
+      } else if constexpr (F & GC_X1) {
+        ur = (T)c0 * x0r[l] + (T)c1 * x1r[l];
+        ui = (T)c0 * x0i[l] + (T)c1 * x1i[l];
+      } else {
+        ur *= (T)c0;
+        ui *= (T)c0;
+      }
       const T m2 = ur * ur + ui * ui;
-      // gamma u - (kappa + i zeta) |u|^2 u + s
-      const T gr = (T)g.gamma * ur - m2 * ((T)g.kappa * ur - (T)g.zeta * ui) + src_r[l];
-      const T gi = (T)g.gamma * ui - m2 * ((T)g.kappa * ui + (T)g.zeta * ur) + src_i[l];
-      o_r[l] = (T)a0 * x0r[l] + (T)a1 * x1r[l] + (T)b * gr + (T)e * x2r[l];
-      o_i[l] = (T)a0 * x0i[l] + (T)a1 * x1i[l] + (T)b * gi + (T)e * x2i[l];
+      // gamma u - (kappa + i zeta) |u|^2 u
+      o_r[l] = (T)g.gamma * ur - m2 * ((T)g.kappa * ur - (T)g.zeta * ui);
+      o_i[l] = (T)g.gamma * ui - m2 * ((T)g.kappa * ui + (T)g.zeta * ur);
+    }
+    if (g.nsrc > 0) {
+      T src_r[4] = {0, 0, 0, 0}, src_i[4] = {0, 0, 0, 0};
+      for (int k = 0; k < g.nsrc; ++k) {
+        const T* S = reinterpret_cast<const T*>(g.S[k]);
+        T sr[4], si[4];
+        ld4(S + q, sr);
+        ld4(S + P + q, si);
+        const T er = (T)g.e_re[k], ei = (T)g.e_im[k];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          src_r[l] += er * sr[l] - ei * si[l];
+          src_i[l] += er * si[l] + ei * sr[l];
+        }
+      }
+#pragma unroll
+      for (int l = 0; l < 4; ++l) { o_r[l] += src_r[l]; o_i[l] += src_i[l]; }
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      if constexpr (F & GC_B) { o_r[l] *= (T)b; o_i[l] *= (T)b; }
+      if constexpr (F & GC_A) {
+        T ar = (T)a0 * x0r[l], ai = (T)a0 * x0i[l];
+        if constexpr (F & GC_X1) { ar += (T)a1 * x1r[l]; ai += (T)a1 * x1i[l]; }
+        o_r[l] += ar;
+        o_i[l] += ai;
+      }
+      if constexpr (F & GC_X2) { o_r[l] += (T)e * x2r[l]; o_i[l] += (T)e * x2i[l]; }
     }
     st4(out + q, o_r);
     st4(out + P + q, o_i);
+  }
+}
+
+template <typename T, int F>
+void gcombo_dispatch(int f, size_t P, const GDev& g, const T* X0, const T* X1, const T* X2, double c0, double c1,
+                     double a0, double a1, double b, double e, T* out, cudaStream_t st) {
+  if constexpr (F < 32) {
+    if (f == F)
+      launch_pdl(gcombo_kernel<T, F>, grid_for(P / 4, 256), 256, 0, st, P, g, X0, X1, X2, c0, c1, a0, a1, b, e, out);
+    else
+      gcombo_dispatch<T, F + 1>(f, P, g, X0, X1, X2, c0, c1, a0, a1, b, e, out, st);
   }
 }
 
@@ -214,80 +255,103 @@ struct LamDev {
   double c_re, c_im;
 };
 
-__device__ __forceinline__ void lam_at(const LamDev& L, size_t q, double& re, double& im) {
-  double s = 0.0;
-  size_t rem = q;
-  for (int mu = 0; mu < L.d; ++mu) {
-    int j = (int)(rem % L.p[mu]);
-    rem /= L.p[mu];
-    s += L.lam[mu][j];
+// eigenvalues of K at the 4 elements q .. q + 3 of one row of direction 1
+__device__ __forceinline__ void lam_quad(const LamDev& L, size_t q, double (&re)[4], double (&im)[4]) {
+  size_t rem = q / (size_t)L.p[0];
+  const int j1 = (int)(q - rem * (size_t)L.p[0]);
+  double l2 = 0.0, l3 = 0.0;
+  if (L.d == 3) {
+    const size_t j3 = rem / (size_t)L.p[1];
+    l2 = L.lam[1][rem - j3 * (size_t)L.p[1]];
+    l3 = L.lam[2][j3];
+  } else if (L.d == 2) {
+    l2 = L.lam[1][rem];
   }
-  re = L.c_re * s;
-  im = L.c_im * s;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const double s = (L.lam[0][j1 + l] + l2) + l3;
+    re[l] = L.c_re * s;
+    im[l] = L.c_im * s;
+  }
 }
 
 template <typename T>
 struct SpecDev {
-  int nx, nf;
   const T* X[4];
   const T* F[4];
   int fkind[4];
   double W[4][4];
+  int nz[4], one[4];   // bit x: W[f][x] != 0, W[f][x] == 1
   T* out;
   const T* base;
   T* out2;
 };
 
-template <typename T>
+// FP64 arithmetic bound, like gcombo_kernel: the numbers of operands and factors
+// are known at compile time, absent weights cost nothing and weights of one no
+// product.
+template <typename T, int NX, int NF>
 __global__ void spec_kernel(size_t P, LamDev L, SpecDev<T> a) {
+  pdl_enter();
   const size_t nv = P / 4;
   for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nv; v += (size_t)gridDim.x * blockDim.x) {
     const size_t q = v * 4;
-    T xr[4][4], xi[4][4];
+    T xr[NX][4], xi[NX][4];
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      if (x < a.nx) {
-        ld4(a.X[x] + q, xr[x]);
-        ld4(a.X[x] + P + q, xi[x]);
-      }
+    for (int x = 0; x < NX; ++x) {
+      ld4(a.X[x] + q, xr[x]);
+      ld4(a.X[x] + P + q, xi[x]);
     }
-    T o_r[4] = {0, 0, 0, 0}, o_i[4] = {0, 0, 0, 0};
+    T o_r[4], o_i[4];
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      if (f >= a.nf) break;
+    for (int f = 0; f < NF; ++f) {
       T sr[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0};
+      bool any = false;
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        if (x < a.nx && a.W[f][x] != 0.0) {
-          const T w = (T)a.W[f][x];
+      for (int x = 0; x < NX; ++x) {
+        if (!(a.nz[f] >> x & 1)) continue;
+        const bool one = a.one[f] >> x & 1;
+        const T w = (T)a.W[f][x];
 #pragma unroll
-          for (int l = 0; l < 4; ++l) {
+        for (int l = 0; l < 4; ++l) {
+          if (!any) {
+            sr[l] = one ? xr[x][l] : w * xr[x][l];
+            si[l] = one ? xi[x][l] : w * xi[x][l];
+          } else if (one) {
+            sr[l] += xr[x][l];
+            si[l] += xi[x][l];
+          } else {
             sr[l] += w * xr[x][l];
             si[l] += w * xi[x][l];
           }
         }
+        any = true;
       }
       if (a.fkind[f] == F_ONE) {
 #pragma unroll
-        for (int l = 0; l < 4; ++l) { o_r[l] += sr[l]; o_i[l] += si[l]; }
+        for (int l = 0; l < 4; ++l) {
+          o_r[l] = f == 0 ? sr[l] : o_r[l] + sr[l];
+          o_i[l] = f == 0 ? si[l] : o_i[l] + si[l];
+        }
       } else {
         T fr[4], fi[4];
         if (a.fkind[f] == F_TENSOR) {
           ld4(a.F[f] + q, fr);
           ld4(a.F[f] + P + q, fi);
         } else {
+          double lr[4], li[4];
+          lam_quad(L, q, lr, li);
 #pragma unroll
           for (int l = 0; l < 4; ++l) {
-            double lr, li;
-            lam_at(L, q + l, lr, li);
-            fr[l] = (T)lr;
-            fi[l] = (T)li;
+            fr[l] = (T)lr[l];
+            fi[l] = (T)li[l];
           }
         }
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-          o_r[l] += fr[l] * sr[l] - fi[l] * si[l];
-          o_i[l] += fr[l] * si[l] + fi[l] * sr[l];
+          const T yr = fr[l] * sr[l] - fi[l] * si[l], yi = fr[l] * si[l] + fi[l] * sr[l];
+          o_r[l] = f == 0 ? yr : o_r[l] + yr;
+          o_i[l] = f == 0 ? yi : o_i[l] + yi;
         }
       }
     }
@@ -396,6 +460,7 @@ __global__ void fill_F_kernel(size_t P, LamDev L, Shape s, int func, int ell, do
 template <typename T>
 __global__ void exact_flow_kernel(size_t P, double gamma, double kappa, double zeta, double t, double tp1,
                                   const T* __restrict__ X, T* __restrict__ Y) {
+  pdl_enter();
   // w(t) = exp(t gamma - (kappa + i zeta)/(2 kappa) log(1 + 2 t phi_1(2 gamma t) kappa |w0|^2)) w0
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     const double wr = X[q], wi = X[P + q];
@@ -446,12 +511,12 @@ LamDev lamdev(const Shape& s, const LamVecs& lv) {
 // ===================================================================== host
 template <typename T>
 void pack(const Shape& s, const T* user, T* X, cudaStream_t st, long long& nl) {
-  pack_kernel<T><<<grid_for(s.P / 4, 256), 256, 0, st>>>(s, user, X);
+  launch_pdl(pack_kernel<T>, grid_for(s.P / 4, 256), 256, 0, st, s, user, X);
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
 void unpack(const Shape& s, const T* X, T* user, cudaStream_t st, long long& nl, int* nonfinite) {
-  unpack_kernel<T><<<grid_for(s.P / 4, 256), 256, 0, st>>>(s, X, user, nonfinite);
+  launch_pdl(unpack_kernel<T>, grid_for(s.P / 4, 256), 256, 0, st, s, X, user, nonfinite);
   FCGLE_LAUNCHED(nl);
 }
 
@@ -473,25 +538,41 @@ void gcombo(const Shape& s, const GParams& gp, double t, const T* X0, const T* X
       g.e_re[k] = g.e_im[k] = 0.0;
     }
   }
-  gcombo_kernel<T><<<grid_for(s.P / 4, 256), 256, 0, st>>>(s.P, g, X0, X1, X2, c0, c1, a0, a1, b, e, out);
+  const int f = (X1 ? GC_X1 : 0) | (c0 == 1.0 && (!X1 || c1 == 1.0) ? GC_UNIT : 0) |
+                (a0 != 0.0 || (X1 && a1 != 0.0) ? GC_A : 0) | (b != 1.0 ? GC_B : 0) | (X2 && e != 0.0 ? GC_X2 : 0);
+  gcombo_dispatch<T, 0>(f, s.P, g, X0, X1, X2, c0, c1, a0, a1, b, e, out, st);
   FCGLE_LAUNCHED(nl);
 }
 
 template <typename T>
 void spec_combo(const Shape& s, const LamVecs& lv, const SpecArgs<T>& a, cudaStream_t st, long long& nl) {
   SpecDev<T> d;
-  d.nx = a.nx;
-  d.nf = a.nf;
   for (int i = 0; i < 4; ++i) {
     d.X[i] = a.X[i];
     d.F[i] = a.F[i];
     d.fkind[i] = a.fkind[i];
-    for (int j = 0; j < 4; ++j) d.W[i][j] = a.W[i][j];
+    d.nz[i] = d.one[i] = 0;
+    for (int j = 0; j < 4; ++j) {
+      d.W[i][j] = a.W[i][j];
+      if (a.W[i][j] != 0.0) d.nz[i] |= 1 << j;
+      if (a.W[i][j] == 1.0) d.one[i] |= 1 << j;
+    }
   }
   d.out = a.out;
   d.base = a.base;
   d.out2 = a.out2;
-  spec_kernel<T><<<grid_for(s.P / 4, 256), 256, 0, st>>>(s.P, lamdev(s, lv), d);
+  const int grid = grid_for(s.P / 4, 256);
+  const LamDev L = lamdev(s, lv);
+  if (a.nx == 1 && a.nf == 1)
+    launch_pdl(spec_kernel<T, 1, 1>, grid, 256, 0, st, s.P, L, d);
+  else if (a.nx == 2 && a.nf == 1)
+    launch_pdl(spec_kernel<T, 2, 1>, grid, 256, 0, st, s.P, L, d);
+  else if (a.nx == 2 && a.nf == 2)
+    launch_pdl(spec_kernel<T, 2, 2>, grid, 256, 0, st, s.P, L, d);
+  else if (a.nx == 4 && a.nf == 3)
+    launch_pdl(spec_kernel<T, 4, 3>, grid, 256, 0, st, s.P, L, d);
+  else
+    throw std::logic_error("spectral combination without a kernel");
   FCGLE_LAUNCHED(nl);
 }
 
@@ -514,7 +595,7 @@ void exact_flow(const Shape& s, double gamma, double kappa, double zeta, double 
   // t phi_1(2 gamma t), in FP64 on the host
   const double z = 2.0 * gamma * t;
   const double p1 = std::fabs(z) < 1e-8 ? 1.0 + z / 2.0 : std::expm1(z) / z;
-  exact_flow_kernel<T><<<grid_for(s.P, 256), 256, 0, st>>>(s.P, gamma, kappa, zeta, t, p1, X, Y);
+  launch_pdl(exact_flow_kernel<T>, grid_for(s.P, 256), 256, 0, st, s.P, gamma, kappa, zeta, t, p1, X, Y);
   FCGLE_LAUNCHED(nl);
 }
 
@@ -527,16 +608,17 @@ void sumsq(const Shape& s, const T* X, double* out_dev, cudaStream_t st, long lo
 
 #define INST(T)                                                                                           \
   template void pack<T>(const Shape&, const T*, T*, cudaStream_t, long long&);                           \
-  template void unpack<T>(const Shape&, const T*, T*, cudaStream_t, long long&, int*);                         \
-  template void gcombo<T>(const Shape&, const GParams&, double, const T*, const T*, const T*, double,     \
-                          double, double, double, double, double, T*, cudaStream_t, long long&);         \
-  template void spec_combo<T>(const Shape&, const LamVecs&, const SpecArgs<T>&, cudaStream_t, long long&); \
-  template void fill_F<T>(const Shape&, const LamVecs&, int, int, double, T*, cudaStream_t, long long&);  \
-  template void exact_flow<T>(const Shape&, double, double, double, double, const T*, T*, cudaStream_t,   \
-                              long long&);                                                               \
+  template void unpack<T>(const Shape&, const T*, T*, cudaStream_t, long long&, int*);                   \
   template void sumsq<T>(const Shape&, const T*, double*, cudaStream_t, long long&);
 INST(float)
 INST(double)
 #undef INST
+// the FP64 engine's
+template void gcombo<double>(const Shape&, const GParams&, double, const double*, const double*, const double*, double,
+                             double, double, double, double, double, double*, cudaStream_t, long long&);
+template void spec_combo<double>(const Shape&, const LamVecs&, const SpecArgs<double>&, cudaStream_t, long long&);
+template void fill_F<double>(const Shape&, const LamVecs&, int, int, double, double*, cudaStream_t, long long&);
+template void exact_flow<double>(const Shape&, double, double, double, double, const double*, double*, cudaStream_t,
+                                 long long&);
 
 }  // namespace fcgle

@@ -69,13 +69,41 @@ __device__ __forceinline__ void load4(const T* p, typename Bits<T>::U (&u)[4]) {
   }
 }
 
+// The digits of one element as a balanced number: half a digit added at every
+// place but the top one, so that place a is (w >> RB (NS - 1 - a)) mod 2^RB - 2^{RB - 1}.
+template <typename T>
+struct Balanced;
+template <>
+struct Balanced<double> {
+  using W = long long;
+};
+template <>
+struct Balanced<float> {
+  using W = int;
+};
+template <typename T>
+__device__ __forceinline__ typename Balanced<T>::W balanced(typename Bits<T>::U u, int emax, bool bad) {
+  using U = typename Bits<T>::U;
+  using W = typename Balanced<T>::W;
+  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
+  const int e = (int)((u >> MB) & Bits<T>::kExpMask);
+  const U mant = ((u & ((U(1) << MB) - 1)) | (e ? U(1) << MB : U(0))) << UP;
+  const int s = emax - max(e, 1);
+  const U m = s < (int)(8 * sizeof(U)) - 2 ? (mant + ((U(1) << s) >> 1)) >> s : U(0);
+  W x = (u >> (8 * sizeof(U) - 1)) ? -(W)m : (W)m;
+  if (bad) x = 0;
+  W off = 0;
+#pragma unroll
+  for (int j = 0; j + 1 < NS; ++j) off += W(1) << (RB * j + RB - 1);
+  return x + off;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
                                                     long long seg_stride, int pitch, int group,
                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex) {
   using U = typename Bits<T>::U;
   constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant;
-  constexpr U kMantMask = (U(1) << MB) - 1;
   constexpr int UP = SliceCfg<T>::BITS - MB - 2;   // spare bits below the last one of the largest entry
   pdl_trigger();
   pdl_wait();
@@ -107,21 +135,9 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
       for (int q = lig; q < quads; q += group) {
         U u[4];
         load4<T>(src + 4 * q, u);
-        long long w[4];
+        typename Balanced<T>::W w[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int e = (int)((u[v] >> MB) & Bits<T>::kExpMask);
-          const unsigned long long mant = ((unsigned long long)(u[v] & kMantMask) | (e ? 1ull << MB : 0ull)) << UP;
-          const int s = emax - max(e, 1);
-          const unsigned long long m = s < 62 ? (mant + ((1ull << s) >> 1)) >> s : 0ull;
-          long long x = (u[v] >> (8 * sizeof(U) - 1)) ? -(long long)m : (long long)m;
-          if (bad) x = 0;
-          // balanced digits: add half a digit at every place but the top one
-          long long off = 0;
-#pragma unroll
-          for (int j = 0; j + 1 < NS; ++j) off += 1ll << (RB * j + RB - 1);
-          w[v] = x + off;
-        }
+        for (int v = 0; v < 4; ++v) w[v] = balanced<T>(u[v], emax, bad);
 #pragma unroll
         for (int a = 0; a < NS; ++a) {
           uint32_t h[4];
@@ -142,17 +158,91 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
   }
 }
 
+// The same pass for rows of up to 8 x 32 x IT elements in segments of a multiple
+// of 8: a lane keeps its 8-element pieces in registers between the two halves
+// and stores 16 bytes per digit (FP32 at 432^3: 473 us with 4-element pieces read
+// twice, 303 this way = 5.3 TB/s; FP64 at 128 x 120 x 136: 25 -> 20 us).
+template <typename T, int IT>
+__global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
+                                                     long long seg_stride, int pitch, int group,
+                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex) {
+  using U = typename Bits<T>::U;
+  using W = typename Balanced<T>::W;
+  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
+  pdl_trigger();
+  pdl_wait();
+  const int per_block = 256 / group, lig = threadIdx.x % group;
+  const int cps = seg_len / 8, chunks = nseg * cps;
+  for (long long row0 = (long long)blockIdx.x * per_block; row0 < rows; row0 += (long long)gridDim.x * per_block) {
+    const long long row = row0 + threadIdx.x / group;
+    const bool live = row < rows;
+    U u[IT][8];
+    int emax = 1;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int c = lig + group * it;
+      if (live && c < chunks) {
+        const int seg = c >= cps ? 1 : 0;
+        const T* src = X + seg * seg_stride + row * seg_len + 8 * (c - seg * cps);
+        U h[4];
+        load4<T>(src, h);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) u[it][v] = h[v];
+        load4<T>(src + 4, h);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) u[it][4 + v] = h[v];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) emax = max(emax, (int)((u[it][v] >> MB) & Bits<T>::kExpMask));
+      }
+    }
+    for (int o = group / 2; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    if (!live) continue;
+    const bool bad = emax == Bits<T>::kExpMask;
+    if (lig == 0) ex[row] = bad ? kSliceBad : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int c = lig + group * it;
+      if (c < chunks) {
+        W w[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) w[v] = balanced<T>(u[it][v], emax, bad);
+        __nv_bfloat16* dst = dig + row * pitch + 8 * c;
+#pragma unroll
+        for (int a = 0; a < NS; ++a) {
+          uint32_t h[8];
+#pragma unroll
+          for (int v = 0; v < 8; ++v) {
+            const int d = a == 0 ? (int)(w[v] >> (RB * (NS - 1)))
+                                 : ((int)(w[v] >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
+            h[v] = __float_as_uint((float)d);
+          }
+          uint4 o;
+          o.x = __byte_perm(h[0], h[1], 0x7632);
+          o.y = __byte_perm(h[2], h[3], 0x7632);
+          o.z = __byte_perm(h[4], h[5], 0x7632);
+          o.w = __byte_perm(h[6], h[7], 0x7632);
+          *reinterpret_cast<uint4*>(dst + (size_t)a * rows * pitch) = o;
+        }
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------ product
 // Measured with the slicing pass (one real product, GB300): FP64 128 x 120 x 136
-// 73 us (900 us on the CUDA cores, whose FP64 rate is 1.1 TFLOP/s), 400 x 400 30
-// (414), 1023 x 1024 107 (4090), 432 x 432 x 100 926 (27010); relative error
-// 1.0e-16 .. 1.4e-16 (2.5e-16 .. 1.1e-15).  FP32 1023 x 1024 48 us (150), 432 x
-// 432 x 100 399 (1080); error 5e-8 (4e-7 .. 6e-7).
+// 58 us (900 us on the CUDA cores, whose FP64 rate is 1.1 TFLOP/s), 400 x 400 29
+// (412), 1023 x 1024 95 (4090), 432 x 432 x 100 811 (27014); relative error
+// 1.0e-16 .. 1.4e-16 (2.5e-16 .. 1.1e-15).  FP32 1023 x 1024 34 us (150), 432 x
+// 432 x 100 270 (1080); error 5e-8 (4e-7 .. 6e-7).
 // What bounds it: the bf16 tensor cores and, close behind, the operand bytes
 // an SM pulls from L2 (FP64: 84 KB per 32 k against 1792 MMA clocks, 47 bytes
 // per clock).  All levels of a tile share tensor memory (FP64 7 x 64, FP32
 // 4 x 128 columns), so the accumulators are single-buffered and the MMAs of
-// the next tile wait while the epilogue reads them; the stores overlap.
+// the next tile wait while the epilogue reads them.  16 epilogue warps therefore
+// only add the levels up to integer sums (16 or 32 columns each), hand tensor
+// memory back, and round and store while the next tile runs (8 warps that rounded
+// first: 1125 against 754 us for FP32 at 432^3, 67 against 51 for FP64 at
+// 128 x 120 x 136).
 template <typename T>
 struct GemmCfg;
 template <>
@@ -167,8 +257,10 @@ struct GemmCfg<float> {
 constexpr int kSegK = 1024;     // longest contraction whose digit sums stay exact (below 2^24)
 constexpr int kGK = 32;         // k per stage: 64-byte bf16 rows, 64-byte swizzle
 constexpr int kGM = 128;        // data rows per tile
-constexpr int kGEpi = 8;        // epilogue warps
-constexpr int kGThreads = 32 * (2 + kGEpi);
+constexpr int kGEpi = 16;       // epilogue warps
+constexpr int kGThreads = 32 * (4 + kGEpi);   // producer, MMA issuer, two idle ones
+// registers: 128 x 40 + 512 x 104 = 58368 of the 640 x 96 = 61440 at launch
+constexpr int kGRegCtl = 40, kGRegEpi = 104;
 
 template <typename T>
 struct GemmLayout {
@@ -193,9 +285,9 @@ struct GemmParams {
   int* err;
 };
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                : "r"(taddr));
 }
 // K-major, SWIZZLE_64B: rows of 64 bytes, 8-row groups 512 bytes apart
@@ -219,16 +311,32 @@ struct Sum<double> {
           (long long)__float2int_rn(P[6]);
   }
   // |hi| < 2^{39 + kb}: rounded to 53 bits through a 63-bit integer, V itself
-  // where it fits, else V / 2^kb, which then still has at least 62 - kb >= 52 bits
+  // where it fits, else V / 2^kb, which then still has at least 62 - kb >= 52
+  // bits.  To double by 32-bit integer arithmetic: FP64 additions and the
+  // conversion instruction run on the FP64 pipe at two lanes per clock and SM.
   __device__ __forceinline__ double get(int e, int kb) const {
-    const int s = (hi + (1ll << 38)) >> 39 == 0 ? 0 : kb;
-    const long long t = (hi << (24 - s)) + ((lo + ((1ll << s) >> 1)) >> s);
-    if (t == 0) return 0.0;
-    const double d = (double)t;
+    const int s = (hi + (1ll << 38)) >> 39 == 0 ? 0 : kb, up = 24 - s;   // kb <= 24: shifts below 32
+    const uint32_t h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
+    const long long lr = lo + ((1ll << s) >> 1);
+    const uint32_t l0 = (uint32_t)lr, l1 = (uint32_t)(lr >> 32);
+    const unsigned long long tu =
+        (((unsigned long long)__funnelshift_l(h0, h1, up) << 32) | (h0 << up)) +
+        (((unsigned long long)(uint32_t)((int)l1 >> s) << 32) | __funnelshift_r(l0, l1, s));
+    const long long t = (long long)tu;
     const int k = e + 48 + s;
-    // d has an exponent in [0, 63]: scale by adding to its exponent field while the result is normal
-    if (k > -1000 && k < 900) return __longlong_as_double(__double_as_longlong(d) + ((long long)k << 52));
-    return ldexp(d, k);
+    if (k <= -1000 || k >= 900) return ldexp((double)t, k);
+    // normalise to 64 bits, round to nearest even, fill in sign and exponent
+    const uint32_t sg = (uint32_t)((int)(tu >> 32) >> 31);
+    const unsigned long long mag = (tu ^ (((unsigned long long)sg << 32) | sg)) + (sg & 1u);
+    const uint32_t m1 = (uint32_t)(mag >> 32), m0 = (uint32_t)mag;
+    const uint32_t x1 = m1 ? m1 : m0, x0 = m1 ? m0 : 0u;
+    const int lz = __clz((int)x1);
+    const uint32_t n1 = __funnelshift_l(x0, x1, lz), n0 = x0 << lz;   // lz < 32 unless t == 0
+    const uint32_t up1 = (n0 >> 10) & (uint32_t)((n0 & 0x3FFu) != 0u || (n0 & 0x800u)) & 1u;
+    const uint32_t field = (uint32_t)(1022 + 63 - lz - (m1 ? 0 : 32) + k);
+    const unsigned long long bits = (((unsigned long long)((n1 >> 11) + (field << 20)) << 32) |
+                                     __funnelshift_r(n0, n1, 11)) + up1;
+    return tu == 0ull ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)(sg & 0x80000000u) << 32)));
   }
 };
 template <>
@@ -245,8 +353,7 @@ struct Sum<float> {
 };
 
 template <typename T>
-__device__ __forceinline__ T finish(const Sum<T>& s, int er, int i, const int* em, const GemmParams& gp) {
-  const int ei = i < gp.m ? __ldg(em + i) : 0;
+__device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei, const GemmParams& gp) {
   return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei, gp.kb);
 }
 
@@ -297,6 +404,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();
 
+  if (warp < 4) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGRegCtl));
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
@@ -370,42 +479,41 @@ __global__ void __launch_bounds__(kGThreads, 1)
       mma_commit(fin_bar);
       mbar_wait(fin_bar, 0, abort_flag, gp.err, 58, true);
     }
+  }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kGRegEpi));
     // ------------------------------------------------------------ epilogue
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    constexpr int NC = NT / 2;   // columns of this warp
+    // lane = data row, NC columns per warp: the levels into integer (FP32: float)
+    // sums, tensor memory back to the MMA warp, then rounding and stores
+    constexpr int NC = NT / 4;
+    const int q = warp & 3, cg = (warp - 4) >> 2;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     uint32_t t = 0;
     bool ok = true;
     const int segs = SEG ? (gp.k_chunks + kSegK / kGK - 1) / (kSegK / kGK) : 1;
     for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
       const long long row = (u / gp.m_tiles) * kGM + q * 32 + lane;
-      const int i0 = (int)(u % gp.m_tiles) * NT + half * NC;
+      const int i0 = (int)(u % gp.m_tiles) * NT + cg * NC;
       const bool live = row < gp.rows;
       const int er = live ? ex[row] : 0;
-      T y[NC];
-      Sum<T> sum[SEG ? NC : 1];
+      Sum<T> sum[NC];
       for (int sg = 0; sg < segs; ++sg, ++t) {
         if (!mbar_wait(acc_full, t & 1, abort_flag, gp.err, 59)) { ok = false; break; }
         tc_fence_after();
 #pragma unroll
-        for (int c0 = 0; c0 < NC; c0 += 8) {
-          uint32_t v[NLEV][8];
+        for (int c0 = 0; c0 < NC; c0 += 4) {
+          uint32_t v[NLEV][4];
 #pragma unroll
-          for (int l = 0; l < NLEV; ++l) tmem_ld8(tmem_base + lane_off + l * NT + half * NC + c0, v[l]);
+          for (int l = 0; l < NLEV; ++l) tmem_ld4(tmem_base + lane_off + l * NT + cg * NC + c0, v[l]);
           tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int l = 0; l < NLEV; ++l) tmem_loaded(v[l]);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
             float P[NLEV];
 #pragma unroll
             for (int l = 0; l < NLEV; ++l) P[l] = __uint_as_float(v[l][j]);
-            if constexpr (SEG) {
-              sum[c0 + j].add(P);
-            } else {
-              Sum<T> one;
-              one.add(P);
-              y[c0 + j] = finish(one, er, i0 + c0 + j, em, gp);
-            }
+            sum[c0 + j].add(P);
           }
         }
         tc_fence_before();
@@ -413,16 +521,18 @@ __global__ void __launch_bounds__(kGThreads, 1)
         if (lane == 0) mbar_arrive(acc_empty);
       }
       if (!ok) break;
-      if constexpr (SEG) {
-#pragma unroll
-        for (int j = 0; j < NC; ++j) y[j] = finish(sum[j], er, i0 + j, em, gp);
-      }
       if (live) {
         const long long c = row / gp.R;
-        T* dst = Y + c * gp.plane + (row - c * gp.R);
+        T* dst = Y + c * gp.plane + (row - c * gp.R) + (long long)i0 * gp.R;
+        const int4* e4 = reinterpret_cast<const int4*>(em + i0);   // readable up to a whole tile
 #pragma unroll
-        for (int j = 0; j < NC; ++j)
-          if (i0 + j < gp.m) dst[(long long)(i0 + j) * gp.R] = y[j];
+        for (int j4 = 0; j4 < NC / 4; ++j4) {
+          const int4 x = __ldg(e4 + j4);
+          const int ei[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (i0 + 4 * j4 + j < gp.m) dst[(long long)(4 * j4 + j) * gp.R] = finish(sum[4 * j4 + j], er, ei[j], gp);
+        }
       }
     }
   }
@@ -451,6 +561,21 @@ void slice_map(Sliced& s, bool matrix) {
 template <typename T>
 void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, cudaStream_t st,
                 long long& nl) {
+  const int chunks = nseg * seg_len / 8;
+  if (seg_len % 8 == 0 && chunks <= 128) {
+    int group = 1;
+    while (group < 32 && group < chunks) group *= 2;
+    const long long per_block = 256 / group;
+    const int blocks = (int)std::min<long long>((s.rows + per_block - 1) / per_block, (long long)num_sms() * 32);
+    const int it = (chunks + group - 1) / group;
+    launch_pdl(it == 1   ? slice8_kernel<T, 1>
+               : it == 2 ? slice8_kernel<T, 2>
+               : it == 3 ? slice8_kernel<T, 3>
+                         : slice8_kernel<T, 4>,
+               blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group, s.dig, s.ex);
+    FCGLE_LAUNCHED(nl);
+    return;
+  }
   const int quads = seg_len / 4;
   const int group = quads <= 8 ? 8 : (quads <= 16 ? 16 : 32);
   const long long per_block = 256 / group;

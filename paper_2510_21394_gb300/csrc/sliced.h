@@ -44,6 +44,9 @@ inline size_t slice_bytes(long long rows, int K) {
   return (size_t)SliceCfg<T>::NS * (size_t)rows * (size_t)slice_pitch(K) * 2;
 }
 
+// exponents of a matrix operand: the product reads them by whole tiles
+inline size_t slice_exponents(long long rows) { return (size_t)((rows + 127) / 128 * 128); }
+
 // Fills s.tm for s.dig / s.rows / s.K.  matrix: the box of the matrix operand
 // (M rows), else of the data operand.
 template <typename T>
