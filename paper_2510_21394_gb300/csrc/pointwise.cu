@@ -83,8 +83,27 @@ __device__ __forceinline__ RowMap row_map(const Shape& s, size_t rho) {
   return m;
 }
 
-template <typename T>
-__global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__ X) {
+// 4 values as bf16 hi + lo at hi[q..], lo[q..]
+__device__ __forceinline__ void st4_split(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t q, const float (&x)[4]) {
+  uint2 h, l;
+  uint32_t* hp = &h.x;
+  uint32_t* lp = &l.x;
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(x[2 * v], x[2 * v + 1]);
+    const float2 f = __bfloat1622float2(a);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(x[2 * v] - f.x, x[2 * v + 1] - f.y);
+    hp[v] = *reinterpret_cast<const uint32_t*>(&a);
+    lp[v] = *reinterpret_cast<const uint32_t*>(&b);
+  }
+  *reinterpret_cast<uint2*>(hi + q) = h;
+  *reinterpret_cast<uint2*>(lo + q) = l;
+}
+
+// SPLIT: the values go to hi and lo instead of X
+template <typename T, bool SPLIT>
+__global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__ X, __nv_bfloat16* __restrict__ hi,
+                            __nv_bfloat16* __restrict__ lo) {
   pdl_enter();
   const size_t P = s.P, quads_per_row = (size_t)s.p[0] / 4, nq = P / 4;
   const int n1 = s.n[0];
@@ -117,8 +136,13 @@ __global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__
           }
       }
     }
-    st4<T>(X + 4 * q4, re);
-    st4<T>(X + P + 4 * q4, im);
+    if constexpr (SPLIT) {
+      st4_split(hi, lo, 4 * q4, re);
+      st4_split(hi, lo, P + 4 * q4, im);
+    } else {
+      st4<T>(X + 4 * q4, re);
+      st4<T>(X + P + 4 * q4, im);
+    }
   }
 }
 
@@ -511,7 +535,12 @@ LamDev lamdev(const Shape& s, const LamVecs& lv) {
 // ===================================================================== host
 template <typename T>
 void pack(const Shape& s, const T* user, T* X, cudaStream_t st, long long& nl) {
-  launch_pdl(pack_kernel<T>, grid_for(s.P / 4, 256), 256, 0, st, s, user, X);
+  launch_pdl(pack_kernel<T, false>, grid_for(s.P / 4, 256), 256, 0, st, s, user, X, nullptr, nullptr);
+  FCGLE_LAUNCHED(nl);
+}
+void pack_split(const Shape& s, const float* user, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st,
+                long long& nl) {
+  launch_pdl(pack_kernel<float, true>, grid_for(s.P / 4, 256), 256, 0, st, s, user, nullptr, hi, lo);
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
