@@ -102,23 +102,6 @@ __global__ void gv_kernel(size_t P, GP g, const T* __restrict__ z, const T* __re
   block_acc<3>(v, acc, ADJ_GAMMA);
 }
 
-template <typename T>
-__global__ void gu_kernel(size_t P, GP g, const T* __restrict__ u, const T* __restrict__ la,
-                          const T* __restrict__ lb, double ca, double cb, T* __restrict__ out, double* acc) {
-  double v[3] = {0.0, 0.0, 0.0};
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
-    const double ar = la[q], ai = la[P + q], br = lb[q], bi = lb[P + q];
-    const double kr = ca * ar + cb * br, ki = ca * ai + cb * bi;
-    const double zr = u[q], zi = u[P + q];
-    double orr, oi;
-    gadj(g, zr, zi, kr, ki, orr, oi);
-    out[q] = (T)(ar + br + orr);
-    out[P + q] = (T)(ai + bi + oi);
-    gpar(zr, zi, kr, ki, v);
-  }
-  block_acc<3>(v, acc, ADJ_GAMMA);
-}
-
 struct LD {
   const double* lam[kMaxDim];
   int p[kMaxDim];
@@ -464,12 +447,6 @@ void adj_gv(const Shape& s, const GParams& gp, const T* z, const T* w, double c,
   FCGLE_LAUNCHED(nl);
 }
 template <typename T>
-void adj_gu(const Shape& s, const GParams& gp, const T* u, const T* la, const T* lb, double ca, double cb, T* out,
-            double* acc, cudaStream_t st, long long& nl) {
-  gu_kernel<T><<<grid_of(s.P), 256, 0, st>>>(s.P, GP{gp.gamma, gp.kappa, gp.zeta}, u, la, lb, ca, cb, out, acc);
-  FCGLE_LAUNCHED(nl);
-}
-template <typename T>
 void adj_spec_dot(const Shape& s, const LamVecs& lv, const T* x, const T* y, double* acc, cudaStream_t st,
                   long long& nl) {
   if constexpr (std::is_same<T, float>::value)
@@ -518,8 +495,6 @@ void adj_exp_h_combo(const Shape& s, const LamVecs& lv, double theta, const T* x
   template void adj_misfit<T>(const Shape&, const T*, const T*, T*, double*, cudaStream_t, long long&);          \
   template void adj_gv<T>(const Shape&, const GParams&, const T*, const T*, double, T*, AdjSplit, double*,       \
                           cudaStream_t, long long&);                                                            \
-  template void adj_gu<T>(const Shape&, const GParams&, const T*, const T*, const T*, double, double, T*,       \
-                          double*, cudaStream_t, long long&);                                                   \
   template void adj_spec_dot<T>(const Shape&, const LamVecs&, const T*, const T*, double*, cudaStream_t,        \
                                 long long&);                                                                    \
   template void adj_axpby<T>(const Shape&, double, const T*, double, const T*, T*, AdjSplit, cudaStream_t,        \

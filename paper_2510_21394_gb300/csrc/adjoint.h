@@ -35,8 +35,6 @@
 
 #include "common.h"
 
-struct __nv_bfloat16;
-
 namespace fcgle {
 
 // A tensor a split-BF16 operator reads, as its two bf16 planes pairs (2 P values
@@ -68,11 +66,6 @@ void adj_misfit(const Shape& s, const T* u, const T* target, T* lam, double* acc
 template <typename T>
 void adj_gv(const Shape& s, const GParams& gp, const T* z, const T* w, double c, T* mu, AdjSplit sp, double* acc,
             cudaStream_t st, long long& nl);
-
-// lk1 = ca la + cb lb;  out = la + lb + (D_u g)^* lk1;  acc[GAMMA..ZETA] += Re<lk1, (u, ...)>
-template <typename T>
-void adj_gu(const Shape& s, const GParams& gp, const T* u, const T* la, const T* lb, double ca, double cb, T* out,
-            double* acc, cudaStream_t st, long long& nl);
 
 // acc[Z_RE, Z_IM] += sum conj(x) Lam_D y  (Lam_D from the lam_mu vectors, weight 1)
 template <typename T>
