@@ -27,7 +27,8 @@
  * Streams.  Every device entry point is asynchronous on the handle's CUDA
  *   stream (given at setup, changeable with fcgle_set_stream); the caller
  *   synchronises.  _host entry points synchronise before returning.
- *   The tensor-core mode-product kernels of FCGLE_BF16X3 handles are launched
+ *   The tensor-core mode-product kernels and the slicing, layout and
+ *   pointwise kernels of a step are launched
  *   with programmatic dependent launch: each may start its prologue while the
  *   previous kernel of the stream drains and waits for that kernel's
  *   completion before touching global memory, so stream order is kept.  The
@@ -333,8 +334,10 @@ fcgle_status fcgle_internal_elems(fcgle_handle h, size_t* P);
  * integration, FP32 in and out: split-TF32 (x = hi + lo, both TF32, three
  * tensor-core products hi.hi + hi.lo + lo.hi, about 2^-21 relative) when
  * d >= 2, R is a multiple of 8 and p_mu <= 256 (the tensor core's FP32
- * accumulation error grows with the contracted length), FP32 on the CUDA
- * cores otherwise.  flags bit 3 (BF16X3 handles, d = 3, p_2 <= 256, with
+ * accumulation error grows with the contracted length).  Handles with d >= 2
+ * and any p > 256 use FP32 products by integer slices (both operands as
+ * fixed-point numbers of 25 bits and a sign per row of the contraction, summed
+ * exactly on the bf16 tensor cores); otherwise FP32 on the CUDA cores.  flags bit 3 (BF16X3 handles, d = 3, p_2 <= 256, with
  * bit 1, direction 0): the slab-fused mode-1 and mode-2 products in the
  * natural order, Y[c][j3][i2][i1] = sum M_2[i2][j2] M_1[i1][j1]
  * X[c][j3][j2][j1] with M_mu = Q_mu^T (bit 0) or Q_mu.  flags bit 4 (BF16X3

@@ -8,12 +8,11 @@
 //   complex matrix in real block form B = [[Re E, -Im E], [Im E, Re E]]
 //   (2p x 2p):                    row = r, R rows; kk = (c, k), K = 2p;
 //     A(r, (c, k)) = X[c][r][k];   Y[c'][i][r] = C[r][(c', i)].
-// GB300's FP64 rate is a small fraction of its tensor-core rate, so this
-// is a plain shared-memory tiled SIMT GEMM (64 x 64 tile, 4 x 4 per thread):
-// it is FP64-ALU bound by a wide margin at every size used here.  The same
-// kernel in FP32 (real matrices only) serves the split-BF16 engine for the
-// few transforms per solve that must not carry the split-BF16 error (the
-// first forward and the last backward Tucker operator of a time integration).
+// A plain shared-memory tiled SIMT GEMM (64 x 64 tile, 4 x 4 per thread), bound
+// by the FP64 ALU (1.1 TFLOP/s on GB300).  It runs the contractions below 16
+// and unaligned operands; every other FP64 product is the sliced one of
+// sliced.cu.  The same kernel in FP32 (real matrices only) serves the precise
+// transforms of the adjoint and of 1D split-BF16 handles.
 #include "common.h"
 
 namespace fcgle {
