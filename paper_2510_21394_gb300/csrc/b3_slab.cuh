@@ -40,9 +40,7 @@
 //               the 16-column groups (convert) or 32-column boxes (store) of
 //               parity (w - 2) / 4
 // Every mbarrier wait is bounded (mbar_wait); on expiry the CTA records an
-// error code, drains its own TMA and MMA work (in a cluster: waits, bounded, for
-// its peer's copies and arrivals too, and leaves together with it), frees its TMEM
-// and returns.
+// error code, drains its own TMA and MMA work, frees its TMEM and returns.
 //
 // Requirements (checked by the host): p2 <= 256; p1 and p2 multiples of 8
 // (16-byte rows of every tensor map).
@@ -80,48 +78,11 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t addr) {
          ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
-// ---- clusters of two CTAs that share operands: each loads half of what both
-// need and multicasts it, and a stage is free when both have consumed it
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-      "%3}], [%4], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_3d_mc(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-      "%3, %4}], [%5], %6;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "h"(mask)
-      : "memory");
-}
-// arrives on the barrier at the same offset in every CTA of the mask
-__device__ __forceinline__ void mma_commit_mc(uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"(mask)
-      : "memory");
-}
-
-// SHARE (an even number of i1-blocks): units 2 j and 2 j + 1, the same slab and
-// two i1-blocks, run on a cluster of two CTAs; the slab's chunks and those of M2
-// are loaded once for both (TMA multicast, each CTA loading half).  At 256^3 the
-// kernel is not bound by L2 (77 us either way); with rows that are no multiple of
-// 64 bytes a box row touches a third sector, and 248 x 248 x 256 takes 82 us
-// instead of 94.  One i1-block, sharing M1 and M2 between two slabs: no gain at
-// 128^3.
-template <bool SHARE>
+// One CTA per unit; no operand is shared between CTAs.  At 256^3 L2 traffic is not
+// the bound (77 us with each slab chunk and M2 loaded once per CTA pair, 77 us
+// without); where a row is no multiple of 64 bytes a box row touches a third
+// sector (248 x 248 x 256: 94 us, 82 us with shared loads).  The kernel also runs
+// in the multi-process paths, so it uses no multicast loads.
 __global__ void __launch_bounds__(SL_THREADS, 1)
     mp_b3_slab12_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_constant__ CUtensorMap tm_xlo,
                         const __grid_constant__ CUtensorMap tm_m1hi, const __grid_constant__ CUtensorMap tm_m1lo,
@@ -150,7 +111,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < SL_NS; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), SHARE ? 2 : 1);   // the MMA of every CTA that reads the stage
+      mbar_init(empty_bar(s), 1);
     }
     mbar_init(d1_full, 1);
     for (int c = 0; c < 4; ++c) mbar_init(u_full(c), SL_NEPI);
@@ -166,10 +127,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
-  if constexpr (SHARE)
-    cluster_sync();   // the peer's barriers are initialised too
-  else
-    __syncthreads();
+  __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();
@@ -183,7 +141,6 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
       uint32_t g = 0;
       bool ok = true;
       const uint32_t xbytes = (uint32_t)sp.n2 * 64;   // one N2 x 32 bf16 box
-      const uint32_t rank = SHARE ? cluster_rank() : 0;
       const int m2boxes = sp.n2 > 128 ? 2 : 1;
       for (long long u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const int z = (int)(u / sp.mb1), b1 = (int)(u % sp.mb1);
@@ -194,12 +151,8 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
           mbar_arrive_tx(full_bar(s), 16384 + 2 * xbytes);
           tma_load_2d(st, &tm_m1hi, kc * SL_K, b1 * BM, full_bar(s));
           tma_load_2d(st + 8192, &tm_m1lo, kc * SL_K, b1 * BM, full_bar(s));
-          if constexpr (SHARE) {
-            tma_load_3d_mc(st + 16384 + rank * 16384, rank ? &tm_xlo : &tm_xhi, kc * SL_K, 0, z, full_bar(s), 3);
-          } else {
-            tma_load_3d(st + 16384, &tm_xhi, kc * SL_K, 0, z, full_bar(s));
-            tma_load_3d(st + 32768, &tm_xlo, kc * SL_K, 0, z, full_bar(s));
-          }
+          tma_load_3d(st + 16384, &tm_xhi, kc * SL_K, 0, z, full_bar(s));
+          tma_load_3d(st + 32768, &tm_xlo, kc * SL_K, 0, z, full_bar(s));
         }
         for (int kc = 0; kc < sp.kc2 && ok; ++kc, ++g) {
           const int s = (int)(g % SL_NS);
@@ -207,23 +160,15 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
           const uint32_t st = sbase + s * kSlStage;
           mbar_arrive_tx(full_bar(s), (uint32_t)m2boxes * 16384);
           for (int b = 0; b < m2boxes; ++b) {
-            if constexpr (SHARE) {
-              tma_load_2d_mc(st + rank * 16384 + b * 8192, rank ? &tm_m2lo : &tm_m2hi, kc * SL_K, b * BM, full_bar(s),
-                             3);
-            } else {
-              tma_load_2d(st + b * 8192, &tm_m2hi, kc * SL_K, b * BM, full_bar(s));
-              tma_load_2d(st + 16384 + b * 8192, &tm_m2lo, kc * SL_K, b * BM, full_bar(s));
-            }
+            tma_load_2d(st + b * 8192, &tm_m2hi, kc * SL_K, b * BM, full_bar(s));
+            tma_load_2d(st + 16384 + b * 8192, &tm_m2lo, kc * SL_K, b * BM, full_bar(s));
           }
         }
       }
-      // drain: every issued stage must have landed before the CTA may exit (in a
-      // cluster: landed in both CTAs and released by both)
+      // drain: every issued stage must have landed before the CTA may exit
       const uint32_t issued = g;
-      for (uint32_t q = issued >= SL_NS ? issued - SL_NS : 0; q < issued; ++q) {
+      for (uint32_t q = issued >= SL_NS ? issued - SL_NS : 0; q < issued; ++q)
         mbar_wait(full_bar(q % SL_NS), (q / SL_NS) & 1, abort_flag, err, 37, true);
-        if constexpr (SHARE) mbar_wait(empty_bar(q % SL_NS), (q / SL_NS) & 1, abort_flag, err, 42, true);
-      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -232,12 +177,6 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
       const uint32_t idesc =
           (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(sp.n2 >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       const int ksteps2 = sp.n2 / 16;
-      auto release = [](uint32_t bar) {
-        if constexpr (SHARE)
-          mma_commit_mc(bar, 3);
-        else
-          mma_commit(bar);
-      };
       uint32_t g = 0, t = 0;
       bool ok = true;
       for (long long u = blockIdx.x; u < units && ok; u += gridDim.x, ++t) {
@@ -259,7 +198,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
             mma_bf16(tmem_base, sw64_desc(ahi + off), sw64_desc(blo + off), idesc, 1u);
             mma_bf16(tmem_base, sw64_desc(alo + off), sw64_desc(bhi + off), idesc, 1u);
           }
-          release(empty_bar(s));
+          mma_commit(empty_bar(s));
         }
         if (!ok) break;
         mma_commit(d1_full);
@@ -284,7 +223,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
               mma_bf16_ts(e_tmem, ulo, sw64_desc(bhi + off), idesc, 1u);
             }
           }
-          release(empty_bar(s));
+          mma_commit(empty_bar(s));
         }
         if (!ok) break;
         mma_commit(d2_full);
@@ -378,12 +317,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   }
 
   tc_fence_before();
-  if constexpr (SHARE) {
-    __syncwarp();
-    cluster_sync();   // no CTA leaves while its peer may still write to it or arrive on its barriers
-  } else {
-    __syncthreads();
-  }
+  __syncthreads();
   tc_fence_after();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
 }

@@ -475,8 +475,8 @@ class EngineB3 : public EngineBase {
       FusedLaunch<b3::EpiLRK2A>::attributes();
       FusedLaunch<b3::EpiLRK2B>::attributes();
       FusedLaunch<b3::EpiStrangB>::attributes();
-      for (auto* k : {b3::mp_b3_slab12_kernel<false>, b3::mp_b3_slab12_kernel<true>})
-        FCGLE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b3::kSlSmemBytes));
+      FCGLE_CUDA(cudaFuncSetAttribute(b3::mp_b3_slab12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)b3::kSlSmemBytes));
       FusedLaunchCx<b3::EpiStoreF32>::attributes();
       FusedLaunchCx<b3::EpiStoreSplitGen>::attributes();
       FusedLaunchCx<b3::EpiUpdateG>::attributes();
@@ -1371,12 +1371,9 @@ class EngineB3 : public EngineBase {
     encode_bf16_3d(&tyh, out.hi, (uint64_t)p1, (uint64_t)p2, 2 * (uint64_t)p3, 32, 32, 0);
     encode_bf16_3d(&tyl, out.lo, (uint64_t)p1, (uint64_t)p2, 2 * (uint64_t)p3, 32, 32, 0);
     const long long units = 2LL * p3 * sp.mb1;
-    // an even number of i1-blocks: units 2 j and 2 j + 1 run on a cluster of two CTAs that share the slab
-    const int cluster = sp.mb1 % 2 == 0 ? 2 : 1;
-    const int grid = (int)std::min<long long>(units, num_sms() / cluster * cluster);
-    launch_pdl_cluster(cluster, cluster == 1 ? b3::mp_b3_slab12_kernel<false> : b3::mp_b3_slab12_kernel<true>, grid,
-                       b3::SL_THREADS, b3::kSlSmemBytes, st_, txh, txl, m1.tm_hi64, m1.tm_lo64, m2.tm_hi64, m2.tm_lo64,
-                       tyh, tyl, sp);
+    const int grid = (int)std::min<long long>(units, num_sms());
+    launch_pdl(b3::mp_b3_slab12_kernel, grid, b3::SL_THREADS, b3::kSlSmemBytes, st_, txh, txl, m1.tm_hi64,
+               m1.tm_lo64, m2.tm_hi64, m2.tm_lo64, tyh, tyl, sp);
     FCGLE_LAUNCHED(launches);
   }
 

@@ -26,34 +26,19 @@ inline bool pdl_enabled() {
   return on;
 }
 
-// cluster > 1: blocks in clusters of that size along x (grid a multiple of it).
 template <class... P, class... A>
-void launch_pdl_cluster(int cluster, void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st,
-                        A&&... args) {
+void launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  unsigned n = 0;
-  if (pdl_enabled()) {
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n++].val.programmaticStreamSerializationAllowed = 1;
-  }
-  if (cluster > 1) {
-    attr[n].id = cudaLaunchAttributeClusterDimension;
-    attr[n].val.clusterDim.x = (unsigned)cluster;
-    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
-    ++n;
-  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = n;
+  cfg.numAttrs = pdl_enabled() ? 1 : 0;
   FCGLE_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
-}
-template <class... P, class... A>
-void launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
-  launch_pdl_cluster(1, kernel, grid, threads, smem, st, std::forward<A>(args)...);
 }
 
 inline int num_sms() {
