@@ -57,6 +57,16 @@ void throw_cuda(cudaError_t e, const char* where);
     if (e__ != cudaSuccess) ::fcgle::throw_cuda(e__, "kernel launch"); \
   } while (0)
 
+// Host to device in the order of stream st, complete on return.  Setup data goes
+// this way and not by plain cudaMemcpy: that one runs on the legacy default
+// stream, which streams made with cudaStreamNonBlocking (a batch's) do not wait
+// for, and from pageable memory it may return before the last bytes have landed,
+// so that a kernel on st could read a matrix that is still on its way.
+inline void upload(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  FCGLE_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
+  FCGLE_CUDA(cudaStreamSynchronize(st));
+}
+
 // ------------------------------------------------------- pointwise kernels
 // Layout conversion between the user layout (interleaved complex, dense,
 // vec order) and the internal planar padded layout.

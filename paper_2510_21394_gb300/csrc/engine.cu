@@ -127,7 +127,7 @@ class Engine : public EngineBase {
       std::vector<double> lp(D.p, 0.0);
       for (int j = 0; j < D.n; ++j) lp[j] = D.lam[j];
       lam_[mu].reset(new DevBuf<double>(D.p));
-      FCGLE_CUDA(cudaMemcpy(lam_[mu]->ptr, lp.data(), D.p * sizeof(double), cudaMemcpyHostToDevice));
+      upload(lam_[mu]->ptr, lp.data(), D.p * sizeof(double), st_);
       // forward matrix M[i][k] = Q[k][i] (Q^T), backward M[i][k] = Q[i][k]; zero padded to p x p
       std::vector<double> Mf((size_t)D.p * D.p, 0.0), Mb((size_t)D.p * D.p, 0.0);
       for (int i = 0; i < D.n; ++i)
@@ -137,8 +137,8 @@ class Engine : public EngineBase {
         }
       mf64_[mu][0].reset(new DevBuf<double>(Mf.size()));
       mf64_[mu][1].reset(new DevBuf<double>(Mb.size()));
-      FCGLE_CUDA(cudaMemcpy(mf64_[mu][0]->ptr, Mf.data(), Mf.size() * 8, cudaMemcpyHostToDevice));
-      FCGLE_CUDA(cudaMemcpy(mf64_[mu][1]->ptr, Mb.data(), Mb.size() * 8, cudaMemcpyHostToDevice));
+      upload(mf64_[mu][0]->ptr, Mf.data(), Mf.size() * 8, st_);
+      upload(mf64_[mu][1]->ptr, Mb.data(), Mb.size() * 8, st_);
     }
     // ---- sliced products: digits of the matrices, workspace for those of the data
     size_t xbytes = 0;

@@ -396,8 +396,8 @@ class EngineB3 : public EngineBase {
       }
       lamf_[mu].reset(new DevMem<float>(s_.p[mu]));
       lamd_[mu].reset(new DevMem<double>(s_.p[mu]));
-      FCGLE_CUDA(cudaMemcpy(lamf_[mu]->ptr, lf.data(), lf.size() * 4, cudaMemcpyHostToDevice));
-      FCGLE_CUDA(cudaMemcpy(lamd_[mu]->ptr, ld.data(), ld.size() * 8, cudaMemcpyHostToDevice));
+      upload(lamf_[mu]->ptr, lf.data(), lf.size() * 4, st_);
+      upload(lamd_[mu]->ptr, ld.data(), ld.size() * 8, st_);
       const int p = s_.p[mu];
       std::vector<double> Mf((size_t)p * p, 0.0), Mb((size_t)p * p, 0.0);
       for (int i = 0; i < D.n; ++i)
@@ -860,8 +860,8 @@ class EngineB3 : public EngineBase {
       const size_t bytes = hi.size() * 2;
       FCGLE_CUDA(cudaMalloc(&c->hi, bytes));
       FCGLE_CUDA(cudaMalloc(&c->lo, bytes));
-      FCGLE_CUDA(cudaMemcpy(c->hi, hi.data(), bytes, cudaMemcpyHostToDevice));
-      FCGLE_CUDA(cudaMemcpy(c->lo, lo.data(), bytes, cudaMemcpyHostToDevice));
+      upload(c->hi, hi.data(), bytes, st_);
+      upload(c->lo, lo.data(), bytes, st_);
       encode_bf16(&c->tm_hi, c->hi, (uint64_t)c->k_pad, rows, b3::BM);
       encode_bf16(&c->tm_lo, c->lo, (uint64_t)c->k_pad, rows, b3::BM);
       v.push_back(std::move(c));
@@ -952,8 +952,8 @@ class EngineB3 : public EngineBase {
     const size_t bytes = hi.size() * 2;
     FCGLE_CUDA(cudaMalloc(&m.hi, bytes));
     FCGLE_CUDA(cudaMalloc(&m.lo, bytes));
-    FCGLE_CUDA(cudaMemcpy(m.hi, hi.data(), bytes, cudaMemcpyHostToDevice));
-    FCGLE_CUDA(cudaMemcpy(m.lo, lo.data(), bytes, cudaMemcpyHostToDevice));
+    upload(m.hi, hi.data(), bytes, st_);
+    upload(m.lo, lo.data(), bytes, st_);
     encode_bf16(&m.tm_hi, m.hi, m.k_pad, m.m_pad, b3::BM);
     encode_bf16(&m.tm_lo, m.lo, m.k_pad, m.m_pad, b3::BM);
     encode_bf16_sw64(&m.tm_hi64, m.hi, m.k_pad, m.m_pad, b3::BM);
@@ -961,7 +961,7 @@ class EngineB3 : public EngineBase {
     std::vector<float> f((size_t)p * p);
     for (size_t e = 0; e < f.size(); ++e) f[e] = (float)M[e];
     FCGLE_CUDA(cudaMalloc(&m.f32, f.size() * 4));
-    FCGLE_CUDA(cudaMemcpy(m.f32, f.data(), f.size() * 4, cudaMemcpyHostToDevice));
+    upload(m.f32, f.data(), f.size() * 4, st_);
     // split-TF32: hi = tf32(M), lo = tf32(M - hi), zero padded to (m_pad, k_pad32)
     m.k_pad32 = (p + 31) / 32 * 32;
     std::vector<float> th((size_t)m.m_pad * m.k_pad32, 0.0f), tl(th);
@@ -974,8 +974,8 @@ class EngineB3 : public EngineBase {
       }
     FCGLE_CUDA(cudaMalloc(&m.thi, th.size() * 4));
     FCGLE_CUDA(cudaMalloc(&m.tlo, tl.size() * 4));
-    FCGLE_CUDA(cudaMemcpy(m.thi, th.data(), th.size() * 4, cudaMemcpyHostToDevice));
-    FCGLE_CUDA(cudaMemcpy(m.tlo, tl.data(), tl.size() * 4, cudaMemcpyHostToDevice));
+    upload(m.thi, th.data(), th.size() * 4, st_);
+    upload(m.tlo, tl.data(), tl.size() * 4, st_);
     encode_f32(&m.tm_thi, m.thi, m.k_pad32, m.m_pad, b3::BM);
     encode_f32(&m.tm_tlo, m.tlo, m.k_pad32, m.m_pad, b3::BM);
   }

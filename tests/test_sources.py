@@ -13,3 +13,13 @@ def test_no_multicast_loads():
     for f in files:
         with open(f) as fh:
             assert "multicast::cluster" not in fh.read(), os.path.basename(f)
+
+
+def test_setup_uploads_follow_the_stream():
+    # a plain cudaMemcpy runs on the legacy default stream, which non-blocking
+    # streams (a batch's) do not wait for: host data reaches a handle by upload()
+    files = glob.glob(os.path.join(CSRC, "*.cu*")) + glob.glob(os.path.join(CSRC, "*.cpp"))
+    for f in files:
+        with open(f) as fh:
+            for line in fh:
+                assert not ("cudaMemcpy(" in line and "cudaMemcpyHostToDevice" in line), (os.path.basename(f), line)
