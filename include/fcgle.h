@@ -311,6 +311,12 @@ fcgle_status fcgle_sync(fcgle_handle h);
  * FCGLE_ERR_INVALID_ARG before anything runs. */
 fcgle_status fcgle_selftest_bounded_wait(void* cuda_stream, int* code_out);
 
+/* Segment length of an FP64 sliced product with the real matrix M (rows x K,
+ * row-major, on the host): the largest number of terms, in equal segments of
+ * whole 32s, whose leading digit sums the FP32 accumulator holds exactly
+ * whatever the data.  A host computation; no GPU is used. */
+fcgle_status fcgle_selftest_slice_segment(const double* M, int rows, int K, int* terms);
+
 /* Sizes: N (complex elements of a user tensor) and the bytes of one user
  * tensor. */
 fcgle_status fcgle_sizes(fcgle_handle h, size_t* n_elems, size_t* n_bytes);

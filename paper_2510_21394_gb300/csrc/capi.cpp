@@ -14,6 +14,7 @@
 #include "engine.h"
 #include "norm_static.h"
 #include "selftest.h"
+#include "sliced.h"
 
 struct fcgle_ctx {
   fcgle_params prm;
@@ -320,6 +321,14 @@ fcgle_status fcgle_norm_static(const fcgle_params* p, const void* u, void* cuda_
     if (p->precision != FCGLE_FP64 && p->precision != FCGLE_BF16X3) throw InvalidArg("unknown precision");
     const double s = norm_static_sumsq(u, p->precision == FCGLE_FP64, N, (cudaStream_t)cuda_stream);
     *out_host = std::sqrt(cell * s);
+  });
+}
+
+fcgle_status fcgle_selftest_slice_segment(const double* M, int rows, int K, int* terms) {
+  return guarded([&] {
+    if (!M || !terms) throw InvalidArg("NULL argument");
+    if (rows < 1 || K < 1) throw InvalidArg("rows and K must be >= 1");
+    *terms = slice_segment<double>(M, rows, K);
   });
 }
 

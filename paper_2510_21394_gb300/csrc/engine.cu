@@ -121,7 +121,19 @@ class Engine : public EngineBase {
         dir_[mu].p = s_.p[mu];
       }
     }
-    // ---- device copies: lam_mu (padded), mode-product matrices
+    // ---- shapes of the sliced products
+    size_t xbytes = 0;
+    long long xrows = 0;
+    for (int mu = 0; mu < prm.d; ++mu)
+      for (int cx = 0; cx < 2; ++cx) {
+        Sliced& x = xs_[mu][cx];
+        x.rows = (long long)(s_.P / s_.p[mu]) * (cx ? 1 : 2);
+        x.K = s_.p[mu] * (cx ? 2 : 1);
+        if (!sliceable(x.K, x.rows)) continue;
+        xbytes = std::max(xbytes, slice_bytes<double>(x.rows, x.K));
+        xrows = std::max(xrows, x.rows);
+      }
+    // ---- device copies: lam_mu (padded), mode-product matrices and their digits
     for (int mu = 0; mu < prm.d; ++mu) {
       const Direction& D = dir_[mu];
       std::vector<double> lp(D.p, 0.0);
@@ -139,24 +151,17 @@ class Engine : public EngineBase {
       mf64_[mu][1].reset(new DevBuf<double>(Mb.size()));
       upload(mf64_[mu][0]->ptr, Mf.data(), Mf.size() * 8, st_);
       upload(mf64_[mu][1]->ptr, Mb.data(), Mb.size() * 8, st_);
-    }
-    // ---- sliced products: digits of the matrices, workspace for those of the data
-    size_t xbytes = 0;
-    long long xrows = 0;
-    for (int mu = 0; mu < prm.d; ++mu)
-      for (int cx = 0; cx < 2; ++cx) {
-        Sliced& x = xs_[mu][cx];
-        x.rows = (long long)(s_.P / s_.p[mu]) * (cx ? 1 : 2);
-        x.K = s_.p[mu] * (cx ? 2 : 1);
-        if (!sliceable(x.K, x.rows)) continue;
-        xbytes = std::max(xbytes, slice_bytes<double>(x.rows, x.K));
-        xrows = std::max(xrows, x.rows);
+      if (sliceable(xs_[mu][0].K, xs_[mu][0].rows)) {
+        ms_[mu][0].build(mf64_[mu][0]->ptr, Mf, D.p, st_, launches);
+        ms_[mu][1].build(mf64_[mu][1]->ptr, Mb, D.p, st_, launches);
       }
+    }
+    // ---- workspace for the digits of the data
     if (xbytes) {
       xdig_.reset(new DevBuf<uint8_t>(xbytes));
       xex_.reset(new DevBuf<int>((size_t)xrows));
     }
-    for (int mu = 0; mu < prm.d; ++mu) {
+    for (int mu = 0; mu < prm.d; ++mu)
       for (int cx = 0; cx < 2; ++cx) {
         Sliced& x = xs_[mu][cx];
         if (!sliceable(x.K, x.rows)) continue;
@@ -164,9 +169,6 @@ class Engine : public EngineBase {
         x.ex = xex_->ptr;
         slice_map<double>(x, false);
       }
-      if (sliceable(xs_[mu][0].K, xs_[mu][0].rows))
-        for (int f = 0; f < 2; ++f) ms_[mu][f].build(mf64_[mu][f]->ptr, s_.p[mu], st_, launches);
-    }
     lv_.c_re = prm.nu;
     lv_.c_im = prm.eta;
     for (int mu = 0; mu < kMaxDim; ++mu) lv_.lam[mu] = mu < prm.d ? lam_[mu]->ptr : nullptr;
@@ -390,8 +392,10 @@ class Engine : public EngineBase {
     Sliced s;
     std::unique_ptr<DevBuf<uint8_t>> dig;
     std::unique_ptr<DevBuf<int>> ex;
-    void build(const double* M, int K, cudaStream_t st, long long& nl) {
+    // M: on the device, Mh: the same on the host
+    void build(const double* M, const std::vector<double>& Mh, int K, cudaStream_t st, long long& nl) {
       s.rows = s.K = K;
+      s.seg = slice_segment(Mh.data(), K, K);
       dig.reset(new DevBuf<uint8_t>(slice_bytes<double>(K, K)));
       ex.reset(new DevBuf<int>(slice_exponents(K)));
       s.dig = reinterpret_cast<__nv_bfloat16*>(dig->ptr);
@@ -544,7 +548,7 @@ class Engine : public EngineBase {
       v.emplace_back();
       v.back().f64.reset(new DevBuf<double>(Bm.size()));
       FCGLE_CUDA(cudaMemcpyAsync(v.back().f64->ptr, Bm.data(), Bm.size() * 8, cudaMemcpyHostToDevice, st_));
-      if (sliceable(xs_[mu][1].K, xs_[mu][1].rows)) v.back().sl.build(v.back().f64->ptr, 2 * p, st_, launches);
+      if (sliceable(xs_[mu][1].K, xs_[mu][1].rows)) v.back().sl.build(v.back().f64->ptr, Bm, 2 * p, st_, launches);
       FCGLE_CUDA(cudaStreamSynchronize(st_));
     }
     return v;

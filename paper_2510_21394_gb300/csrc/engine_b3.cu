@@ -440,6 +440,7 @@ class EngineB3 : public EngineBase {
         for (int f = 0; f < 2; ++f) {
           Mat& m = mat_[mu][f];
           m.sl.rows = m.sl.K = m.p;
+          m.sl.seg = slice_segment<float>(nullptr, m.p, m.p);   // the same for every matrix
           FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<float>(m.p, m.p)));
           FCGLE_CUDA(cudaMalloc(&m.sl.ex, slice_exponents(m.p) * sizeof(int)));
           slice_map<float>(m.sl, true);

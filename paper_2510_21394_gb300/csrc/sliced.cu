@@ -9,11 +9,29 @@
 // holds exactly, and
 //     Y[i][r] = 2^{E_i + E_r} sum_s 2^{RB (2 NS - 2 - s)} P_s,
 //     P_s = sum_{a + b = s} sum_k m_a[i][k] x_b[r][k],   s < NLEV,
-// where every P_s is a sum of integers that the FP32 accumulator holds exactly
-// (products of the top digits <= 2^14, 2^24 over 1024 of them; longer
-// contractions go in segments).  The levels s >= NLEV are below the rounding of T.  The epilogue
-// adds the levels as 64-bit integers (FP64 arithmetic would cost more than the
-// product) and rounds once.
+// each P_s summed as integers in the FP32 accumulator.  The epilogue adds the
+// levels as 64-bit integers (FP64 arithmetic would cost more than the product)
+// and rounds once.
+//
+// What the accumulator holds exactly: integers up to 2^24.  Level s takes s + 1
+// products per k, of digits |d| <= 2^{RB - 1} (the top ones <= 128), so FP64 P_s
+// is at most (s + 1) 2^14 per k.  A unit lost in P_s is 2^{-8 s} of a unit of
+// P_0: levels 0 .. 3 have to be exact, and are, whatever the data: contractions
+// go in segments short enough for the digits of the matrix at hand
+// (slice_segment; 256 terms always do, and 400 to 1024 for eigenvector matrices,
+// whose lower digits average half the largest).  Levels 4 .. 6 reach at most 7/4
+// of what level 3 does; a unit lost there is 2^-46 of one full-size term
+// max|x| max|M_i|, and it takes hundreds of terms with all digits in line to lose
+// one.  FP32: P_0 <= 2^14 per k is exact over 1024 terms; digits below the
+// top one reach 256, so P_1 .. P_3 may pass 2^24 (up to 2^27) when hundreds of
+// their digits are in line, and then lose up to 2^-14 max|x| max|M_i| over 1024
+// terms, which is what 1024 roundings of an FP32 product come to; digits that
+// are not in line stay below 2^21.
+//
+// Cut off: half a unit of an operand's last digit, and the levels s >= NLEV, for
+// an error per entry of about 2^-55 sqrt(K) max|x| max|M_i| (FP64; FP32: 2^-26),
+// relative to the largest entries of the two fibers, not to the entry's own
+// terms.
 //
 // Orientation: the data rows (c, r) are the MMA's M (TMEM lanes), so that a
 // warp stores 32 consecutive r of one output index i; 64 (FP64) or 128 (FP32)
@@ -25,8 +43,11 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstdlib>
+#include <cstring>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "b3_kernel.cuh"
 #include "sliced.h"
@@ -82,13 +103,13 @@ struct Balanced<float> {
   using W = int;
 };
 template <typename T>
-__device__ __forceinline__ typename Balanced<T>::W balanced(typename Bits<T>::U u, int emax, bool bad) {
+__host__ __device__ __forceinline__ typename Balanced<T>::W balanced(typename Bits<T>::U u, int emax, bool bad) {
   using U = typename Bits<T>::U;
   using W = typename Balanced<T>::W;
   constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
   const int e = (int)((u >> MB) & Bits<T>::kExpMask);
   const U mant = ((u & ((U(1) << MB) - 1)) | (e ? U(1) << MB : U(0))) << UP;
-  const int s = emax - max(e, 1);
+  const int s = emax - (e > 1 ? e : 1);
   const U m = s < (int)(8 * sizeof(U)) - 2 ? (mant + ((U(1) << s) >> 1)) >> s : U(0);
   W x = (u >> (8 * sizeof(U) - 1)) ? -(W)m : (W)m;
   if (bad) x = 0;
@@ -254,7 +275,7 @@ struct GemmCfg<float> {
   static constexpr int NLEV = 4, NT = 128, NSTAGE = 4;
 };
 
-constexpr int kSegK = 1024;     // longest contraction whose digit sums stay exact (below 2^24)
+constexpr int kSegK = 1024;     // longest contraction whose level 0 stays exact (below 2^24)
 constexpr int kGK = 32;         // k per stage: 64-byte bf16 rows, 64-byte swizzle
 constexpr int kGM = 128;        // data rows per tile
 constexpr int kGEpi = 16;       // epilogue warps
@@ -282,6 +303,7 @@ struct GemmParams {
   int m_tiles, k_chunks;
   long long units;
   int kb;            // bits of the contraction length (FP64 epilogue)
+  int seg;           // k-chunks of a segment
   int* err;
 };
 
@@ -357,7 +379,7 @@ __device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei, const GemmP
   return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei, gp.kb);
 }
 
-// SEG: contractions longer than kSegK go in segments, each drained from tensor
+// SEG: the contraction goes in segments of gp.seg chunks, each drained from tensor
 // memory into the integer sums before the next begins.
 template <typename T, bool SEG>
 __global__ void __launch_bounds__(kGThreads, 1)
@@ -439,7 +461,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
       bool ok = true;
       for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
         for (int kc = 0; kc < gp.k_chunks; ++kc, ++g) {
-          const bool begin = SEG ? kc % (kSegK / kGK) == 0 : kc == 0;
+          const bool begin = SEG ? kc % gp.seg == 0 : kc == 0;
           if (begin) {
             if (!mbar_wait(acc_empty, (t & 1) ^ 1, abort_flag, gp.err, 52)) { ok = false; break; }
             tc_fence_after();
@@ -469,7 +491,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
             }
           }
           mma_commit(empty_bar(s));
-          if (kc + 1 == gp.k_chunks || (SEG && (kc + 1) % (kSegK / kGK) == 0)) {
+          if (kc + 1 == gp.k_chunks || (SEG && (kc + 1) % gp.seg == 0)) {
             mma_commit(acc_full);
             ++t;
           }
@@ -490,7 +512,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     uint32_t t = 0;
     bool ok = true;
-    const int segs = SEG ? (gp.k_chunks + kSegK / kGK - 1) / (kSegK / kGK) : 1;
+    const int segs = SEG ? (gp.k_chunks + gp.seg - 1) / gp.seg : 1;
     for (long long u = blockIdx.x; u < gp.units && ok; u += gridDim.x) {
       const long long row = (u / gp.m_tiles) * kGM + q * 32 + lane;
       const int i0 = (int)(u % gp.m_tiles) * NT + cg * NC;
@@ -544,6 +566,53 @@ __global__ void __launch_bounds__(kGThreads, 1)
 }
 
 }  // namespace
+
+// The levels that have to be exact are summed in the worst case, with the data's
+// digits at their largest and in line with the matrix's: sum over a <= s of
+// 2^{RB - 1} |m_a| for every row and segment (FP32: only P_0, which is within
+// 2^24 over kSegK terms whatever the digits).
+template <typename T>
+int slice_segment(const T* M, int rows, int K) {
+  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB;
+  const int chunks = (K + kGK - 1) / kGK;
+  int seg = std::min(chunks, kSegK / kGK);
+  if (sizeof(T) == 8) {
+    constexpr int kExact = 4;   // levels 0 .. 3
+    // per row and chunk: sum of |m_0| + .. + |m_3|, which bounds the lower levels too
+    std::vector<int> sum((size_t)rows * chunks, 0);
+    for (int i = 0; i < rows; ++i) {
+      const T* row = M + (size_t)i * K;
+      int emax = 1;
+      auto bits = [](T x) {
+        typename Bits<T>::U u;
+        std::memcpy(&u, &x, sizeof(u));
+        return u;
+      };
+      for (int k = 0; k < K; ++k) emax = std::max(emax, (int)((bits(row[k]) >> Bits<T>::kMant) & Bits<T>::kExpMask));
+      const bool bad = emax == Bits<T>::kExpMask;
+      for (int k = 0; k < K; ++k) {
+        const auto w = balanced<T>(bits(row[k]), emax, bad);
+        for (int a = 0; a < kExact; ++a) {
+          const int dig = a == 0 ? (int)(w >> (RB * (NS - 1)))
+                                 : ((int)(w >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
+          sum[(size_t)i * chunks + k / kGK] += std::abs(dig);
+        }
+      }
+    }
+    for (int n = (chunks + seg - 1) / seg;; ++n) {
+      seg = (chunks + n - 1) / n;
+      bool fits = true;
+      for (int i = 0; i < rows && fits; ++i)
+        for (int c0 = 0; c0 < chunks && fits; c0 += seg) {
+          long long level = 0;
+          for (int c = c0; c < std::min(c0 + seg, chunks); ++c) level += sum[(size_t)i * chunks + c];
+          fits = (level << (RB - 1)) <= (1ll << 24);
+        }
+      if (fits) break;   // at the latest with 8 chunks = 256 terms: 4 x 128 x 128 x 256 = 2^24
+    }
+  }
+  return seg * kGK;
+}
 
 template <typename T>
 void slice_map(Sliced& s, bool matrix) {
@@ -605,13 +674,16 @@ void sliced_gemm(const Sliced& x, const Sliced& m, T* Y, long long R, long long 
   gp.units = (x.rows + kGM - 1) / kGM * gp.m_tiles;
   gp.kb = 0;
   while ((1 << gp.kb) < x.K) ++gp.kb;
+  gp.seg = m.seg / kGK;
   gp.err = err;
-  launch_pdl(x.K <= kSegK ? sliced_gemm_kernel<T, false> : sliced_gemm_kernel<T, true>, (int)std::min<long long>(gp.units, num_sms()), kGThreads, GemmLayout<T>::kSmem, st,
-             x.tm, m.tm, (const int*)x.ex, (const int*)m.ex, Y, gp);
+  launch_pdl(gp.k_chunks <= gp.seg ? sliced_gemm_kernel<T, false> : sliced_gemm_kernel<T, true>,
+             (int)std::min<long long>(gp.units, num_sms()), kGThreads, GemmLayout<T>::kSmem, st, x.tm, m.tm,
+             (const int*)x.ex, (const int*)m.ex, Y, gp);
   FCGLE_LAUNCHED(nl);
 }
 
 #define INST(T)                                                                                                  \
+  template int slice_segment<T>(const T*, int, int);                                                             \
   template void slice_map<T>(Sliced&, bool);                                                                     \
   template void slice_rows<T>(const T*, const Sliced&, int, int, long long, cudaStream_t, long long&);           \
   template void sliced_gemm<T>(const Sliced&, const Sliced&, T*, long long, long long, int*, cudaStream_t, long long&);

@@ -35,6 +35,7 @@ struct Sliced {
   int* ex = nullptr;
   long long rows = 0;
   int K = 0;
+  int seg = 0;      // matrix operand: terms of the contraction whose leading levels are summed exactly
   CUtensorMap tm;   // boxes of (32 k, 128 rows or the matrix tile) of one slice
 };
 
@@ -51,6 +52,10 @@ inline size_t slice_exponents(long long rows) { return (size_t)((rows + 127) / 1
 // (M rows), else of the data operand.
 template <typename T>
 void slice_map(Sliced& s, bool matrix);
+
+// Terms of a segment of the contraction with M (rows x K, host): a multiple of 32.
+template <typename T>
+int slice_segment(const T* M, int rows, int K);
 
 // Slices the rows of X: row r is nseg segments of seg_len contiguous elements,
 // segment c at X + c * seg_stride + r * seg_len; s.K = nseg * seg_len.

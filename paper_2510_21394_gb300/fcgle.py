@@ -51,8 +51,8 @@ EXPORTS = ["fcgle_setup", "fcgle_set_stream", "fcgle_set_source", "fcgle_apply_f
            "fcgle_launch_count", "fcgle_destroy", "fcgle_status_string", "fcgle_last_error",
            "fcgle_internal_elems", "fcgle_mode_product", "fcgle_adjoint", "fcgle_set_coefficients",
            "fcgle_batch_create", "fcgle_batch_instance", "fcgle_batch_integrate", "fcgle_batch_launch_count",
-           "fcgle_batch_destroy", "fcgle_norm_static", "fcgle_selftest_bounded_wait", "fcgle_spectral_scalars",
-           "fcgle_autotune_report", "fcgle_set_exp_form", "fcgle_set_tucker_form"]
+           "fcgle_batch_destroy", "fcgle_norm_static", "fcgle_selftest_bounded_wait", "fcgle_selftest_slice_segment",
+           "fcgle_spectral_scalars", "fcgle_autotune_report", "fcgle_set_exp_form", "fcgle_set_tucker_form"]
 
 
 class fcgle_params(ctypes.Structure):
@@ -101,6 +101,7 @@ def _load():
         "fcgle_batch_destroy": [H],
         "fcgle_norm_static": [ctypes.POINTER(fcgle_params), P, P, ctypes.POINTER(D)],
         "fcgle_selftest_bounded_wait": [P, ctypes.POINTER(I)],
+        "fcgle_selftest_slice_segment": [ctypes.POINTER(ctypes.c_double), I, I, ctypes.POINTER(I)],
         "fcgle_spectral_scalars": [H, I, I, D, I, ctypes.POINTER(D), ctypes.POINTER(D), I],
         "fcgle_autotune_report": [ctypes.c_char_p, ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)],
         "fcgle_set_exp_form": [H, I],
@@ -326,6 +327,15 @@ def fcgle_selftest_bounded_wait(stream=None):
     code = ctypes.c_int(-1)
     status = _lib.fcgle_selftest_bounded_wait(_stream(stream), ctypes.byref(code))
     return status, code.value
+
+
+def fcgle_selftest_slice_segment(M):
+    """Segment length (terms) of an FP64 sliced product with the matrix M (rows, K)."""
+    M = torch.as_tensor(M, dtype=torch.float64, device="cpu").contiguous()
+    terms = ctypes.c_int(0)
+    ptr = ctypes.cast(M.data_ptr(), ctypes.POINTER(ctypes.c_double))
+    _check(_lib.fcgle_selftest_slice_segment(ptr, M.shape[0], M.shape[1], ctypes.byref(terms)))
+    return terms.value
 
 
 def fcgle_sync(h):

@@ -1,0 +1,59 @@
+"""FP64 sliced products with data whose digits are in line with the matrix's, so
+that the digit sums come near their bounds, against extended precision.
+
+Tolerance: that of test_gpu_sliced.py (each operand entry cut at 2^-55 of its
+row's largest, random over K, times 8, plus the rounding of the result)."""
+import numpy as np
+import pytest
+
+from test_slice_segment import _digits
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fc():
+    import __graft_entry__ as g
+    g.build()
+    from paper_2510_21394_gb300 import fcgle
+    return fcgle
+
+
+@pytest.mark.parametrize("n", [1023, 1500])
+def test_digits_in_line(fc, n):
+    s = fc.Solver([n, 8], [(-4.0, 4.0), (-3.0, 3.0)], [1.3, 1.7], 1.0, 0.4, 0.5, 1.0, 0.2, precision="fp64")
+    p = (n + 3) // 4 * 4
+    R = fc.fcgle_internal_elems(s.h) // p
+
+    def product(X):
+        Xd = torch.from_numpy(np.ascontiguousarray(X)).cuda().reshape(-1)
+        Y = torch.full_like(Xd, 7.0)
+        fc.fcgle_mode_product(s.h, 0, 1, Xd, Y)
+        s.sync()
+        return Y.reshape(2, p, R).permute(0, 2, 1).reshape(2 * R, p).cpu().numpy()
+
+    cols = []
+    for k0 in range(0, p, 2 * R):
+        E = np.zeros((2 * R, p))
+        m = min(2 * R, p - k0)
+        E[np.arange(m), k0 + np.arange(m)] = 1.0
+        cols.append(product(E)[:m])
+    M = np.concatenate(cols).T                      # M[i][k]
+    # row r: digits 127 in line with those of row i = i_r of M, digit b with level
+    # 3 - b, so that all four products of level 3 have one sign; odd rows: all of one sign
+    rows = np.linspace(0, n - 1, 2 * R).astype(int)
+    dig = _digits(M[rows])
+    X = np.zeros((2 * R, p))
+    for r in range(2 * R):
+        for b in range(4):
+            sgn = np.where(dig[3 - b, r] < 0, -1.0, 1.0) if r % 2 == 0 else np.ones(p)
+            X[r] += 127.0 * sgn * 2.0 ** (-8 * b)
+    X[:, n:] = 0.0
+    Y = product(X)
+    T = X.astype(np.longdouble) @ M.astype(np.longdouble).T
+    err = np.abs(Y.astype(np.longdouble) - T)
+    xm = np.abs(X).max(axis=1, keepdims=True).astype(np.longdouble)
+    mm = np.abs(M).max(axis=1)[None, :].astype(np.longdouble)
+    assert np.all(err <= 2.0 ** -53 * np.abs(T) + 8 * 2.0 ** -55 * np.sqrt(p) * xm * mm)
+    s.close()
