@@ -18,10 +18,10 @@
 // is at most (s + 1) 2^14 per k.  A unit lost in P_s is 2^{-8 s} of a unit of
 // P_0: levels 0 .. 3 have to be exact, and are, whatever the data: contractions
 // go in segments short enough for the digits of the matrix at hand
-// (slice_segment; 256 terms always do, and 400 to 1024 for eigenvector matrices,
+// (slice_segment; 256 terms always do, and 350 to 450 with eigenvector matrices,
 // whose lower digits average half the largest).  Levels 4 .. 6 reach at most 7/4
-// of what level 3 does; a unit lost there is 2^-46 of one full-size term
-// max|x| max|M_i|, and it takes hundreds of terms with all digits in line to lose
+// of what level 3 does; a unit lost there is at most 2^-46 of one full-size
+// term max|x| max|M_i| (2^-22 at level 1), and it takes hundreds of terms with all digits in line to lose
 // one.  FP32: P_0 <= 2^14 per k is exact over 1024 terms; digits below the
 // top one reach 256, so P_1 .. P_3 may pass 2^24 (up to 2^27) when hundreds of
 // their digits are in line, and then lose up to 2^-14 max|x| max|M_i| over 1024
@@ -302,7 +302,6 @@ struct GemmParams {
   int m;             // output indices
   int m_tiles, k_chunks;
   long long units;
-  int kb;            // bits of the contraction length (FP64 epilogue)
   int seg;           // k-chunks of a segment
   int* err;
 };
@@ -332,12 +331,12 @@ struct Sum<double> {
     lo += ((long long)__float2int_rn(P[4]) << 16) + ((long long)__float2int_rn(P[5]) << 8) +
           (long long)__float2int_rn(P[6]);
   }
-  // |hi| < 2^{39 + kb}: rounded to 53 bits through a 63-bit integer, V itself
-  // where it fits, else V / 2^kb, which then still has at least 62 - kb >= 52
-  // bits.  To double by 32-bit integer arithmetic: FP64 additions and the
-  // conversion instruction run on the FP64 pipe at two lanes per clock and SM.
-  __device__ __forceinline__ double get(int e, int kb) const {
-    const int s = (hi + (1ll << 38)) >> 39 == 0 ? 0 : kb, up = 24 - s;   // kb <= 24: shifts below 32
+  // |hi| < 2^38 K: rounded to 53 bits through a 63-bit integer t = V / 2^s, s the
+  // smallest shift that makes it fit, so that t is V itself or has 62 bits.  To
+  // double by 32-bit integer arithmetic: FP64 additions and the conversion
+  // instruction run on the FP64 pipe at two lanes per clock and SM.
+  __device__ __forceinline__ double get(int e) const {
+    const int s = max(0, 26 - __clzll(hi ^ (hi >> 63))), up = 24 - s;   // bits of |hi| beyond 38; K <= 2^24: s <= 24
     const uint32_t h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
     const long long lr = lo + ((1ll << s) >> 1);
     const uint32_t l0 = (uint32_t)lr, l1 = (uint32_t)(lr >> 32);
@@ -367,7 +366,7 @@ struct Sum<float> {
   __device__ __forceinline__ void add(const float (&P)[4]) {
     t += fmaf(fmaf(fmaf(P[3], 1.f / 512.f, P[2]), 1.f / 512.f, P[1]), 1.f / 512.f, P[0]);
   }
-  __device__ __forceinline__ float get(int e, int) const {
+  __device__ __forceinline__ float get(int e) const {
     const int k = e + 36;
     if (k >= -126 && k <= 127) return t * __int_as_float((k + 127) << 23);
     return ldexpf(t, k);
@@ -375,8 +374,8 @@ struct Sum<float> {
 };
 
 template <typename T>
-__device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei, const GemmParams& gp) {
-  return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei, gp.kb);
+__device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei) {
+  return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei);
 }
 
 // SEG: the contraction goes in segments of gp.seg chunks, each drained from tensor
@@ -553,7 +552,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
           const int ei[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (i0 + 4 * j4 + j < gp.m) dst[(long long)(4 * j4 + j) * gp.R] = finish(sum[4 * j4 + j], er, ei[j], gp);
+            if (i0 + 4 * j4 + j < gp.m) dst[(long long)(4 * j4 + j) * gp.R] = finish(sum[4 * j4 + j], er, ei[j]);
         }
       }
     }
@@ -672,8 +671,6 @@ void sliced_gemm(const Sliced& x, const Sliced& m, T* Y, long long R, long long 
   gp.m_tiles = (gp.m + GemmCfg<T>::NT - 1) / GemmCfg<T>::NT;
   gp.k_chunks = (x.K + kGK - 1) / kGK;
   gp.units = (x.rows + kGM - 1) / kGM * gp.m_tiles;
-  gp.kb = 0;
-  while ((1 << gp.kb) < x.K) ++gp.kb;
   gp.seg = m.seg / kGK;
   gp.err = err;
   launch_pdl(gp.k_chunks <= gp.seg ? sliced_gemm_kernel<T, false> : sliced_gemm_kernel<T, true>,

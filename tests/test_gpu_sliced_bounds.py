@@ -3,6 +3,8 @@ that the digit sums come near their bounds, against extended precision.
 
 Tolerance: that of test_gpu_sliced.py (each operand entry cut at 2^-55 of its
 row's largest, random over K, times 8, plus the rounding of the result)."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -20,8 +22,8 @@ def fc():
     return fcgle
 
 
-@pytest.mark.parametrize("n", [1023, 1500])
-def test_digits_in_line(fc, n):
+def _problem(fc, n):
+    """FP64 handle of (n, 8), its product of direction 0 on rows (2 R, p), and the matrix M[i][k] read back."""
     s = fc.Solver([n, 8], [(-4.0, 4.0), (-3.0, 3.0)], [1.3, 1.7], 1.0, 0.4, 0.5, 1.0, 0.2, precision="fp64")
     p = (n + 3) // 4 * 4
     R = fc.fcgle_internal_elems(s.h) // p
@@ -39,7 +41,12 @@ def test_digits_in_line(fc, n):
         m = min(2 * R, p - k0)
         E[np.arange(m), k0 + np.arange(m)] = 1.0
         cols.append(product(E)[:m])
-    M = np.concatenate(cols).T                      # M[i][k]
+    return s, p, R, product, np.concatenate(cols).T
+
+
+@pytest.mark.parametrize("n", [1023, 1500])
+def test_digits_in_line(fc, n):
+    s, p, R, product, M = _problem(fc, n)
     # row r: digits 127 in line with those of row i = i_r of M, digit b with level
     # 3 - b, so that all four products of level 3 have one sign; odd rows: all of one sign
     rows = np.linspace(0, n - 1, 2 * R).astype(int)
@@ -56,4 +63,29 @@ def test_digits_in_line(fc, n):
     xm = np.abs(X).max(axis=1, keepdims=True).astype(np.longdouble)
     mm = np.abs(M).max(axis=1)[None, :].astype(np.longdouble)
     assert np.all(err <= 2.0 ** -53 * np.abs(T) + 8 * 2.0 ** -55 * np.sqrt(p) * xm * mm)
+    s.close()
+
+
+@pytest.mark.parametrize("n,terms", [(1500, 8), (1500, 40), (400, 8)])
+def test_exact_sums_round_once(fc, n, terms):
+    """Operands without a cut: data with one digit, matrix entries within 1/4 of
+    their row's largest.  The integer sum is then exact, and the result is its
+    rounding to 53 bits (through an integer of 62 bits: 2^-53 (1 + 2^-8))."""
+    s, p, R, product, M = _problem(fc, n)
+    rng = np.random.default_rng(11)
+    X = np.zeros((2 * R, p))
+    big = np.abs(M) >= np.abs(M).max(axis=1, keepdims=True) / 4
+    ok = np.zeros((2 * R, p), bool)
+    for r in range(2 * R):
+        k = rng.permutation(np.flatnonzero(big[rng.integers(0, n)]))[:terms]   # one output at least qualifies
+        X[r, k] = 127.0 / 64.0 * np.where(M[rng.integers(0, n), k] < 0, -1.0, 1.0)
+        ok[r] = big[:, k].all(axis=1)
+    ok[:, n:] = False
+    assert ok.any(axis=1).all()
+    Y = product(X)
+    for r in range(2 * R):
+        k = np.flatnonzero(X[r])
+        for i in np.flatnonzero(ok[r])[:40]:
+            t = sum(Fraction(float(X[r, c])) * Fraction(float(M[i, c])) for c in k)
+            assert abs(Fraction(float(Y[r, i])) - t) <= abs(t) * Fraction(257, 256) / 2 ** 53
     s.close()
