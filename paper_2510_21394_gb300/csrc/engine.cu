@@ -401,7 +401,7 @@ class Engine : public EngineBase {
       s.dig = reinterpret_cast<__nv_bfloat16*>(dig->ptr);
       s.ex = ex->ptr;
       slice_map<double>(s, true);
-      slice_rows<double>(M, s, 1, K, 0, st, nl);
+      slice_rows<double>(M, s, 1, K, 0, SliceOut<double>{}, st, nl);
     }
   };
   // The sliced product (two launches) against the CUDA cores, us: 12.6 / 21.0 at
@@ -415,7 +415,7 @@ class Engine : public EngineBase {
     const Sliced& x = xs_[mu][cx];
     if (m.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
       const long long plane = R * s_.p[mu];
-      slice_rows<double>(X, x, cx ? 2 : 1, s_.p[mu], plane, st_, launches);
+      slice_rows<double>(X, x, cx ? 2 : 1, s_.p[mu], plane, SliceOut<double>{M, Y, R, plane, x.K}, st_, launches);
       sliced_gemm<double>(x, m.s, Y, R, plane, err_->ptr, st_, launches);
       return;
     }
@@ -548,7 +548,9 @@ class Engine : public EngineBase {
       v.emplace_back();
       v.back().f64.reset(new DevBuf<double>(Bm.size()));
       FCGLE_CUDA(cudaMemcpyAsync(v.back().f64->ptr, Bm.data(), Bm.size() * 8, cudaMemcpyHostToDevice, st_));
-      if (sliceable(xs_[mu][1].K, xs_[mu][1].rows)) v.back().sl.build(v.back().f64->ptr, Bm, 2 * p, st_, launches);
+      // (e^{theta K} of a growing mode can overflow: then on the CUDA cores, entry by entry)
+      const bool finite = std::all_of(Bm.begin(), Bm.end(), [](double x) { return std::isfinite(x); });
+      if (finite && sliceable(xs_[mu][1].K, xs_[mu][1].rows)) v.back().sl.build(v.back().f64->ptr, Bm, 2 * p, st_, launches);
       FCGLE_CUDA(cudaStreamSynchronize(st_));
     }
     return v;

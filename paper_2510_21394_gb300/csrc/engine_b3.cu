@@ -444,7 +444,7 @@ class EngineB3 : public EngineBase {
           FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<float>(m.p, m.p)));
           FCGLE_CUDA(cudaMalloc(&m.sl.ex, slice_exponents(m.p) * sizeof(int)));
           slice_map<float>(m.sl, true);
-          slice_rows<float>(m.f32, m.sl, 1, m.p, 0, st_, launches);
+          slice_rows<float>(m.f32, m.sl, 1, m.p, 0, SliceOut<float>{}, st_, launches);
         }
       }
     }
@@ -1063,7 +1063,7 @@ class EngineB3 : public EngineBase {
     const Mat& m = mat_[mu][fwd ? 0 : 1];
     const long long R = P_ / s_.p[mu];
     if (m.sl.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
-      slice_rows<float>(X, xs_[mu], 1, s_.p[mu], 0, st_, launches);
+      slice_rows<float>(X, xs_[mu], 1, s_.p[mu], 0, SliceOut<float>{m.f32, Y, R, P_, m.p}, st_, launches);
       sliced_gemm<float>(xs_[mu], m.sl, Y, R, P_, err_->ptr, st_, launches);
     } else {
       mp_f32(X, Y, m.f32, s_.p[mu], (size_t)R, st_, launches);

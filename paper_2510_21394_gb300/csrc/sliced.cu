@@ -59,7 +59,10 @@ namespace {
 
 using namespace b3;
 
-constexpr int kSliceBad = 0x40000000;   // exponent of a row that holds a NaN or an Inf
+// exponents of rows that digits cannot hold: a NaN among the entries (the product
+// writes NaN), an Inf but no NaN (the slicing pass writes the row's results)
+constexpr int kSliceNaN = 0x40000000, kSliceInf = 0x40000001;
+__device__ __forceinline__ bool unsliced(int e) { return e >= kSliceNaN; }
 
 // ------------------------------------------------------------ slicing pass
 // HBM-bound (FP64: 8 bytes read and 14 written per element), so one pass: a
@@ -119,10 +122,44 @@ __host__ __device__ __forceinline__ typename Balanced<T>::W balanced(typename Bi
   return x + off;
 }
 
+// After a block's rows are cut, by the lanes that found a row with an Inf or a NaN
+// among theirs: rows whose only non-finite entries are infinities get their
+// results here, M[i][k] (+-Inf) summed over these, which is what the sum over all
+// entries comes to.  Apart from the loop over the rows, which it would cost registers.
+template <typename T>
+__device__ __noinline__ void infinite_rows(const T* X, long long rows, int nseg, int seg_len, long long seg_stride,
+                                           int group, int* ex, const SliceOut<T>& o) {
+  if (!o.M) return;
+  const int per_block = 256 / group, lig = threadIdx.x % group, K = nseg * seg_len;
+  for (long long row = (long long)blockIdx.x * per_block + threadIdx.x / group; row < rows;
+       row += (long long)gridDim.x * per_block) {
+    const T* src = X + row * seg_len;
+    bool nan = false, inf = false;
+    for (int k = 0; k < K && !nan; ++k) {
+      const T x = src[(k / seg_len) * seg_stride + k % seg_len];
+      nan = isnan(x);
+      inf |= isinf(x);
+    }
+    if (nan || !inf) continue;
+    const long long c = row / o.R;
+    T* dst = o.Y + c * o.plane + (row - c * o.R);
+    for (int i = lig; i < o.m; i += group) {
+      T sum = 0;
+      for (int k = 0; k < K && !isnan(sum); ++k) {
+        const T x = src[(k / seg_len) * seg_stride + k % seg_len];
+        if (isinf(x)) sum += o.M[(size_t)i * K + k] * x;
+      }
+      dst[(long long)i * o.R] = sum;
+    }
+    if (lig == 0) ex[row] = kSliceInf;   // the same lane wrote kSliceNaN
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
                                                     long long seg_stride, int pitch, int group,
-                                                    __nv_bfloat16* __restrict__ dig, int* __restrict__ ex) {
+                                                    __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
+                             const __grid_constant__ SliceOut<T> o) {
   using U = typename Bits<T>::U;
   constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant;
   constexpr int UP = SliceCfg<T>::BITS - MB - 2;   // spare bits below the last one of the largest entry
@@ -131,6 +168,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
   const int per_block = 256 / group;
   const int lig = threadIdx.x % group;
   const int quads = seg_len / 4;
+  bool any_bad = false;
   for (long long row0 = (long long)blockIdx.x * per_block; row0 < rows; row0 += (long long)gridDim.x * per_block) {
     const long long row = row0 + threadIdx.x / group;
     const bool live = row < rows;
@@ -148,8 +186,9 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
     for (int o = group / 2; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
     if (!live) continue;
     const bool bad = emax == Bits<T>::kExpMask;
+    any_bad |= bad;
     // x = mant 2^{e - bias - MB}; v = (mant << UP) >> (emax - e): unit 2^{emax - bias - MB - UP}
-    if (lig == 0) ex[row] = bad ? kSliceBad : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
+    if (lig == 0) ex[row] = bad ? kSliceNaN : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
     for (int c = 0; c < nseg; ++c) {
       const T* src = X + c * seg_stride + row * seg_len;
       __nv_bfloat16* dst = dig + row * pitch + c * seg_len;
@@ -169,14 +208,15 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
                                  : ((int)(w[v] >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
             h[v] = __float_as_uint((float)d);
           }
-          uint2 o;
-          o.x = (h[0] >> 16) | (h[1] & 0xFFFF0000u);
-          o.y = (h[2] >> 16) | (h[3] & 0xFFFF0000u);
-          *reinterpret_cast<uint2*>(dst + (size_t)a * rows * pitch + 4 * q) = o;
+          uint2 d2;
+          d2.x = (h[0] >> 16) | (h[1] & 0xFFFF0000u);
+          d2.y = (h[2] >> 16) | (h[3] & 0xFFFF0000u);
+          *reinterpret_cast<uint2*>(dst + (size_t)a * rows * pitch + 4 * q) = d2;
         }
       }
     }
   }
+  if (any_bad) infinite_rows<T>(X, rows, nseg, seg_len, seg_stride, group, ex, o);
 }
 
 // The same pass for rows of up to 8 x 32 x IT elements in segments of a multiple
@@ -186,7 +226,8 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
 template <typename T, int IT>
 __global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
                                                      long long seg_stride, int pitch, int group,
-                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex) {
+                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
+                             const __grid_constant__ SliceOut<T> o) {
   using U = typename Bits<T>::U;
   using W = typename Balanced<T>::W;
   constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
@@ -194,6 +235,7 @@ __global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, lo
   pdl_wait();
   const int per_block = 256 / group, lig = threadIdx.x % group;
   const int cps = seg_len / 8, chunks = nseg * cps;
+  bool any_bad = false;
   for (long long row0 = (long long)blockIdx.x * per_block; row0 < rows; row0 += (long long)gridDim.x * per_block) {
     const long long row = row0 + threadIdx.x / group;
     const bool live = row < rows;
@@ -219,7 +261,8 @@ __global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, lo
     for (int o = group / 2; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
     if (!live) continue;
     const bool bad = emax == Bits<T>::kExpMask;
-    if (lig == 0) ex[row] = bad ? kSliceBad : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
+    any_bad |= bad;
+    if (lig == 0) ex[row] = bad ? kSliceNaN : emax - (Bits<T>::kExpMask >> 1) - MB - UP;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const int c = lig + group * it;
@@ -237,16 +280,17 @@ __global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, lo
                                  : ((int)(w[v] >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
             h[v] = __float_as_uint((float)d);
           }
-          uint4 o;
-          o.x = __byte_perm(h[0], h[1], 0x7632);
-          o.y = __byte_perm(h[2], h[3], 0x7632);
-          o.z = __byte_perm(h[4], h[5], 0x7632);
-          o.w = __byte_perm(h[6], h[7], 0x7632);
-          *reinterpret_cast<uint4*>(dst + (size_t)a * rows * pitch) = o;
+          uint4 d4;
+          d4.x = __byte_perm(h[0], h[1], 0x7632);
+          d4.y = __byte_perm(h[2], h[3], 0x7632);
+          d4.z = __byte_perm(h[4], h[5], 0x7632);
+          d4.w = __byte_perm(h[6], h[7], 0x7632);
+          *reinterpret_cast<uint4*>(dst + (size_t)a * rows * pitch) = d4;
         }
       }
     }
   }
+  if (any_bad) infinite_rows<T>(X, rows, nseg, seg_len, seg_stride, group, ex, o);
 }
 
 // ------------------------------------------------------------ product
@@ -375,7 +419,7 @@ struct Sum<float> {
 
 template <typename T>
 __device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei) {
-  return er == kSliceBad || ei == kSliceBad ? (T)NAN : s.get(er + ei);
+  return unsliced(er) || unsliced(ei) ? (T)NAN : s.get(er + ei);
 }
 
 // SEG: the contraction goes in segments of gp.seg chunks, each drained from tensor
@@ -542,7 +586,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         if (lane == 0) mbar_arrive(acc_empty);
       }
       if (!ok) break;
-      if (live) {
+      if (live && er != kSliceInf) {   // rows with an Inf are the slicing pass's
         const long long c = row / gp.R;
         T* dst = Y + c * gp.plane + (row - c * gp.R) + (long long)i0 * gp.R;
         const int4* e4 = reinterpret_cast<const int4*>(em + i0);   // readable up to a whole tile
@@ -627,8 +671,8 @@ void slice_map(Sliced& s, bool matrix) {
 }
 
 template <typename T>
-void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, cudaStream_t st,
-                long long& nl) {
+void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, const SliceOut<T>& o,
+                cudaStream_t st, long long& nl) {
   const int chunks = nseg * seg_len / 8;
   if (seg_len % 8 == 0 && chunks <= 128) {
     int group = 1;
@@ -640,7 +684,7 @@ void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long se
                : it == 2 ? slice8_kernel<T, 2>
                : it == 3 ? slice8_kernel<T, 3>
                          : slice8_kernel<T, 4>,
-               blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group, s.dig, s.ex);
+               blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group, s.dig, s.ex, o);
     FCGLE_LAUNCHED(nl);
     return;
   }
@@ -649,7 +693,7 @@ void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long se
   const long long per_block = 256 / group;
   const long long blocks = std::min<long long>((s.rows + per_block - 1) / per_block, (long long)num_sms() * 16);
   launch_pdl(slice_kernel<T>, (int)blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group,
-             s.dig, s.ex);
+             s.dig, s.ex, o);
   FCGLE_LAUNCHED(nl);
 }
 
@@ -682,7 +726,8 @@ void sliced_gemm(const Sliced& x, const Sliced& m, T* Y, long long R, long long 
 #define INST(T)                                                                                                  \
   template int slice_segment<T>(const T*, int, int);                                                             \
   template void slice_map<T>(Sliced&, bool);                                                                     \
-  template void slice_rows<T>(const T*, const Sliced&, int, int, long long, cudaStream_t, long long&);           \
+  template void slice_rows<T>(const T*, const Sliced&, int, int, long long, const SliceOut<T>&, cudaStream_t,    \
+                              long long&);                                                                       \
   template void sliced_gemm<T>(const Sliced&, const Sliced&, T*, long long, long long, int*, cudaStream_t, long long&);
 INST(float)
 INST(double)

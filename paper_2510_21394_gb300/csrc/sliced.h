@@ -57,11 +57,22 @@ void slice_map(Sliced& s, bool matrix);
 template <typename T>
 int slice_segment(const T* M, int rows, int K);
 
-// Slices the rows of X: row r is nseg segments of seg_len contiguous elements,
-// segment c at X + c * seg_stride + r * seg_len; s.K = nseg * seg_len.
+// Where the product of a data operand goes: the matrix (m x K, row-major, finite)
+// and Y, R, plane of sliced_gemm.  M == nullptr: a matrix operand.
 template <typename T>
-void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, cudaStream_t st,
-                long long& nl);
+struct SliceOut {
+  const T* M = nullptr;
+  T* Y = nullptr;
+  long long R = 1, plane = 0;
+  int m = 0;
+};
+
+// Slices the rows of X: row r is nseg segments of seg_len contiguous elements,
+// segment c at X + c * seg_stride + r * seg_len; s.K = nseg * seg_len.  Rows with
+// an Inf have no digits: their results are written here, to o.Y (not X).
+template <typename T>
+void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, const SliceOut<T>& o,
+                cudaStream_t st, long long& nl);
 
 // Y[c][i][r] = sum_k M[i][k] X[(c, r)][k] for the sliced operands x (rows =
 // planes * R) and m (rows = output indices i), c = row / R; plane: elements

@@ -1,4 +1,4 @@
-"""FP64 sliced products with data whose digits are in line with the matrix's, so
+"""FP64 sliced products at their bounds and beyond: infinities, and data whose digits are in line with the matrix's, so
 that the digit sums come near their bounds, against extended precision.
 
 Tolerance: that of test_gpu_sliced.py (each operand entry cut at 2^-55 of its
@@ -88,4 +88,44 @@ def test_exact_sums_round_once(fc, n, terms):
         for i in np.flatnonzero(ok[r])[:40]:
             t = sum(Fraction(float(X[r, c])) * Fraction(float(M[i, c])) for c in k)
             assert abs(Fraction(float(Y[r, i])) - t) <= abs(t) * Fraction(257, 256) / 2 ** 53
+    s.close()
+
+
+@pytest.mark.parametrize("prec,ns", [("fp64", [40, 24]), ("fp64", [134, 9]), ("bf16x3", [264, 16]), ("bf16x3", [1040, 8])])
+def test_infinities_keep_their_sign(fc, prec, ns):
+    """A row with infinities gives what the sum gives: +-Inf by the matrix entry's
+    sign, NaN where infinities of both signs meet or a zero entry does."""
+    s = fc.Solver(ns, [(-4.0, 4.0)] * 2, [1.3, 1.7], 1.0, 0.4, 0.5, 1.0, 0.2, precision=prec)
+    f64 = prec == "fp64"
+    dt, pad = (np.float64, 4) if f64 else (np.float32, 8)
+    p = (ns[0] + pad - 1) // pad * pad
+    R = fc.fcgle_internal_elems(s.h) // p
+
+    def product(X):
+        Xd = torch.from_numpy(np.ascontiguousarray(X)).cuda().reshape(-1)
+        Y = torch.full_like(Xd, 7.0)
+        fc.fcgle_mode_product(s.h, 0, 1 if f64 else 5, Xd, Y)
+        s.sync()
+        return Y.reshape(2, p, R).permute(0, 2, 1).reshape(2 * R, p).cpu().numpy()
+
+    cols = []
+    for k0 in range(0, p, 2 * R):
+        E = np.zeros((2 * R, p), dt)
+        m = min(2 * R, p - k0)
+        E[np.arange(m), k0 + np.arange(m)] = 1.0
+        cols.append(product(E)[:m])
+    M = np.concatenate(cols).T
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((2 * R, p)).astype(dt)
+    X[:, ns[0]:] = 0.0
+    want = product(X)
+    bad = {2: {5: np.inf}, 3: {7: -np.inf}, 5: {0: np.inf, 9: np.inf}, 6: {1: np.inf, 2: -np.inf},
+           2 * R - 1: {ns[0] - 1: np.inf}, 9: {3: np.inf, 4: np.nan}}
+    for r, e in bad.items():
+        for k, v in e.items():
+            X[r, k] = v
+        with np.errstate(invalid="ignore"):
+            want[r] = sum(M[:, k] * dt(v) for k, v in e.items())
+    Y = product(X)
+    assert np.array_equal(Y, want, equal_nan=True)
     s.close()
