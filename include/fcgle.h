@@ -131,6 +131,11 @@ typedef struct fcgle_ctx* fcgle_handle;
  * For BF16X3 handles the setup also runs the kernel autotuner (see
  * fcgle_autotune_report) on that stream for problem shapes this process has
  * not tuned yet, and waits for it; do not call it during a stream capture.
+ * Device memory per internal element (P of fcgle_internal_elems): FP64 220
+ * bytes (12 tensors, and 28 bytes for the digits of the products), and 16 more
+ * for every spectral function f(theta Lam) in use and every source term; BF16X3
+ * 96 bytes (8 FP32 and 4 split tensors) and 8 per source term; besides, some
+ * tens of bytes per entry of the matrices Q_mu.
  * On success *out owns everything; release it with fcgle_destroy. */
 fcgle_status fcgle_setup(const fcgle_params* params, void* cuda_stream, fcgle_handle* out);
 

@@ -156,17 +156,19 @@ class Engine : public EngineBase {
         ms_[mu][1].build(mf64_[mu][1]->ptr, Mb, D.p, st_, launches);
       }
     }
-    // ---- workspace for the digits of the data
+    // ---- workspace for the digits of the data, 28 bytes per grid point, and their
+    // exponents; apply_f and norm work in tensors of the schemes, so that a handle
+    // holds 12 tensors and this
     if (xbytes) {
-      xdig_.reset(new DevBuf<uint8_t>(xbytes));
-      xex_.reset(new DevBuf<int>((size_t)xrows));
+      xbytes = (xbytes + 255) / 256 * 256;
+      xdig_.reset(new DevBuf<uint8_t>(xbytes + (size_t)xrows * sizeof(int)));
     }
     for (int mu = 0; mu < prm.d; ++mu)
       for (int cx = 0; cx < 2; ++cx) {
         Sliced& x = xs_[mu][cx];
         if (!sliceable(x.K, x.rows)) continue;
         x.dig = reinterpret_cast<__nv_bfloat16*>(xdig_->ptr);
-        x.ex = xex_->ptr;
+        x.ex = reinterpret_cast<int*>(xdig_->ptr + xbytes);
         slice_map<double>(x, false);
       }
     lv_.c_re = prm.nu;
@@ -245,8 +247,8 @@ class Engine : public EngineBase {
 
   // ------------------------------------------------------------ apply_f
   void apply_f(int func, int k, double theta, const void* v, void* out) override {
-    T* X = B(0);
-    T* Xh = B(1);
+    T* X = B(kS);
+    T* Xh = B(kFh);
     pack<T>(s_, (const T*)v, X, st_, launches);
     if (func == FCGLE_F_EXP || (func == FCGLE_F_PHI && k == 0)) {
       expK(theta, X, X);
@@ -367,7 +369,7 @@ class Engine : public EngineBase {
   }
 
   double norm(const void* u) override {
-    T* X = B(0);
+    T* X = B(kS);
     pack<T>(s_, (const T*)u, X, st_, launches);
     sumsq<T>(s_, X, scratch_->ptr, st_, launches);
     double h = 0.0;
@@ -380,8 +382,7 @@ class Engine : public EngineBase {
 
  private:
   // buffer roles
-  enum { kU = 2, kUh = 3, kG = 4, kGh = 5, kFh = 6, kD2 = 7, kD3 = 8, kD4 = 9, kS = 10, kW = 11, kT0 = 12, kT1 = 13,
-         kNumBuf = 14 };
+  enum { kU = 0, kUh, kG, kGh, kFh, kD2, kD3, kD4, kS, kW, kT0, kT1, kNumBuf };
   T* B(int i) { return buf_[i]->ptr; }
 
   static bool needs_uhat(int scheme) { return scheme == FCGLE_ETD2RK || scheme == FCGLE_KROGSTAD; }
@@ -759,7 +760,6 @@ class Engine : public EngineBase {
   SlicedMat ms_[kMaxDim][2];
   Sliced xs_[kMaxDim][2];   // digits of the data as direction mu's product reads them (real, complex block form)
   std::unique_ptr<DevBuf<uint8_t>> xdig_;
-  std::unique_ptr<DevBuf<int>> xex_;
   std::unique_ptr<DevBuf<T>> adj_mem_;   // storage of the adjoint, adj_size_ elements
   size_t adj_size_ = 0, adj_used_ = 0;
 };

@@ -420,20 +420,22 @@ class EngineB3 : public EngineBase {
     gs_.zeta = (float)prm.zeta;
     gs_.nsrc = 0;
     for (int i = 0; i < kNumF32; ++i) {
-      f32_[i].reset(new DevMem<float>(2 * s_.P));
-      FCGLE_CUDA(cudaMemsetAsync(f32_[i]->ptr, 0, 2 * s_.P * 4, st_));
+      // kD3 and kEA in one piece where the sliced products use them (below)
+      const bool pair = use_sliced() && i == kD3, second = use_sliced() && i == kEA;
+      if (!second) f32_[i].reset(new DevMem<float>((pair ? 4 : 2) * s_.P));
+      f32p_[i] = second ? f32p_[kD3] + 2 * s_.P : f32_[i]->ptr;
+      FCGLE_CUDA(cudaMemsetAsync(f32p_[i], 0, 2 * s_.P * 4, st_));
     }
     if (use_sliced()) {
-      // digits [3][2 R][p] bf16 = 12 P bytes of one direction at a time, then 2 R exponents
-      size_t rows = 0;
-      for (int mu = 0; mu < prm.d; ++mu) rows = std::max(rows, 2 * s_.P / (size_t)s_.p[mu]);
-      xdig_.reset(new DevMem<__nv_bfloat16>(6 * s_.P));
-      xex_.reset(new DevMem<int>(rows));
+      // digits [3][2 R][p] bf16 = 12 P bytes of one direction at a time, then 2 R
+      // exponents (at most P / 2 bytes, p >= 16), in the 16 P bytes of kD3 and kEA:
+      // no scheme holds anything there while a precise operator runs, and none reads
+      // them before it has written them whole, so the digits cost no memory
       for (int mu = 0; mu < prm.d; ++mu) {
         if (!sliceable(mu)) continue;
         Sliced& x = xs_[mu];
-        x.dig = xdig_->ptr;
-        x.ex = xex_->ptr;
+        x.dig = reinterpret_cast<__nv_bfloat16*>(F32(kD3));
+        x.ex = reinterpret_cast<int*>(F32(kD3) + 3 * s_.P);
         x.rows = 2 * (P_ / s_.p[mu]);
         x.K = s_.p[mu];
         slice_map<float>(x, false);
@@ -783,7 +785,7 @@ class EngineB3 : public EngineBase {
     CUtensorMap tm_hi64, tm_lo64;   // the same hi / lo in 32-wide, 64-byte-swizzled boxes (slab-fused product)
   };
 
-  float* F32(int i) { return f32_[i]->ptr; }
+  float* F32(int i) { return f32p_[i]; }
   uint32_t P32() const { return (uint32_t)s_.P; }
   SplitOut SP(int i) { return SplitOut{sp_[i]->ptr, sp_[i]->ptr + 2 * s_.P}; }
 
@@ -1688,10 +1690,9 @@ class EngineB3 : public EngineBase {
   b3::GStatic gs_{};
   double sig_re_[kMaxSrc] = {0, 0, 0, 0}, sig_im_[kMaxSrc] = {0, 0, 0, 0};
   std::unique_ptr<DevMem<float>> f32_[kNumF32];
-  // digits of the data as direction mu's sliced product reads them, and their buffers
+  float* f32p_[kNumF32] = {};
+  // digits of the data as direction mu's sliced product reads them
   Sliced xs_[kMaxDim];
-  std::unique_ptr<DevMem<__nv_bfloat16>> xdig_;
-  std::unique_ptr<DevMem<int>> xex_;
   std::unique_ptr<DevMem<__nv_bfloat16>> sp_[kNumSplit];
   std::unique_ptr<DevMem<float>> src_[kMaxSrc];
   std::unique_ptr<DevMem<float>> host_stage_;
