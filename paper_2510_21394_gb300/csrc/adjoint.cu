@@ -54,7 +54,7 @@ struct GP {
 };
 
 template <typename T>
-__global__ void misfit_kernel(size_t P, const T* __restrict__ u, const T* __restrict__ tg, T* __restrict__ lam,
+__global__ void misfit_kernel(size_t P, const T* u, const T* tg, T* __restrict__ lam,
                               double* acc) {
   pdl_enter();
   double v[1] = {0.0};
@@ -87,7 +87,7 @@ __device__ __forceinline__ void gpar(double zr, double zi, double wr, double wi,
 }
 
 template <typename T>
-__global__ void gv_kernel(size_t P, GP g, const T* __restrict__ z, const T* __restrict__ w, double c,
+__global__ void gv_kernel(size_t P, GP g, const T* z, const T* w, double c,
                           T* __restrict__ mu, double* acc) {
   pdl_enter();
   double v[3] = {0.0, 0.0, 0.0};
@@ -122,7 +122,7 @@ __device__ __forceinline__ bool lam_sum(const LD& L, size_t q, double& s) {
 }
 
 template <typename T>
-__global__ void spec_dot_kernel(size_t P, LD L, const T* __restrict__ x, const T* __restrict__ y, double* acc) {
+__global__ void spec_dot_kernel(size_t P, LD L, const T* x, const T* y, double* acc) {
   pdl_enter();
   double v[2] = {0.0, 0.0};
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
@@ -136,7 +136,7 @@ __global__ void spec_dot_kernel(size_t P, LD L, const T* __restrict__ x, const T
 }
 
 template <typename T>
-__global__ void axpby_kernel(size_t n, double a, const T* __restrict__ x1, double b, const T* __restrict__ x2,
+__global__ void axpby_kernel(size_t n, double a, const T* x1, double b, const T* x2,
                              T* __restrict__ y) {
   pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x)
@@ -159,8 +159,8 @@ __device__ __forceinline__ void exp_z(const LD& L, size_t q, double cre, double 
 // y1 = e^z (x + c1 k), y2 = e^z (x + c2 k): the two stage values of a
 // Lawson-RK2 step (V^ and W^), one pass over x and k
 template <typename T>
-__global__ void exp_pair_kernel(size_t P, LD L, double cre, double cim, const T* __restrict__ x,
-                                const T* __restrict__ k, double c1, double c2, T* __restrict__ y1, T* __restrict__ y2) {
+__global__ void exp_pair_kernel(size_t P, LD L, double cre, double cim, const T* x,
+                                const T* k, double c1, double c2, T* __restrict__ y1, T* __restrict__ y2) {
   pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
     double er, ei;
@@ -179,7 +179,7 @@ __global__ void exp_pair_kernel(size_t P, LD L, double cre, double cim, const T*
 // a = e^{z} x, b = e^{z} m (z already conjugated by the caller):
 // y = ca a + cb b and sum = a + b, one pass; y may alias x
 template <typename T>
-__global__ void exp_combo_kernel(size_t P, LD L, double cre, double cim, const T* x, const T* __restrict__ m,
+__global__ void exp_combo_kernel(size_t P, LD L, double cre, double cim, const T* x, const T* m,
                                  double ca, double cb, T* y, T* __restrict__ sum) {
   pdl_enter();
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {
@@ -262,7 +262,7 @@ __device__ __forceinline__ void gadj_f(float gam, float kap, float zet, float zr
   oi = ar * wi - ai * wr + bi * wr - br * wi;
 }
 
-__global__ void gv_kernel_f(uint32_t P, GP g, const float* __restrict__ z, const float* __restrict__ w, float c,
+__global__ void gv_kernel_f(uint32_t P, GP g, const float* z, const float* w, float c,
                             float* __restrict__ mu, AdjSplit sp, double* acc) {
   pdl_enter();
   float f[3] = {0.f, 0.f, 0.f};
@@ -316,8 +316,8 @@ __device__ __forceinline__ void expm1_z_f(const Quad& Q, int v, float ar, float 
 }
 
 // y1 = e^z (x + c1 k), y2 = e^z (x + c2 k) (FP32 form of exp_pair_kernel)
-__global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const float* __restrict__ x,
-                                  const float* __restrict__ k, float c1, float c2, float* __restrict__ y1,
+__global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const float* x,
+                                  const float* k, float c1, float c2, float* __restrict__ y1,
                                   float* __restrict__ y2, AdjSplit sp) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
@@ -350,7 +350,7 @@ __global__ void exp_pair_kernel_f(uint32_t P, LD L, float ar, float ai, const fl
 }
 
 // a = e^z x, b = e^z m; y = ca a + cb b, sum = a + b (FP32 form of exp_combo_kernel; y may alias x)
-__global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const float* x, const float* __restrict__ m,
+__global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const float* x, const float* m,
                                    float ca, float cb, float* y, float* __restrict__ sum, AdjSplit sp) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
@@ -382,7 +382,7 @@ __global__ void exp_combo_kernel_f(uint32_t P, LD L, float ar, float ai, const f
   }
 }
 
-__global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* __restrict__ x, const float* __restrict__ y,
+__global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* x, const float* y,
                                   double* acc) {
   pdl_enter();
   float f[2] = {0.f, 0.f};
@@ -404,8 +404,8 @@ __global__ void spec_dot_kernel_f(uint32_t P, LD L, const float* __restrict__ x,
   block_acc<2>(v, acc, ADJ_Z_RE);
 }
 
-__global__ void axpby_kernel_f(uint32_t n, float a, const float* __restrict__ x1, float b,
-                               const float* __restrict__ x2, float* __restrict__ y, AdjSplit sp) {
+__global__ void axpby_kernel_f(uint32_t n, float a, const float* x1, float b,
+                               const float* x2, float* __restrict__ y, AdjSplit sp) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float u[4], w[4] = {0.f, 0.f, 0.f, 0.f};

@@ -47,7 +47,7 @@ __device__ __forceinline__ void ldv(const float* p, float (&o)[V]) {
   }
 }
 template <int V>
-__device__ __forceinline__ void ldv_ro(const float* p, float (&o)[V]) {   // read-only operands
+__device__ __forceinline__ void ldv_ro(const float* p, float (&o)[V]) {   // constants of the handle (see pdl.cuh)
   if constexpr (V == 4) {
     const float4 x = __ldg(reinterpret_cast<const float4*>(p));
     o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
@@ -160,8 +160,8 @@ __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_
       }
     }
     if (!have) {
-      ldv_ro<V>(g.S[k] + q, sr);
-      ldv_ro<V>(g.S[k] + P + q, si);
+      ldv<V>(g.S[k] + q, sr);
+      ldv<V>(g.S[k] + P + q, si);
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) {

@@ -247,7 +247,7 @@ float tf32_rna_host(float x) {
 // (P is a multiple of 8: every kernel handles 4 consecutive elements per step)
 
 // V = a u + b g(t, u) (split); optionally V2 = a2 u + b2 g(t, u) (split)
-__global__ void gsplit_kernel(uint32_t P, b3::GStatic g, b3::GTime t, const float* __restrict__ U, float a, float b,
+__global__ void gsplit_kernel(uint32_t P, b3::GStatic g, b3::GTime t, const float* U, float a, float b,
                               SplitOut V, float a2, float b2, SplitOut V2) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
@@ -274,7 +274,7 @@ __global__ void gsplit_kernel(uint32_t P, b3::GStatic g, b3::GTime t, const floa
 
 // V = Phi_t(u) (split)
 // U = Phi_t(W)
-__global__ void flow_kernel(uint32_t P, b3::Flow f, const float* __restrict__ W, float* __restrict__ U) {
+__global__ void flow_kernel(uint32_t P, b3::Flow f, const float* W, float* __restrict__ U) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float wr[4], wi[4], ur[4], ui[4];
@@ -288,7 +288,7 @@ __global__ void flow_kernel(uint32_t P, b3::Flow f, const float* __restrict__ W,
 }
 
 // V = Phi_t(u) -> split (Strang's first half step, Kronecker-product form)
-__global__ void flow_split_kernel(uint32_t P, b3::Flow f, const float* __restrict__ U, SplitOut V) {
+__global__ void flow_split_kernel(uint32_t P, b3::Flow f, const float* U, SplitOut V) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float ur[4], ui[4], vr[4], vi[4];
@@ -301,7 +301,7 @@ __global__ void flow_split_kernel(uint32_t P, b3::Flow f, const float* __restric
 }
 
 // V = Phi_t(u) - u -> split (Strang's first half step as an increment)
-__global__ void flow_incr_split_kernel(uint32_t P, b3::Flow f, const float* __restrict__ U, SplitOut V) {
+__global__ void flow_incr_split_kernel(uint32_t P, b3::Flow f, const float* U, SplitOut V) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < P; q += 4 * gridDim.x * blockDim.x) {
     float ur[4], ui[4], vr[4], vi[4];
@@ -314,7 +314,7 @@ __global__ void flow_incr_split_kernel(uint32_t P, b3::Flow f, const float* __re
 }
 
 // FP32 -> split-TF32: hi = tf32(x), lo = tf32(x - hi); n % 4 == 0
-__global__ void tf32_split_kernel(uint32_t n, const float* __restrict__ X, float* __restrict__ hi,
+__global__ void tf32_split_kernel(uint32_t n, const float* X, float* __restrict__ hi,
                                   float* __restrict__ lo) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
@@ -331,7 +331,7 @@ __global__ void tf32_split_kernel(uint32_t n, const float* __restrict__ X, float
 }
 
 // FP32 -> split (raw mode-product entry point); n % 4 == 0
-__global__ void to_split_kernel(uint32_t n, const float* __restrict__ X, SplitOut Y) {
+__global__ void to_split_kernel(uint32_t n, const float* X, SplitOut Y) {
   pdl_enter();
   for (uint32_t q = 4 * (blockIdx.x * blockDim.x + threadIdx.x); q < n; q += 4 * gridDim.x * blockDim.x) {
     float x[4];

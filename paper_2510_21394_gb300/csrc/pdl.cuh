@@ -9,6 +9,12 @@ namespace fcgle {
 // has completed and its writes are visible (pdl_wait) before it touches global
 // memory that another kernel writes.  The wait ends when that kernel ends;
 // without the launch attribute both are no-ops.
+//
+// Such a kernel is alive while its predecessors still write, so it must not read
+// their results through the read-only path (ld.global.nc, which is defined only
+// for data that nothing writes during the kernel): neither __ldg nor const
+// __restrict__ parameters, from which the compiler may make the same loads.
+// Constants of the handle, complete before setup returns, may be read so.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {

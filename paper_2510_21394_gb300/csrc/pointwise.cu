@@ -102,7 +102,7 @@ __device__ __forceinline__ void st4_split(__nv_bfloat16* hi, __nv_bfloat16* lo, 
 
 // SPLIT: the values go to hi and lo instead of X
 template <typename T, bool SPLIT>
-__global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__ X, __nv_bfloat16* __restrict__ hi,
+__global__ void pack_kernel(Shape s, const T* user, T* __restrict__ X, __nv_bfloat16* __restrict__ hi,
                             __nv_bfloat16* __restrict__ lo) {
   pdl_enter();
   const size_t P = s.P, quads_per_row = (size_t)s.p[0] / 4, nq = P / 4;
@@ -147,7 +147,7 @@ __global__ void pack_kernel(Shape s, const T* __restrict__ user, T* __restrict__
 }
 
 template <typename T>
-__global__ void unpack_kernel(Shape s, const T* __restrict__ X, T* __restrict__ user, int* __restrict__ nonfinite) {
+__global__ void unpack_kernel(Shape s, const T* X, T* __restrict__ user, int* __restrict__ nonfinite) {
   pdl_enter();
   const size_t P = s.P, quads_per_row = (size_t)s.p[0] / 4, nq = P / 4;
   const int n1 = s.n[0];
@@ -197,8 +197,8 @@ struct GDev {
 // not have is left out at compile time.  128 x 120 x 136: g(u) alone 102 -> 45 us.
 enum { GC_X1 = 1, GC_UNIT = 2, GC_A = 4, GC_B = 8, GC_X2 = 16 };   // X1; c0 = c1 = 1; a0, a1 terms; b != 1; X2
 template <typename T, int F>
-__global__ void gcombo_kernel(size_t P, GDev g, const T* __restrict__ X0, const T* __restrict__ X1,
-                              const T* __restrict__ X2, double c0, double c1, double a0, double a1, double b,
+__global__ void gcombo_kernel(size_t P, GDev g, const T* X0, const T* X1,
+                              const T* X2, double c0, double c1, double a0, double a1, double b,
                               double e, T* __restrict__ out) {
   pdl_enter();
   const size_t nv = P / 4;
@@ -483,7 +483,7 @@ __global__ void fill_F_kernel(size_t P, LamDev L, Shape s, int func, int ell, do
 // ------------------------------------------------------------ exact flow
 template <typename T>
 __global__ void exact_flow_kernel(size_t P, double gamma, double kappa, double zeta, double t, double tp1,
-                                  const T* __restrict__ X, T* __restrict__ Y) {
+                                  const T* X, T* __restrict__ Y) {
   pdl_enter();
   // w(t) = exp(t gamma - (kappa + i zeta)/(2 kappa) log(1 + 2 t phi_1(2 gamma t) kappa |w0|^2)) w0
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < P; q += (size_t)gridDim.x * blockDim.x) {

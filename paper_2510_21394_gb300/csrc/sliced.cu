@@ -156,7 +156,7 @@ __device__ __noinline__ void infinite_rows(const T* X, long long rows, int nseg,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
+__global__ void __launch_bounds__(256) slice_kernel(const T* X, long long rows, int nseg, int seg_len,
                                                     long long seg_stride, int pitch, int group,
                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
                              const __grid_constant__ SliceOut<T> o) {
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* __restrict__ X, lon
 // and stores 16 bytes per digit (FP32 at 432^3: 473 us with 4-element pieces read
 // twice, 303 this way = 5.3 TB/s; FP64 at 128 x 120 x 136: 25 -> 20 us).
 template <typename T, int IT>
-__global__ void __launch_bounds__(256) slice8_kernel(const T* __restrict__ X, long long rows, int nseg, int seg_len,
+__global__ void __launch_bounds__(256) slice8_kernel(const T* X, long long rows, int nseg, int seg_len,
                                                      long long seg_stride, int pitch, int group,
                                                      __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
                              const __grid_constant__ SliceOut<T> o) {
@@ -427,7 +427,7 @@ __device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei) {
 template <typename T, bool SEG>
 __global__ void __launch_bounds__(kGThreads, 1)
     sliced_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_m,
-                       const int* __restrict__ ex, const int* __restrict__ em, T* __restrict__ Y,
+                       const int* ex, const int* __restrict__ em, T* __restrict__ Y,
                        const GemmParams gp) {
   using L = GemmLayout<T>;
   constexpr int NS = SliceCfg<T>::NS, NLEV = GemmCfg<T>::NLEV, NT = GemmCfg<T>::NT, NSTAGE = GemmCfg<T>::NSTAGE;
