@@ -269,21 +269,25 @@ __device__ __forceinline__ void phi123(float zr, float zi, float (&pr)[3], float
 // fixed and s the real eigenvalue sum of the element, so the series of phi_3
 // becomes a polynomial in the real s with complex coefficients
 // c_m = w^m / (m+3)! (computed on the host in FP64) and each Horner step costs
-// two FMAs instead of a complex multiply-add.  |z| >= 1 (|s| >= smax) takes
-// the recurrence branch of phi123.
+// two FMAs instead of a complex multiply-add.  w^9 leaves the range of FP32 for
+// |w| below 1e-4 or above 1e5, so the polynomial is in x = 2^k s with
+// c_m = (w / 2^k)^m / (m+3)!, 2^k next to |w|; a power of two changes no rounding.
+// |z| >= 1 (|s| >= smax) takes the recurrence branch of phi123.
 struct PhiPoly {
   float cr[10] = {0}, ci[10] = {0};
   float smax = 0.f;
+  float scale = 1.f;   // 2^k
   float wr = 0.f, wi = 0.f;
 };
 __device__ __forceinline__ void phi123_s(const PhiPoly& P, float s, float (&pr)[3], float (&pi)[3]) {
   const float zr = P.wr * s, zi = P.wi * s;
   if (fabsf(s) < P.smax) {
+    const float x = P.scale * s;
     float ar = P.cr[9], ai = P.ci[9];
 #pragma unroll
     for (int m = 8; m >= 0; --m) {
-      ar = fmaf(ar, s, P.cr[m]);
-      ai = fmaf(ai, s, P.ci[m]);
+      ar = fmaf(ar, x, P.cr[m]);
+      ai = fmaf(ai, x, P.ci[m]);
     }
     pr[2] = ar;
     pi[2] = ai;

@@ -1468,16 +1468,19 @@ class EngineB3 : public EngineBase {
   b3::PhiPoly phipoly(double theta) const {
     b3::PhiPoly P;
     const std::complex<double> w(theta * prm_.nu, theta * prm_.eta);
+    const double aw = std::abs(w);
+    const int k = aw > 0.0 ? std::max(-126, std::min(126, std::ilogb(aw))) : 0;
+    const std::complex<double> v(std::ldexp(w.real(), -k), std::ldexp(w.imag(), -k));
     std::complex<double> wm(1.0, 0.0);
     double fact = 6.0;   // (m + 3)! at m = 0
     for (int m = 0; m < 10; ++m) {
       const std::complex<double> c = wm / fact;
       P.cr[m] = (float)c.real();
       P.ci[m] = (float)c.imag();
-      wm *= w;
+      wm *= v;
       fact *= (double)(m + 4);
     }
-    const double aw = std::abs(w);
+    P.scale = (float)std::ldexp(1.0, k);
     P.smax = aw > 0.0 ? (float)(1.0 / aw) : 3.0e38f;
     P.wr = (float)w.real();
     P.wi = (float)w.imag();
