@@ -355,7 +355,9 @@ fcgle_status fcgle_internal_elems(fcgle_handle h, size_t* P);
  * handles, d >= 2, R % 8 == 0, with bit 1, direction d-1): the product above
  * with X read in the natural order, X[c][k][r] (direction mu slowest); Y as
  * above.  Other flag bits or combinations give FCGLE_ERR_INVALID_ARG.  X and
- * Y must not overlap.  direction in 0..d-1. */
+ * Y must not overlap.  They are aligned to 16 bytes, FP64 handles and the
+ * precise product beyond split-TF32 to one element; FCGLE_ERR_INVALID_ARG
+ * otherwise.  direction in 0..d-1. */
 fcgle_status fcgle_mode_product(fcgle_handle h, int direction, int flags, const void* X, void* Y);
 
 /* The kernel autotuner (a library facility, not a step of the method).  The

@@ -193,6 +193,7 @@ class Engine : public EngineBase {
   size_t internal_elems() const override { return s_.P; }
   void mode_product(int mu, bool fwd, const void* X, void* Y) override {
     if (mu < 0 || mu >= s_.d) throw InvalidArg("direction must be in 0..d-1");
+    check_aligned(X, Y, sizeof(T));
     mp((const T*)X, (T*)Y, mu, fwd);
   }
   size_t elem_bytes() const override { return 2 * sizeof(T); }

@@ -34,6 +34,12 @@ struct Direction {
   std::vector<double> lam;   // n eigenvalues of D_mu (negative)
 };
 
+// The buffers of a raw mode product, at the alignment its kernel's accesses need.
+inline void check_aligned(const void* X, const void* Y, size_t bytes) {
+  if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & (bytes - 1))
+    throw InvalidArg("X and Y must be aligned to " + std::to_string(bytes) + " bytes");
+}
+
 class EngineBase {
  public:
   virtual ~EngineBase() = default;

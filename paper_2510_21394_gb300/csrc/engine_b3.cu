@@ -587,7 +587,9 @@ class EngineB3 : public EngineBase {
       // the precise form of the end transforms: FP32 planar in and out
       if (flags & 2) throw InvalidArg("flags bits 1 and 2 exclude each other");
       const long long R = P_ / s_.p[mu];
-      if (s_.d >= 2 && R % 8 == 0 && s_.p[mu] <= kTf32MaxP) {
+      const bool tf32 = s_.d >= 2 && R % 8 == 0 && s_.p[mu] <= kTf32MaxP;
+      check_aligned(X, Y, tf32 ? 16 : sizeof(float));
+      if (tf32) {
         float *ah = F32(kFh), *al = F32(kD2);   // work tensors of the schemes, free here
         launch_pdl(tf32_split_kernel, grid_for(P_ / 2), 256, 0, st_, 2 * P32(), (const float*)X, ah, al);
         FCGLE_LAUNCHED(launches);
@@ -597,6 +599,7 @@ class EngineB3 : public EngineBase {
       }
       return;
     }
+    check_aligned(X, Y, 16);
     if (flags & 24) {
       // natural-order forms (split input and output)
       if (!(flags & 2)) throw InvalidArg("flags bits 3 and 4 need the split form (bit 1)");

@@ -114,8 +114,9 @@ void mp_f64(const double* X, double* Y, const double* M, int p, size_t R, bool c
 
 // FP32 REAL mode with larger register tiles: 128 x 128 block tile, 8 x 8
 // outputs per thread, K in steps of 8 through double-buffered shared memory.
-// Needs p % 8 == 0 and R % 8 == 0 (then a thread's 8 rows never straddle the
-// re/im plane boundary and its stores are 16-byte vectors).
+// Needs p % 8 == 0, R % 8 == 0 and 16-byte aligned X and Y (then a thread's 8 rows
+// never straddle the re/im plane boundary, and its loads and stores are 16-byte
+// vectors); the element-wise kernel above takes the rest.
 constexpr int FM = 128, FN = 128, FK = 8, FT = 256;
 
 __global__ void __launch_bounds__(FT) mp_f32_kernel(const float* __restrict__ X, float* __restrict__ Y,
@@ -197,7 +198,8 @@ __global__ void __launch_bounds__(FT) mp_f32_kernel(const float* __restrict__ X,
 
 void mp_f32(const float* X, float* Y, const float* M, int p, size_t R, cudaStream_t st, long long& nl) {
   const long long rows = 2 * (long long)R;
-  if (p % 8 == 0 && R % 8 == 0) {
+  const bool aligned = ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
+  if (p % 8 == 0 && R % 8 == 0 && aligned) {
     dim3 grid((unsigned)((rows + FM - 1) / FM), (unsigned)((p + FN - 1) / FN));
     mp_f32_kernel<<<grid, FT, 0, st>>>(X, Y, M, p, (long long)R);
   } else {
