@@ -139,15 +139,17 @@ __device__ __forceinline__ void lds16(uint32_t src, float (&v)[4]) {
                : "memory");
 }
 
+// The contractions are spelled out: left to the compiler they depend on how the
+// functor around is built, and a grouped launch would not give the bits of a single one.
 template <int V>
 __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_t P, uint32_t q, const float (&ur)[V],
                                        const float (&ui)[V], float (&gr)[V], float (&gi)[V],
                                        const SrcIn& src = SrcIn{}) {
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    const float m2 = ur[v] * ur[v] + ui[v] * ui[v];
-    gr[v] = g.gamma * ur[v] - m2 * (g.kappa * ur[v] - g.zeta * ui[v]);
-    gi[v] = g.gamma * ui[v] - m2 * (g.kappa * ui[v] + g.zeta * ur[v]);
+    const float m2 = fmaf(ur[v], ur[v], __fmul_rn(ui[v], ui[v]));
+    gr[v] = fmaf(g.gamma, ur[v], -__fmul_rn(m2, fmaf(g.kappa, ur[v], -__fmul_rn(g.zeta, ui[v]))));
+    gi[v] = fmaf(g.gamma, ui[v], -__fmul_rn(m2, fmaf(g.kappa, ui[v], __fmul_rn(g.zeta, ur[v]))));
   }
   for (int k = 0; k < g.nsrc; ++k) {
     float sr[V], si[V];
@@ -165,8 +167,8 @@ __device__ __forceinline__ void g_eval(const GStatic& g, const GTime& t, uint32_
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      gr[v] += t.e_re[k] * sr[v] - t.e_im[k] * si[v];
-      gi[v] += t.e_re[k] * si[v] + t.e_im[k] * sr[v];
+      gr[v] = fmaf(t.e_re[k], sr[v], fmaf(-t.e_im[k], si[v], gr[v]));
+      gi[v] = fmaf(t.e_re[k], si[v], fmaf(t.e_im[k], sr[v], gi[v]));
     }
   }
 }
@@ -442,8 +444,8 @@ struct EpiUpdateG {
     if (b != 0.f) g_eval<V>(g, t, P, q, ur, ui, gr, gi, src);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      vr[v] = a * ur[v] + b * gr[v];
-      vi[v] = a * ui[v] + b * gi[v];
+      vr[v] = fmaf(a, ur[v], __fmul_rn(b, gr[v]));
+      vi[v] = fmaf(a, ui[v], __fmul_rn(b, gi[v]));
     }
     emit_csplit<V>(em, Vout, P, q, vr, vi);
   }
