@@ -15,8 +15,9 @@
 //   kLam       the functor needs the eigenvalue sums (member L),
 //   kG         the functor evaluates g (member g; its source terms are fetched
 //              like operands),
-//   store<V>(q, sv, re, im, in, src, em): sv = eigenvalue sums of the V elements
-//              (kLam), in[2 k], in[2 k + 1] = operand k, src = source values;
+//   store<V, SH>(q, sv, re, im, in, src, em): sv = eigenvalue sums of the V elements
+//              (kLam), in[2 k], in[2 k + 1] = operand k, src = source values, SH: the
+//              phi polynomial is in shared memory at src.ph;
 //              writes its FP32 outputs and leaves the split one in em,
 //   split()    where the split output goes (hi == nullptr: none).
 // (The plain split product without a pointwise stage is b3_plain.cuh.)
@@ -131,6 +132,7 @@ struct GTime {
 struct SrcIn {
   uint32_t addr = 0;
   int n = 0;
+  uint32_t ph = 0;   // grouped launches: shared address of this problem's phi polynomial
 };
 __device__ __forceinline__ void lds16(uint32_t src, float (&v)[4]) {
   asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
@@ -275,32 +277,85 @@ __device__ __forceinline__ void phi123(float zr, float zi, float (&pr)[3], float
 // |w| below 1e-4 or above 1e5, so the polynomial is in x = 2^k s with
 // c_m = (w / 2^k)^m / (m+3)!, 2^k next to |w|; a power of two changes no rounding.
 // |z| >= 1 (|s| >= smax) takes the recurrence branch of phi123.
-struct PhiPoly {
-  float cr[10] = {0}, ci[10] = {0};
+struct alignas(16) PhiPoly {
+  float4 c[5] = {};   // c[j]: re, im of c_{2 j}, re, im of c_{2 j + 1}
   float smax = 0.f;
   float scale = 1.f;   // 2^k
   float wr = 0.f, wi = 0.f;
 };
+// phi_1 .. phi_3 from phi_3 = ar + i ai, |z| < 1
+__device__ __forceinline__ void phi_down(float zr, float zi, float ar, float ai, float (&pr)[3], float (&pi)[3]) {
+  pr[2] = ar;
+  pi[2] = ai;
+  pr[1] = zr * ar - zi * ai + 0.5f;
+  pi[1] = zr * ai + zi * ar;
+  pr[0] = zr * pr[1] - zi * pi[1] + 1.f;
+  pi[0] = zr * pi[1] + zi * pr[1];
+}
 __device__ __forceinline__ void phi123_s(const PhiPoly& P, float s, float (&pr)[3], float (&pi)[3]) {
   const float zr = P.wr * s, zi = P.wi * s;
   if (fabsf(s) < P.smax) {
     const float x = P.scale * s;
-    float ar = P.cr[9], ai = P.ci[9];
+    float ar = fmaf(P.c[4].z, x, P.c[4].x), ai = fmaf(P.c[4].w, x, P.c[4].y);
 #pragma unroll
-    for (int m = 8; m >= 0; --m) {
-      ar = fmaf(ar, x, P.cr[m]);
-      ai = fmaf(ai, x, P.ci[m]);
+    for (int j = 3; j >= 0; --j) {
+      ar = fmaf(fmaf(ar, x, P.c[j].z), x, P.c[j].x);
+      ai = fmaf(fmaf(ai, x, P.c[j].w), x, P.c[j].y);
     }
-    pr[2] = ar;
-    pi[2] = ai;
-    pr[1] = zr * ar - zi * ai + 0.5f;
-    pi[1] = zr * ai + zi * ar;
-    pr[0] = zr * pr[1] - zi * pi[1] + 1.f;
-    pi[0] = zr * pi[1] + zi * pr[1];
+    phi_down(zr, zi, ar, ai, pr, pi);
   } else {
     phi123(zr, zi, pr, pi);
   }
 }
+
+// The polynomials of V elements.  SH (grouped launches): from a copy of P in shared
+// memory at sm, read 16 bytes at a time for all V at once, so that its 24 words are
+// neither loaded per element nor held in registers; the same operations per element.
+template <int V, bool SH>
+struct PhiRay {
+  float ar[V], ai[V], smax, wr, wi;
+  __device__ __forceinline__ PhiRay(const PhiPoly&, uint32_t sm, const float (&s)[V]) {
+    const float4 t = lds4(sm + 80);
+    smax = t.x;
+    wr = t.z;
+    wi = t.w;
+    float x[V];
+    float4 c = lds4(sm + 64);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      x[v] = t.y * s[v];
+      ar[v] = fmaf(c.z, x[v], c.x);
+      ai[v] = fmaf(c.w, x[v], c.y);
+    }
+#pragma unroll
+    for (int j = 3; j >= 0; --j) {
+      c = lds4(sm + 16 * j);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        ar[v] = fmaf(fmaf(ar[v], x[v], c.z), x[v], c.x);
+        ai[v] = fmaf(fmaf(ai[v], x[v], c.w), x[v], c.y);
+      }
+    }
+  }
+  __device__ __forceinline__ static float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+  }
+  __device__ __forceinline__ void get(int v, float s, float (&pr)[3], float (&pi)[3]) const {
+    const float zr = wr * s, zi = wi * s;
+    if (fabsf(s) < smax)
+      phi_down(zr, zi, ar[v], ai[v], pr, pi);
+    else
+      phi123(zr, zi, pr, pi);
+  }
+};
+template <int V>
+struct PhiRay<V, false> {
+  const PhiPoly& P;
+  __device__ __forceinline__ PhiRay(const PhiPoly& p, uint32_t, const float (&)[V]) : P(p) {}
+  __device__ __forceinline__ void get(int, float s, float (&pr)[3], float (&pi)[3]) const { phi123_s(P, s, pr, pi); }
+};
 
 // phi_k(z), any k >= 1: Horner form of the series
 // (1/k!)(1 + z/(k+1)(1 + z/(k+2)(...))) for |z| < 1.5, recurrence otherwise.
@@ -370,7 +425,7 @@ struct EpiStoreSplitGen {
   SplitOut Y;
   __device__ SplitOut split() const { return Y; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     emit_csplit<V>(em, Y, P, q, re, im);
@@ -384,7 +439,7 @@ struct EpiStoreF32 {
   float* Y;
   __device__ SplitOut split() const { return SplitOut{}; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn&, SplitVal&) const {
     stv<V>(Y + q, re);
@@ -402,7 +457,7 @@ struct EpiScaleF {
   SplitOut Y;
   __device__ SplitOut split() const { return Y; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], yr[V], yi[V];
@@ -429,7 +484,7 @@ struct EpiUpdateG {
   SplitOut Vout;
   __device__ SplitOut split() const { return Vout; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn& src, SplitVal& em) const {
     float ur[V], ui[V], gr[V], gi[V], vr[V], vi[V];
@@ -462,7 +517,7 @@ struct EpiStageD {
   SplitOut D;
   __device__ SplitOut split() const { return D; }
   __device__ const float* src(int) const { return U; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float sr[V], si[V], g1r[V], g1i[V], g0r[V], g0i[V];
@@ -501,18 +556,19 @@ struct EpiFhat {
   PhiPoly ph;   // phi series coefficients of this launch (theta = theta)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return Uh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float lr[V], li[V], fr[V], fi[V], sr[V], si[V];
     lam_of<V>(L, sv, lr, li);
     cmulv<V>(lr, li, in[0], in[1], fr, fi);
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       fr[v] += re[v];
       fi[v] += im[v];
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       sr[v] = c * (pr[0] * fr[v] - pi[0] * fi[v]);
       si[v] = c * (pr[0] * fi[v] + pi[0] * fr[v]);
     }
@@ -546,16 +602,17 @@ struct EpiKrog2 {
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau / 2)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return Fh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     stv<V>(D2 + q, re);
     stv<V>(D2 + P + q, im);
     float sr[V], si[V];
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       const float ar = 0.5f * (pr[0] * in[0][v] - pi[0] * in[1][v]) + (pr[1] * re[v] - pi[1] * im[v]);
       const float ai = 0.5f * (pr[0] * in[1][v] + pi[0] * in[0][v]) + (pr[1] * im[v] + pi[1] * re[v]);
       sr[v] = tau * ar;
@@ -582,14 +639,15 @@ struct EpiKrog3 {
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int k) const { return k == 0 ? Fh : D2; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[4][V], const SrcIn& src, SplitVal& em) const {
     float sr[V], si[V], wr[V], wi[V];
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       const float fr = pr[0] * in[0][v] - pi[0] * in[1][v], fi = pr[0] * in[1][v] + pi[0] * in[0][v];
       sr[v] = tau * (fr + 2.f * (pr[1] * re[v] - pi[1] * im[v]));
       si[v] = tau * (fi + 2.f * (pr[1] * im[v] + pi[1] * re[v]));
@@ -618,14 +676,15 @@ struct EpiKrogFinal {
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int k) const { return k == 0 ? W : Uh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[4][V], const SrcIn& src, SplitVal& em) const {
     float sr[V], si[V], ur[V], ui[V];
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       const float cr = tau * (4.f * pr[2] - pr[1]), ci = tau * (4.f * pi[2] - pi[1]);
       sr[v] = in[0][v] + cr * re[v] - ci * im[v];
       si[v] = in[1][v] + cr * im[v] + ci * re[v];
@@ -651,14 +710,15 @@ struct EpiEtd2 {
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return Uh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float sr[V], si[V], ur[V], ui[V];
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       sr[v] = tau * (pr[1] * re[v] - pi[1] * im[v]);
       si[v] = tau * (pr[1] * im[v] + pi[1] * re[v]);
       ur[v] = in[0][v] + sr[v];
@@ -692,11 +752,12 @@ struct EpiSpecStep {
   PhiPoly ph;   // phi series coefficients of this launch (kind 1: theta = theta)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return Uh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float lr[V], li[V], ur[V], ui[V];
     lam_of<V>(L, sv, lr, li);
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float zr = theta * lr[v], zi = theta * li[v];
@@ -709,7 +770,7 @@ struct EpiSpecStep {
         mi = zr * fi + zi * fr;
       } else {
         float pr[3], pi[3];
-        phi123_s(ph, sv[v], pr, pi);
+        ray.get(v, sv[v], pr, pi);
         mr = zr * pr[0] - zi * pi[0];
         mi = zr * pi[0] + zi * pr[0];
         fr = 1.f + mr;
@@ -742,7 +803,7 @@ struct EpiLBDF2S {
   SplitOut S;
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int k) const { return k == 0 ? Uh : dU; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
                         const float (&in)[4][V], const SrcIn&, SplitVal& em) const {
     float lr[V], li[V], dr[V], di[V], ur[V], ui[V];
@@ -780,7 +841,7 @@ struct EpiExtrapG {
   SplitOut S;
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return U; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float er[V], ei[V], gr[V], gi[V];
@@ -811,16 +872,17 @@ struct EpiLRK2A {
   PhiPoly ph;   // phi series coefficients of this launch (theta = tau)
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return Uh; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&sv)[V], const float (&re)[V], const float (&im)[V],
-                        const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
+                        const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float lr[V], li[V], vr[V], vi[V], wr[V], wi[V];
     lam_of<V>(L, sv, lr, li);
+    const PhiRay<V, SH> ray(ph, src.ph, sv);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float zr = tau * lr[v], zi = tau * li[v];
       float pr[3], pi[3];
-      phi123_s(ph, sv[v], pr, pi);
+      ray.get(v, sv[v], pr, pi);
       const float mr = zr * pr[0] - zi * pi[0], mi = zr * pi[0] + zi * pr[0];   // e^z - 1
       const float fr = 1.f + mr, fi = mi;                           // e^z
       const float xr = in[0][v], xi = in[1][v];
@@ -848,7 +910,7 @@ struct EpiLRK2B {
   SplitOut S;
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return W; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&in)[2][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V];
@@ -907,7 +969,7 @@ struct EpiStrangB {
   SplitOut S;
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V], dr[V], di[V];
@@ -936,7 +998,7 @@ struct EpiStrangKron {
   SplitOut S;
   __device__ SplitOut split() const { return S; }
   __device__ const float* src(int) const { return nullptr; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&)[1][V], const SrcIn&, SplitVal& em) const {
     float ur[V], ui[V], sr[V], si[V];
@@ -966,7 +1028,7 @@ struct EpiLRK2Kron {
   SplitOut V1, V2;
   __device__ SplitOut split() const { return V1; }
   __device__ const float* src(int) const { return A; }
-  template <int V>
+  template <int V, bool SH = false>
   __device__ void store(uint32_t q, const float (&)[V], const float (&re)[V], const float (&im)[V],
                         const float (&in)[2][V], const SrcIn& src, SplitVal& em) const {
     float gr[V], gi[V], ur[V], ui[V];

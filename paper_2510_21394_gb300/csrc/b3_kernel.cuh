@@ -71,8 +71,8 @@ constexpr int BK = 64;      // k per chunk (one 128-byte bf16 row)
 //    while TMA writes 64 KB per 12 of them: 127 clocks per MMA in the issue
 //    loop.  M is constant, so it is loaded before the wait on the previous
 //    kernel.  (EpiUpdateG 91 -> 73 us at 256^3.)
-//  * setmaxnreg moves registers from the control warps to the epilogue (104
-//    instead of 96), which then does not spill.
+//  * setmaxnreg moves registers from the control warps to the epilogue (104,
+//    grouped 112, instead of 96), which then does not spill.
 // Per launch at 256^3, before -> now, us: EpiStageD 85 -> 78, EpiUpdateG 91 ->
 // 80, EpiFhat 123 -> 104, EpiKrog2 124 -> 103, EpiKrog3 164 -> 123,
 // EpiKrogFinal 154 -> 122 (5.1 .. 5.5 TB/s of 6.8).
@@ -85,9 +85,12 @@ template <class Epi, bool CX = false, bool MT = false>
 struct Cfg {
   static constexpr int kEpi = 16;
   static constexpr int kThreads = 32 * (4 + kEpi);   // 3 control warps, one idle
-  // registers per thread of the control warpgroup and of the four epilogue ones: 128 x 40
-  // + 512 x 104 = 58368 of the 640 x 96 = 61440 the block is launched with
-  static constexpr int kRegCtl = 40, kRegEpi = 104;
+  // registers per thread of the control warpgroup and of the four epilogue ones, out of the
+  // 640 x 96 the block is launched with (checked by the host: a split beyond that would
+  // wait for registers forever).  Grouped launches: the control warps do with 32
+  static constexpr int kRegCtl = 40, kRegEpi = 104, kRegCtlG = 32, kRegEpiG = 112, kRegLaunch = 96;
+  static_assert(128 * kRegCtl + (kThreads - 128) * kRegEpi <= kThreads * kRegLaunch, "register split");
+  static_assert(128 * kRegCtlG + (kThreads - 128) * kRegEpiG <= kThreads * kRegLaunch, "register split");
   static constexpr bool kRing = Epi::kIn > 0 || Epi::kG;   // fetches operands or source terms
   // X and M ring depths
   static constexpr int kNX = CX ? 2 : (MT ? (kRing ? 3 : 6) : (Epi::kIn == 4 ? 2 : (kRing ? 3 : 4)));
@@ -102,6 +105,8 @@ struct Cfg {
   static constexpr uint32_t kOffBar = kOffEpi + kEpi * kEpiWarp;
   static constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;   // + barriers + alignment slack
   static constexpr int kTmemCols = MT ? 512 : 2 * BN;
+  static constexpr uint32_t kSmemGrouped = kSmemBytes + kEpi * (uint32_t)sizeof(PhiPoly);   // after the barriers
+  static_assert(kSmemGrouped <= 232448 || MT, "shared memory budget");
   static_assert(kSmemBytes <= 232448, "shared memory budget");
   static_assert(!(CX && MT), "the complex block does not fit tensor memory");
 };
@@ -307,6 +312,16 @@ __device__ __forceinline__ long long locate(const D* gd, int n, long long u, int
   return u - gd[pid].ubegin;
 }
 
+// the phi polynomial of a functor that has one
+template <class Epi>
+__device__ __forceinline__ auto poly_of(const Epi& e, int) -> decltype(&e.ph) {
+  return &e.ph;
+}
+template <class Epi>
+__device__ __forceinline__ const PhiPoly* poly_of(const Epi&, long) {
+  return nullptr;
+}
+
 // one problem of a grouped fused launch (aligned as its tensor maps)
 template <class Epi>
 struct FusedDesc {
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(Cfg<Epi, CX, MT>::kThreads, 1)
   }
 
   if (warp < 4) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegCtl));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(G ? C::kRegCtlG : C::kRegCtl));
   if (warp == 0) {
     // ------------------------------------------------------------ X producer
     if (lane == 0) {
@@ -572,7 +587,7 @@ __global__ void __launch_bounds__(Cfg<Epi, CX, MT>::kThreads, 1)
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegEpi));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(G ? C::kRegEpiG : C::kRegEpi));
     // ------------------------------------------------------------ epilogue
     // warp: TMEM lane quarter q, 16 rows (half) x 32 columns of each plane (the
     // 32-column half hc), walked as four pieces j of 8 rows x 16 columns: a lane
@@ -660,12 +675,29 @@ __global__ void __launch_bounds__(Cfg<Epi, CX, MT>::kThreads, 1)
     const int prow = lane >> 2, pcol = frag_col(lane) >> 2;
     Walk w;
     w.u = blockIdx.x;
+    // Grouped: the descriptor's phi polynomial is no kernel parameter.  Read from global
+    // memory for every element, its 24 words held up the functors with eigenvalue sums
+    // (96 instances: EpiFhat 917, EpiKrog2 911 us, against 785 and 765 before the epilogue
+    // took two pieces of a row at a time; ETD2RK step 4.20 against 4.09 ms).  Each warp
+    // keeps a copy in shared memory: 747 and 657 us, 3.87 ms.
+    const uint32_t sph = G ? sbase + kOffBar + 256 + (warp - 4) * (uint32_t)sizeof(PhiPoly) : 0u;
+    int sph_pid = -1;
     uint32_t t = 0;
     for (; w.u < nunits; w.u += gridDim.x, ++t) {
       place(w);
       const int a = t & 1;
       const uint32_t tl = tmem_base + ((uint32_t)(q * 32 + 16 * half) << 16) + a * BN + 32 * hc;
       const Epi& E = *functor(w);
+      if constexpr (G) {
+        if (const PhiPoly* ph = poly_of(E, 0); ph && w.pid != sph_pid) {
+          sph_pid = w.pid;
+          __syncwarp();
+          if (lane < (int)(sizeof(PhiPoly) / 4))
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(sph + 4 * lane), "f"(reinterpret_cast<const float*>(ph)[lane])
+                         : "memory");
+          __syncwarp();
+        }
+      }
       // eigenvalue sums of the tile: the part of r, and lam_d of this lane's rows
       LamR<4> lr[2];
       float ld[2] = {0.f, 0.f};
@@ -721,7 +753,7 @@ __global__ void __launch_bounds__(Cfg<Epi, CX, MT>::kThreads, 1)
           for (int k = 0; k < 2 * NOP; ++k) lds16(piece + k * 1024, in[k]);
           float sv[4] = {0.f, 0.f, 0.f, 0.f};
           if constexpr (Epi::kLam) lam_s<4>(lr[h], g ? ld[1] : ld[0], sv);
-          E.template store<4>(e, sv, re, im, in, SrcIn{piece + Epi::kIn * 1024, nsf}, em[h]);
+          E.template store<4, G>(e, sv, re, im, in, SrcIn{piece + Epi::kIn * 1024, nsf, sph}, em[h]);
         } else if (live) {   // rows of odd length (d = 1): element by element
 #pragma unroll 1
           for (int v = 0; v < 4; ++v) {

@@ -4,15 +4,23 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <stdexcept>
+#include <string>
 
 #include "b3_launch.h"
 #include "tma_host.h"
 
 namespace fcgle {
 
+// Shared memory of a fused kernel, and the registers it is launched with, which its
+// setmaxnreg split relies on.
 template <class K>
 void set_smem(K* kernel, uint32_t bytes) {
   FCGLE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  cudaFuncAttributes a;
+  FCGLE_CUDA(cudaFuncGetAttributes(&a, kernel));
+  if (a.numRegs < b3::Cfg<b3::EpiStoreF32>::kRegLaunch)
+    throw std::logic_error("fused kernel built with " + std::to_string(a.numRegs) + " registers");
 }
 
 template <class Epi>
@@ -48,12 +56,12 @@ void FusedLaunch<Epi>::single(bool natural_order, const FusedMaps& m, const b3::
 template <class Epi>
 void FusedLaunch<Epi>::grouped(const void* descs, int n, long long units, cudaStream_t st) {
   static std::once_flag attr;
-  std::call_once(attr, [] { set_smem(b3::mp_b3_kernel<Epi, true>, b3::Cfg<Epi>::kSmemBytes); });
+  std::call_once(attr, [] { set_smem(b3::mp_b3_kernel<Epi, true>, b3::Cfg<Epi>::kSmemGrouped); });
   CUtensorMap z;
   std::memset(&z, 0, sizeof(z));
   b3::KParams kp{};
   launch_pdl(b3::mp_b3_kernel<Epi, true>, (int)std::min<long long>(units, num_sms()), b3::Cfg<Epi>::kThreads,
-             b3::Cfg<Epi>::kSmemBytes, st, z, z, z, z, kp, Epi{}, static_cast<const b3::FusedDesc<Epi>*>(descs), n,
+             b3::Cfg<Epi>::kSmemGrouped, st, z, z, z, z, kp, Epi{}, static_cast<const b3::FusedDesc<Epi>*>(descs), n,
              units);
 }
 

@@ -1478,8 +1478,9 @@ class EngineB3 : public EngineBase {
     double fact = 6.0;   // (m + 3)! at m = 0
     for (int m = 0; m < 10; ++m) {
       const std::complex<double> c = wm / fact;
-      P.cr[m] = (float)c.real();
-      P.ci[m] = (float)c.imag();
+      float* q = &P.c[m / 2].x + 2 * (m % 2);
+      q[0] = (float)c.real();
+      q[1] = (float)c.imag();
       wm *= v;
       fact *= (double)(m + 4);
     }
