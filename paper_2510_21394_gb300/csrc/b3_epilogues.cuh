@@ -928,31 +928,31 @@ struct EpiLRK2B {
 // w(t) = exp(t gamma - (kappa + i zeta)/(2 kappa) log(1 + 2 t phi_1(2 gamma t) kappa |w0|^2)) w0
 struct Flow {
   float gamma_t;   // t gamma
-  float growth;    // e^{t gamma}
   float c2;        // 2 t phi_1(2 gamma t) kappa
   float zk;        // zeta / (2 kappa)
 };
-// The modulus e^{t gamma - L / 2} = e^{t gamma} (1 + c2 |w|^2)^{-1/2}.
 __device__ __forceinline__ void flow_eval(const Flow& f, float wr, float wi, float& yr, float& yi) {
-  const float x = f.c2 * (wr * wr + wi * wi);
-  const float m = f.growth * rsqrtf(1.f + x);
+  const float L = log1pf(f.c2 * (wr * wr + wi * wi));
+  const float m = expf(f.gamma_t - 0.5f * L);
   float s, c;
-  sincosf(-f.zk * log1pf(x), &s, &c);
+  sincosf(-f.zk * L, &s, &c);
   yr = m * (c * wr - s * wi);
   yi = m * (c * wi + s * wr);
 }
 
 // Phi_t(w) - w = (e^E - 1) w with E = t gamma - (1 + i zeta/kappa) L / 2,
 // L = log(1 + c2 |w|^2): e^E - 1 = expm1(Re E) cos(Im E) - 2 sin^2(Im E / 2)
-// + i e^{Re E} sin(Im E), without cancellation for small t; cos and sin of Im E
-// from those of Im E / 2.
+// + i e^{Re E} sin(Im E), without cancellation for small t.  (The modulus as
+// e^{t gamma} rsqrt(1 + c2 |w|^2) and one sincos of Im E / 2 took 4 % less of a
+// Strang run, and added 0.9 to 1.2 % to its error against 64 bits.)
 __device__ __forceinline__ void flow_incr(const Flow& f, float wr, float wi, float& dr, float& di) {
   const float L = log1pf(f.c2 * (wr * wr + wi * wi));
-  float sh, ch;
-  sincosf(-0.5f * f.zk * L, &sh, &ch);
-  const float em = expm1f(f.gamma_t - 0.5f * L);
-  const float v = 2.f * sh * sh;                 // 1 - cos(Im E)
-  const float er = em * (1.f - v) - v, ei = (1.f + em) * (2.f * sh * ch);
+  const float a = f.gamma_t - 0.5f * L, b = -f.zk * L;
+  float s, c, sh, ch;
+  sincosf(b, &s, &c);
+  sincosf(0.5f * b, &sh, &ch);
+  const float em = expm1f(a);
+  const float er = em * c - 2.f * sh * sh, ei = (1.f + em) * s;
   dr = er * wr - ei * wi;
   di = er * wi + ei * wr;
 }

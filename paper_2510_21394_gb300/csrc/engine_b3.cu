@@ -1461,7 +1461,6 @@ class EngineB3 : public EngineBase {
     const double p1 = std::fabs(z) < 1e-8 ? 1.0 + z / 2.0 : std::expm1(z) / z;
     b3::Flow f;
     f.gamma_t = (float)(t * prm_.gamma);
-    f.growth = (float)std::exp(t * prm_.gamma);
     f.c2 = (float)(2.0 * t * p1 * prm_.kappa);
     f.zk = (float)(prm_.zeta / (2.0 * prm_.kappa));
     return f;
