@@ -757,10 +757,10 @@ def run_config2(args, rank, world, local_rank):
                                      "how": "measured here: cuBLAS TF32 (torch.matmul float32, TF32 allowed, 8192^3, "
                                             "best of 5); context for the split-TF32 end transforms"}
         extra["fp64_gpu"] = f64
-        # 28 exact bf16 products of digits per FP64 product (7 digits per operand, pairs i + j < 7)
-        extra["fp64_roofline"] = {"bound": "tensor", "achieved": round(28 * tf64, 1), "peak": round(peak, 1),
-                                  "unit": "TFLOP/s", "frac": round(28 * tf64 / peak, 4),
-                                  "kernel": "slice_kernel + sliced_gemm_kernel<double> (one 1024 x 1024 mode product)",
+        # 36 bf16 products of digits per FP64 product (8 digits per operand, pairs i + j < 8)
+        extra["fp64_roofline"] = {"bound": "tensor", "achieved": round(36 * tf64, 1), "peak": round(peak, 1),
+                                  "unit": "TFLOP/s", "frac": round(36 * tf64 / peak, 4),
+                                  "kernel": "slice_kernel + sliced_gemm_kernel<Slices64> (one 1024 x 1024 mode product)",
                                   "peak_kind": f"{peak_kind} bf16_tflops (burst)", "launch_ms": round(ms_mp64, 5),
                                   "fp64_tflops": round(tf64, 3), "dgemm_tflops": round(dpeak, 3),
                                   "dgemm_how": "measured here: cuBLAS DGEMM (torch.matmul float64, 4096^3, "

@@ -75,10 +75,13 @@ typedef enum {
 } fcgle_status;
 
 /* Arithmetic of the mode products.  FCGLE_FP64: complex128 tensors, FP64
- * mode products.  FCGLE_BF16X3: complex64 tensors (FP32 storage), mode
- * products on the tcgen05 tensor cores with each FP32 operand split as
- * hi + lo (two bf16) and hi*hi + hi*lo + lo*hi accumulated in FP32; the
- * eigendecomposition is FP64 and the spectral scalars f(theta lam) are
+ * mode products: contractions of 16 terms and more by integer slices of 62 bits
+ * with one exponent per fiber, which give every entry to about 2^-60 sqrt(K) of
+ * the largest entries of its two fibers (2^-53 of the result at best, like any
+ * FP64 sum), shorter ones in FP64 arithmetic.  FCGLE_BF16X3: complex64
+ * tensors (FP32 storage), mode products on the tcgen05 tensor cores with each
+ * FP32 operand split as hi + lo (two bf16) and hi*hi + hi*lo + lo*hi accumulated
+ * in FP32; the eigendecomposition is FP64 and the spectral scalars f(theta lam) are
  * formed from FP64 coefficients and evaluated in FP32.
  * FCGLE_TF32 (one-pass TF32 mode products) is not built: fcgle_setup returns
  * FCGLE_ERR_UNSUPPORTED for it.  It would read the same operand bytes as
@@ -131,8 +134,8 @@ typedef struct fcgle_ctx* fcgle_handle;
  * For BF16X3 handles the setup also runs the kernel autotuner (see
  * fcgle_autotune_report) on that stream for problem shapes this process has
  * not tuned yet, and waits for it; do not call it during a stream capture.
- * Device memory per internal element (P of fcgle_internal_elems): FP64 220
- * bytes (12 tensors, and 28 bytes for the digits of the products), and 16 more
+ * Device memory per internal element (P of fcgle_internal_elems): FP64 224
+ * bytes (12 tensors, and 32 bytes for the digits of the products), and 16 more
  * for every spectral function f(theta Lam) in use and every source term; BF16X3
  * 96 bytes (8 FP32 and 4 split tensors) and 8 per source term; besides, some
  * tens of bytes per entry of the matrices Q_mu.
@@ -347,9 +350,10 @@ fcgle_status fcgle_internal_elems(fcgle_handle h, size_t* P);
  * d >= 2, R is a multiple of 8 and p_mu <= 256 (the tensor core's FP32
  * accumulation error grows with the contracted length).  Handles with d >= 2
  * and any p > 256 use FP32 products by integer slices (both operands as
- * fixed-point numbers of 25 bits and a sign per row of the contraction, summed
- * exactly on the bf16 tensor cores); otherwise FP32 on the CUDA cores.  flags bit 3 (BF16X3 handles, d = 3, p_2 <= 256, with
- * bit 1, direction 0): the slab-fused mode-1 and mode-2 products in the
+ * fixed-point numbers of 30 bits and a sign, with one exponent per fiber of the
+ * contraction, multiplied and added as integers on the bf16 tensor cores);
+ * otherwise FP32 on the CUDA cores.  flags bit 3 (BF16X3 handles, d = 3,
+ * p_2 <= 256, with bit 1, direction 0): the slab-fused mode-1 and mode-2 products in the
  * natural order, Y[c][j3][i2][i1] = sum M_2[i2][j2] M_1[i1][j1]
  * X[c][j3][j2][j1] with M_mu = Q_mu^T (bit 0) or Q_mu.  flags bit 4 (BF16X3
  * handles, d >= 2, R % 8 == 0, with bit 1, direction d-1): the product above

@@ -328,7 +328,7 @@ fcgle_status fcgle_selftest_slice_segment(const double* M, int rows, int K, int*
   return guarded([&] {
     if (!M || !terms) throw InvalidArg("NULL argument");
     if (rows < 1 || K < 1) throw InvalidArg("rows and K must be >= 1");
-    *terms = slice_segment<double>(M, rows, K);
+    *terms = slice_segment<Slices64>(M, rows, K);
   });
 }
 

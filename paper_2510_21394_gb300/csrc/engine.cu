@@ -130,7 +130,7 @@ class Engine : public EngineBase {
         x.rows = (long long)(s_.P / s_.p[mu]) * (cx ? 1 : 2);
         x.K = s_.p[mu] * (cx ? 2 : 1);
         if (!sliceable(x.K, x.rows)) continue;
-        xbytes = std::max(xbytes, slice_bytes<double>(x.rows, x.K));
+        xbytes = std::max(xbytes, slice_bytes<Slices64>(x.rows, x.K));
         xrows = std::max(xrows, x.rows);
       }
     // ---- device copies: lam_mu (padded), mode-product matrices and their digits
@@ -156,7 +156,7 @@ class Engine : public EngineBase {
         ms_[mu][1].build(mf64_[mu][1]->ptr, Mb, D.p, st_, launches);
       }
     }
-    // ---- workspace for the digits of the data, 28 bytes per grid point, and their
+    // ---- workspace for the digits of the data, 32 bytes per grid point, and their
     // exponents; apply_f and norm work in tensors of the schemes, so that a handle
     // holds 12 tensors and this
     if (xbytes) {
@@ -169,7 +169,7 @@ class Engine : public EngineBase {
         if (!sliceable(x.K, x.rows)) continue;
         x.dig = reinterpret_cast<__nv_bfloat16*>(xdig_->ptr);
         x.ex = reinterpret_cast<int*>(xdig_->ptr + xbytes);
-        slice_map<double>(x, false);
+        slice_map<Slices64>(x, false);
       }
     lv_.c_re = prm.nu;
     lv_.c_im = prm.eta;
@@ -397,13 +397,13 @@ class Engine : public EngineBase {
     // M: on the device, Mh: the same on the host
     void build(const double* M, const std::vector<double>& Mh, int K, cudaStream_t st, long long& nl) {
       s.rows = s.K = K;
-      s.seg = slice_segment(Mh.data(), K, K);
-      dig.reset(new DevBuf<uint8_t>(slice_bytes<double>(K, K)));
+      s.seg = slice_segment<Slices64>(Mh.data(), K, K);
+      dig.reset(new DevBuf<uint8_t>(slice_bytes<Slices64>(K, K)));
       ex.reset(new DevBuf<int>(slice_exponents(K)));
       s.dig = reinterpret_cast<__nv_bfloat16*>(dig->ptr);
       s.ex = ex->ptr;
-      slice_map<double>(s, true);
-      slice_rows<double>(M, s, 1, K, 0, SliceOut<double>{}, st, nl);
+      slice_map<Slices64>(s, true);
+      slice_rows<Slices64>(M, s, 1, K, 0, SliceOut<double>{}, st, nl);
     }
   };
   // The sliced product (two launches) against the CUDA cores, us: 12.6 / 21.0 at
@@ -417,8 +417,8 @@ class Engine : public EngineBase {
     const Sliced& x = xs_[mu][cx];
     if (m.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
       const long long plane = R * s_.p[mu];
-      slice_rows<double>(X, x, cx ? 2 : 1, s_.p[mu], plane, SliceOut<double>{M, Y, R, plane, x.K}, st_, launches);
-      sliced_gemm<double>(x, m.s, Y, R, plane, err_->ptr, st_, launches);
+      slice_rows<Slices64>(X, x, cx ? 2 : 1, s_.p[mu], plane, SliceOut<double>{M, Y, R, plane, x.K}, st_, launches);
+      sliced_gemm<Slices64>(x, m.s, Y, R, plane, err_->ptr, st_, launches);
       return;
     }
     mp_f64(X, Y, M, s_.p[mu], (size_t)R, cx != 0, st_, launches);

@@ -427,26 +427,26 @@ class EngineB3 : public EngineBase {
       FCGLE_CUDA(cudaMemsetAsync(f32p_[i], 0, 2 * s_.P * 4, st_));
     }
     if (use_sliced()) {
-      // digits [3][2 R][p] bf16 = 12 P bytes of one direction at a time, then 2 R
-      // exponents (at most P / 2 bytes, p >= 16), in the 16 P bytes of kD3 and kEA:
-      // no scheme holds anything there while a precise operator runs, and none reads
-      // them before it has written them whole, so the digits cost no memory
+      // digits [4][2 R][p] bf16 of one direction at a time in the 16 P bytes of kD3 and
+      // kEA, the 2 R exponents in kUp: no scheme holds anything there while a precise
+      // operator runs, and none reads them before it has written them whole, so the
+      // digits cost no memory
       for (int mu = 0; mu < prm.d; ++mu) {
         if (!sliceable(mu)) continue;
         Sliced& x = xs_[mu];
         x.dig = reinterpret_cast<__nv_bfloat16*>(F32(kD3));
-        x.ex = reinterpret_cast<int*>(F32(kD3) + 3 * s_.P);
+        x.ex = reinterpret_cast<int*>(F32(kUp));
         x.rows = 2 * (P_ / s_.p[mu]);
         x.K = s_.p[mu];
-        slice_map<float>(x, false);
+        slice_map<Slices32>(x, false);
         for (int f = 0; f < 2; ++f) {
           Mat& m = mat_[mu][f];
           m.sl.rows = m.sl.K = m.p;
-          m.sl.seg = slice_segment<float>(nullptr, m.p, m.p);   // the same for every matrix
-          FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<float>(m.p, m.p)));
+          m.sl.seg = slice_segment<Slices32>(nullptr, m.p, m.p);   // the same for every matrix
+          FCGLE_CUDA(cudaMalloc(&m.sl.dig, slice_bytes<Slices32>(m.p, m.p)));
           FCGLE_CUDA(cudaMalloc(&m.sl.ex, slice_exponents(m.p) * sizeof(int)));
-          slice_map<float>(m.sl, true);
-          slice_rows<float>(m.f32, m.sl, 1, m.p, 0, SliceOut<float>{}, st_, launches);
+          slice_map<Slices32>(m.sl, true);
+          slice_rows<Slices32>(m.f32, m.sl, 1, m.p, 0, SliceOut<float>{}, st_, launches);
         }
       }
     }
@@ -995,8 +995,8 @@ class EngineB3 : public EngineBase {
   // products adds an error that grows with the contracted length (measured
   // 2.4e-6 at p = 264; at p = 1024 it lifted the error at T of 500 steps from
   // 1.6e-6 to 8.5e-6).  Longer contractions: the sliced product (sliced.cu),
-  // whose accumulation is exact (1e-7 at p = 1024, FP32 on the CUDA cores
-  // 8e-7).  FP32 on the CUDA cores for d = 1 and where tc_ok is false (the
+  // which adds integers and rounds once (6e-8; FP32 on the CUDA cores 8e-7 at
+  // p = 1024).  FP32 on the CUDA cores for d = 1 and where tc_ok is false (the
   // adjoint).
   static constexpr int kTf32MaxP = 256;
   void tucker_f32(const float* X, float* Y, bool fwd, bool tc_ok = true) {
@@ -1068,8 +1068,8 @@ class EngineB3 : public EngineBase {
     const Mat& m = mat_[mu][fwd ? 0 : 1];
     const long long R = P_ / s_.p[mu];
     if (m.sl.dig && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
-      slice_rows<float>(X, xs_[mu], 1, s_.p[mu], 0, SliceOut<float>{m.f32, Y, R, P_, m.p}, st_, launches);
-      sliced_gemm<float>(xs_[mu], m.sl, Y, R, P_, err_->ptr, st_, launches);
+      slice_rows<Slices32>(X, xs_[mu], 1, s_.p[mu], 0, SliceOut<float>{m.f32, Y, R, P_, m.p}, st_, launches);
+      sliced_gemm<Slices32>(xs_[mu], m.sl, Y, R, P_, err_->ptr, st_, launches);
     } else {
       mp_f32(X, Y, m.f32, s_.p[mu], (size_t)R, st_, launches);
     }

@@ -1,7 +1,7 @@
 // Mode products in FP64 and in precise FP32 on the bf16 tensor cores.
 //
 // An FP64 multiply-add on GB300's CUDA cores runs at about 1.1 TFLOP/s per
-// GPU, the bf16 tensor cores at 1.9 PFLOP/s: 28 bf16 products of integer
+// GPU, the bf16 tensor cores at 1.9 PFLOP/s: 36 bf16 products of integer
 // slices (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
 // Algorithms 59 (2012)) are far cheaper than one FP64 product.  Both operands
 // are written as fixed-point numbers with one exponent per row (per fiber of
@@ -14,24 +14,18 @@
 // and rounds once.
 //
 // What the accumulator holds exactly: integers up to 2^24.  Level s takes s + 1
-// products per k, of digits |d| <= 2^{RB - 1} (the top ones <= 128), so FP64 P_s
-// is at most (s + 1) 2^14 per k.  A unit lost in P_s is 2^{-8 s} of a unit of
-// P_0: levels 0 .. 3 have to be exact, and are, whatever the data: contractions
-// go in segments short enough for the digits of the matrix at hand
-// (slice_segment; 256 terms always do, and 350 to 450 with eigenvector matrices,
-// whose lower digits average half the largest).  Levels 4 .. 6 reach at most 7/4
-// of what level 3 does; a unit lost there is at most 2^-46 of one full-size
-// term max|x| max|M_i| (2^-22 at level 1), and it takes hundreds of terms with all digits in line to lose
-// one.  FP32: P_0 <= 2^14 per k is exact over 1024 terms; digits below the
-// top one reach 256, so P_1 .. P_3 may pass 2^24 (up to 2^27) when hundreds of
-// their digits are in line, and then lose up to 2^-14 max|x| max|M_i| over 1024
-// terms, which is what 1024 roundings of an FP32 product come to; digits that
-// are not in line stay below 2^21.
+// products per k of digits |d| <= 128, the top ones <= 64.  A unit lost in P_s is
+// 2^{-8 s - 12} of a full-size term max|x| max|M_i|, and an FP64 product rounds by up to
+// 2^-53 K of one: levels 0 .. 4 have to be exact, and are, whatever the data:
+// contractions go in segments short enough for the digits of the matrix at hand
+// (slice_segment; 256 terms always do, and 350 to 500 with eigenvector matrices, whose
+// digits average half the largest).  Levels 5 .. 7 may lose units of 2^-52 and less
+// when hundreds of their digits are in line.  FP32: P_0 and P_1 are exact over 1024
+// terms (2^12 and 2^14 per k); a unit lost in P_2 is 2^-28 of a full-size term.
 //
-// Cut off: half a unit of an operand's last digit, and the levels s >= NLEV, for
-// an error per entry of about 2^-55 sqrt(K) max|x| max|M_i| (FP64; FP32: 2^-26),
-// relative to the largest entries of the two fibers, not to the entry's own
-// terms.
+// Cut off: a unit of an operand's last digit at most, and the levels s >= NLEV, for an
+// error per entry of about 2^-60 sqrt(K) max|x| max|M_i| (FP32: 2^-29), relative to the
+// largest entries of the two fibers, not to the entry's own terms.
 //
 // Orientation: the data rows (c, r) are the MMA's M (TMEM lanes), so that a
 // warp stores 32 consecutive r of one output index i; 64 (FP64) or 128 (FP32)
@@ -46,6 +40,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <stdexcept>
 #include <string>
 #include <vector>
 
@@ -105,11 +100,13 @@ template <>
 struct Balanced<float> {
   using W = int;
 };
-template <typename T>
-__host__ __device__ __forceinline__ typename Balanced<T>::W balanced(typename Bits<T>::U u, int emax, bool bad) {
+template <class C>
+__host__ __device__ __forceinline__ typename Balanced<typename C::T>::W balanced(typename Bits<typename C::T>::U u,
+                                                                                 int emax, bool bad) {
+  using T = typename C::T;
   using U = typename Bits<T>::U;
   using W = typename Balanced<T>::W;
-  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
+  constexpr int NS = C::NS, RB = C::RB, MB = Bits<T>::kMant, UP = C::BITS - MB - 2;
   const int e = (int)((u >> MB) & Bits<T>::kExpMask);
   const U mant = ((u & ((U(1) << MB) - 1)) | (e ? U(1) << MB : U(0))) << UP;
   const int s = emax - (e > 1 ? e : 1);
@@ -155,14 +152,14 @@ __device__ __noinline__ void infinite_rows(const T* X, long long rows, int nseg,
   }
 }
 
-template <typename T>
+template <class C, typename T = typename C::T>
 __global__ void __launch_bounds__(256) slice_kernel(const T* X, long long rows, int nseg, int seg_len,
                                                     long long seg_stride, int pitch, int group,
                                                     __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
                              const __grid_constant__ SliceOut<T> o) {
   using U = typename Bits<T>::U;
-  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant;
-  constexpr int UP = SliceCfg<T>::BITS - MB - 2;   // spare bits below the last one of the largest entry
+  constexpr int NS = C::NS, RB = C::RB, MB = Bits<T>::kMant;
+  constexpr int UP = C::BITS - MB - 2;   // spare bits below the last one of the largest entry
   pdl_trigger();
   pdl_wait();
   const int per_block = 256 / group;
@@ -197,7 +194,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* X, long long rows, 
         load4<T>(src + 4 * q, u);
         typename Balanced<T>::W w[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) w[v] = balanced<T>(u[v], emax, bad);
+        for (int v = 0; v < 4; ++v) w[v] = balanced<C>(u[v], emax, bad);
 #pragma unroll
         for (int a = 0; a < NS; ++a) {
           uint32_t h[4];
@@ -221,16 +218,16 @@ __global__ void __launch_bounds__(256) slice_kernel(const T* X, long long rows, 
 
 // The same pass for rows of up to 8 x 32 x IT elements in segments of a multiple
 // of 8: a lane keeps its 8-element pieces in registers between the two halves
-// and stores 16 bytes per digit (FP32 at 432^3: 473 us with 4-element pieces read
-// twice, 303 this way = 5.3 TB/s; FP64 at 128 x 120 x 136: 25 -> 20 us).
-template <typename T, int IT>
+// and stores 16 bytes per digit (FP32 at 432^3 with 3 digits: 473 us with 4-element
+// pieces read twice, 303 this way = 5.3 TB/s).
+template <class C, int IT, typename T = typename C::T>
 __global__ void __launch_bounds__(256) slice8_kernel(const T* X, long long rows, int nseg, int seg_len,
                                                      long long seg_stride, int pitch, int group,
                                                      __nv_bfloat16* __restrict__ dig, int* __restrict__ ex,
                              const __grid_constant__ SliceOut<T> o) {
   using U = typename Bits<T>::U;
   using W = typename Balanced<T>::W;
-  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB, MB = Bits<T>::kMant, UP = SliceCfg<T>::BITS - MB - 2;
+  constexpr int NS = C::NS, RB = C::RB, MB = Bits<T>::kMant, UP = C::BITS - MB - 2;
   pdl_trigger();
   pdl_wait();
   const int per_block = 256 / group, lig = threadIdx.x % group;
@@ -269,7 +266,7 @@ __global__ void __launch_bounds__(256) slice8_kernel(const T* X, long long rows,
       if (c < chunks) {
         W w[8];
 #pragma unroll
-        for (int v = 0; v < 8; ++v) w[v] = balanced<T>(u[it][v], emax, bad);
+        for (int v = 0; v < 8; ++v) w[v] = balanced<C>(u[it][v], emax, bad);
         __nv_bfloat16* dst = dig + row * pitch + 8 * c;
 #pragma unroll
         for (int a = 0; a < NS; ++a) {
@@ -294,48 +291,36 @@ __global__ void __launch_bounds__(256) slice8_kernel(const T* X, long long rows,
 }
 
 // ------------------------------------------------------------ product
-// Measured with the slicing pass (one real product, GB300): FP64 128 x 120 x 136
-// 58 us (900 us on the CUDA cores, whose FP64 rate is 1.1 TFLOP/s), 400 x 400 29
-// (412), 1023 x 1024 95 (4090), 432 x 432 x 100 811 (27014); relative error
-// 1.0e-16 .. 1.4e-16 (2.5e-16 .. 1.1e-15).  FP32 1023 x 1024 34 us (150), 432 x
-// 432 x 100 270 (1080); error 5e-8 (4e-7 .. 6e-7).
+// Measured with the slicing pass (one real product, GB300, L2 flushed): FP64 128 x
+// 120 x 136 68 us (900 us on the CUDA cores, whose FP64 rate is 1.1 TFLOP/s), 400 x
+// 400 40 (412), 1023 x 1024 138 (4090), 432 x 432 x 100 945 (27014).  FP32 1023 x
+// 1024 44 us (150), 432 x 432 x 100 337 (1080).
 // What bounds it: the bf16 tensor cores and, close behind, the operand bytes
-// an SM pulls from L2 (FP64: 84 KB per 32 k against 1792 MMA clocks, 47 bytes
-// per clock).  All levels of a tile share tensor memory (FP64 7 x 64, FP32
+// an SM pulls from L2 (FP64: 96 KB per 32 k against 2304 MMA clocks, 43 bytes
+// per clock).  All levels of a tile share tensor memory (FP64 8 x 64, FP32
 // 4 x 128 columns), so the accumulators are single-buffered and the MMAs of
 // the next tile wait while the epilogue reads them.  16 epilogue warps therefore
 // only add the levels up to integer sums (16 or 32 columns each), hand tensor
 // memory back, and round and store while the next tile runs (8 warps that rounded
 // first: 1125 against 754 us for FP32 at 432^3, 67 against 51 for FP64 at
 // 128 x 120 x 136).
-template <typename T>
-struct GemmCfg;
-template <>
-struct GemmCfg<double> {
-  static constexpr int NLEV = 7, NT = 64, NSTAGE = 2;
-};
-template <>
-struct GemmCfg<float> {
-  static constexpr int NLEV = 4, NT = 128, NSTAGE = 4;
-};
-
-constexpr int kSegK = 1024;     // longest contraction whose level 0 stays exact (below 2^24)
+constexpr int kSegK = 1024;     // longest contraction whose levels 0 and 1 stay exact (within 2^24)
 constexpr int kGK = 32;         // k per stage: 64-byte bf16 rows, 64-byte swizzle
 constexpr int kGM = 128;        // data rows per tile
 constexpr int kGEpi = 16;       // epilogue warps
 constexpr int kGThreads = 32 * (4 + kGEpi);   // producer, MMA issuer, two idle ones
-// registers: 128 x 40 + 512 x 104 = 58368 of the 640 x 96 = 61440 at launch
-constexpr int kGRegCtl = 40, kGRegEpi = 104;
+// registers: 128 x 40 + 512 x 104 = 58368 of the 640 x 96 = 61440 at launch (checked by the host)
+constexpr int kGRegCtl = 40, kGRegEpi = 104, kGRegLaunch = 96;
 
-template <typename T>
+template <class C>
 struct GemmLayout {
-  static constexpr int NS = SliceCfg<T>::NS;
-  static constexpr uint32_t kA = kGM * 64, kB = GemmCfg<T>::NT * 64;   // bytes of one slice of a chunk
+  static constexpr int NS = C::NS;
+  static constexpr uint32_t kA = kGM * 64, kB = C::NT * 64;   // bytes of one slice of a chunk
   static constexpr uint32_t kStage = NS * (kA + kB);
-  static constexpr uint32_t kOffBar = GemmCfg<T>::NSTAGE * kStage;
+  static constexpr uint32_t kOffBar = C::NSTAGE * kStage;
   static constexpr uint32_t kSmem = kOffBar + 256 + 1024;
   static_assert(kSmem <= 232448, "shared memory budget");
-  static_assert(GemmCfg<T>::NLEV * GemmCfg<T>::NT <= 512, "tensor memory columns");
+  static_assert(C::NLEV * C::NT <= 512, "tensor memory columns");
   static_assert(kStage % 1024 == 0 && kA % 1024 == 0 && kB % 1024 == 0, "slices start on swizzle atoms");
 };
 
@@ -361,34 +346,29 @@ __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
          ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
-// The levels of one output, added up exactly: FP64 as V = 2^24 hi + lo, FP32
-// from the smallest level up.  add() takes the levels of one segment of the
+// The levels of one output, added up exactly: FP64 as V = 2^32 hi + lo (levels 0 .. 3
+// and 4 .. 7), FP32 from the smallest level up.  add() takes the levels of one segment of the
 // contraction, get() gives the sum times 2^e.
-template <typename T>
-struct Sum;
-template <>
-struct Sum<double> {
+template <class C, typename T = typename C::T>
+struct Sum {   // FP64, RB = 8
+  static_assert(C::NLEV == 8 && C::RB == 8, "sums of eight 8-bit levels");
   long long hi = 0, lo = 0;
-  __device__ __forceinline__ void add(const float (&P)[7]) {
+  __device__ __forceinline__ void add(const float (&P)[C::NLEV]) {
     hi += ((long long)__float2int_rn(P[0]) << 24) + ((long long)__float2int_rn(P[1]) << 16) +
           ((long long)__float2int_rn(P[2]) << 8) + (long long)__float2int_rn(P[3]);
-    lo += ((long long)__float2int_rn(P[4]) << 16) + ((long long)__float2int_rn(P[5]) << 8) +
-          (long long)__float2int_rn(P[6]);
+    lo += ((long long)__float2int_rn(P[4]) << 24) + ((long long)__float2int_rn(P[5]) << 16) +
+          ((long long)__float2int_rn(P[6]) << 8) + (long long)__float2int_rn(P[7]);
   }
-  // |hi| < 2^38 K: rounded to 53 bits through a 63-bit integer t = V / 2^s, s the
+  // |hi| < 2^37 K: rounded to 53 bits through a 63-bit integer t = V / 2^s, s the
   // smallest shift that makes it fit, so that t is V itself or has 62 bits.  To
-  // double by 32-bit integer arithmetic: FP64 additions and the conversion
-  // instruction run on the FP64 pipe at two lanes per clock and SM.
+  // double by integer arithmetic: FP64 additions and the conversion instruction run on
+  // the FP64 pipe at two lanes per clock and SM.
   __device__ __forceinline__ double get(int e) const {
-    const int s = max(0, 26 - __clzll(hi ^ (hi >> 63))), up = 24 - s;   // bits of |hi| beyond 38; K <= 2^24: s <= 24
-    const uint32_t h0 = (uint32_t)hi, h1 = (uint32_t)(hi >> 32);
-    const long long lr = lo + ((1ll << s) >> 1);
-    const uint32_t l0 = (uint32_t)lr, l1 = (uint32_t)(lr >> 32);
+    const int s = max(0, 34 - __clzll(hi ^ (hi >> 63))), up = 32 - s;   // bits of |hi| beyond 30; K <= 2^24: s <= 32
     const unsigned long long tu =
-        (((unsigned long long)__funnelshift_l(h0, h1, up) << 32) | (h0 << up)) +
-        (((unsigned long long)(uint32_t)((int)l1 >> s) << 32) | __funnelshift_r(l0, l1, s));
+        ((unsigned long long)hi << up) + (unsigned long long)((lo + ((1ll << s) >> 1)) >> s);
     const long long t = (long long)tu;
-    const int k = e + 48 + s;
+    const int k = e + 8 * (2 * C::NS - 1 - C::NLEV) + s;
     if (k <= -1000 || k >= 900) return ldexp((double)t, k);
     // normalise to 64 bits, round to nearest even, fill in sign and exponent
     const uint32_t sg = (uint32_t)((int)(tu >> 32) >> 31);
@@ -404,33 +384,34 @@ struct Sum<double> {
     return tu == 0ull ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)(sg & 0x80000000u) << 32)));
   }
 };
-template <>
-struct Sum<float> {
+template <class C>
+struct Sum<C, float> {
   float t = 0.f;
   __device__ __forceinline__ void add(const float (&P)[4]) {
-    t += fmaf(fmaf(fmaf(P[3], 1.f / 512.f, P[2]), 1.f / 512.f, P[1]), 1.f / 512.f, P[0]);
+    constexpr float u = 1.f / (1 << C::RB);
+    t += fmaf(fmaf(fmaf(P[3], u, P[2]), u, P[1]), u, P[0]);
   }
   __device__ __forceinline__ float get(int e) const {
-    const int k = e + 36;
+    const int k = e + C::RB * (2 * C::NS - 2);
     if (k >= -126 && k <= 127) return t * __int_as_float((k + 127) << 23);
     return ldexpf(t, k);
   }
 };
 
-template <typename T>
-__device__ __forceinline__ T finish(const Sum<T>& s, int er, int ei) {
+template <class C, typename T = typename C::T>
+__device__ __forceinline__ T finish(const Sum<C>& s, int er, int ei) {
   return unsliced(er) || unsliced(ei) ? (T)NAN : s.get(er + ei);
 }
 
 // SEG: the contraction goes in segments of gp.seg chunks, each drained from tensor
 // memory into the integer sums before the next begins.
-template <typename T, bool SEG>
+template <class C, bool SEG, typename T = typename C::T>
 __global__ void __launch_bounds__(kGThreads, 1)
     sliced_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_m,
                        const int* ex, const int* __restrict__ em, T* __restrict__ Y,
                        const GemmParams gp) {
-  using L = GemmLayout<T>;
-  constexpr int NS = SliceCfg<T>::NS, NLEV = GemmCfg<T>::NLEV, NT = GemmCfg<T>::NT, NSTAGE = GemmCfg<T>::NSTAGE;
+  using L = GemmLayout<C>;
+  constexpr int NS = C::NS, NLEV = C::NLEV, NT = C::NT, NSTAGE = C::NSTAGE;
   extern __shared__ uint8_t smem_raw[];
   pdl_trigger();
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -561,7 +542,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
       const int i0 = (int)(u % gp.m_tiles) * NT + cg * NC;
       const bool live = row < gp.rows;
       const int er = live ? ex[row] : 0;
-      Sum<T> sum[NC];
+      Sum<C> sum[NC];
       for (int sg = 0; sg < segs; ++sg, ++t) {
         if (!mbar_wait(acc_full, t & 1, abort_flag, gp.err, 59)) { ok = false; break; }
         tc_fence_after();
@@ -596,7 +577,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
           const int ei[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (i0 + 4 * j4 + j < gp.m) dst[(long long)(4 * j4 + j) * gp.R] = finish(sum[4 * j4 + j], er, ei[j]);
+            if (i0 + 4 * j4 + j < gp.m) dst[(long long)(4 * j4 + j) * gp.R] = finish<C>(sum[4 * j4 + j], er, ei[j]);
         }
       }
     }
@@ -611,17 +592,18 @@ __global__ void __launch_bounds__(kGThreads, 1)
 }  // namespace
 
 // The levels that have to be exact are summed in the worst case, with the data's
-// digits at their largest and in line with the matrix's: sum over a <= s of
-// 2^{RB - 1} |m_a| for every row and segment (FP32: only P_0, which is within
-// 2^24 over kSegK terms whatever the digits).
-template <typename T>
-int slice_segment(const T* M, int rows, int K) {
-  constexpr int NS = SliceCfg<T>::NS, RB = SliceCfg<T>::RB;
+// digits at their largest and in line with the matrix's: sum over a < s of 128 |m_a|
+// plus 64 |m_s| for every row and segment, most for s = 4 (FP32: levels 0 and 1,
+// within 2^24 over kSegK terms whatever the digits).
+template <class C>
+int slice_segment(const typename C::T* M, int rows, int K) {
+  using T = typename C::T;
+  constexpr int NS = C::NS, RB = C::RB;
   const int chunks = (K + kGK - 1) / kGK;
   int seg = std::min(chunks, kSegK / kGK);
   if (sizeof(T) == 8) {
-    constexpr int kExact = 4;   // levels 0 .. 3
-    // per row and chunk: sum of |m_0| + .. + |m_3|, which bounds the lower levels too
+    constexpr int kExact = 5;   // levels 0 .. 4
+    // per row and chunk: that sum for s = 4, which bounds the levels before it too
     std::vector<int> sum((size_t)rows * chunks, 0);
     for (int i = 0; i < rows; ++i) {
       const T* row = M + (size_t)i * K;
@@ -634,11 +616,11 @@ int slice_segment(const T* M, int rows, int K) {
       for (int k = 0; k < K; ++k) emax = std::max(emax, (int)((bits(row[k]) >> Bits<T>::kMant) & Bits<T>::kExpMask));
       const bool bad = emax == Bits<T>::kExpMask;
       for (int k = 0; k < K; ++k) {
-        const auto w = balanced<T>(bits(row[k]), emax, bad);
+        const auto w = balanced<C>(bits(row[k]), emax, bad);
         for (int a = 0; a < kExact; ++a) {
           const int dig = a == 0 ? (int)(w >> (RB * (NS - 1)))
                                  : ((int)(w >> (RB * (NS - 1 - a))) & ((1 << RB) - 1)) - (1 << (RB - 1));
-          sum[(size_t)i * chunks + k / kGK] += std::abs(dig);
+          sum[(size_t)i * chunks + k / kGK] += (a + 1 < kExact ? 128 : 64) * std::abs(dig);
         }
       }
     }
@@ -649,20 +631,20 @@ int slice_segment(const T* M, int rows, int K) {
         for (int c0 = 0; c0 < chunks && fits; c0 += seg) {
           long long level = 0;
           for (int c = c0; c < std::min(c0 + seg, chunks); ++c) level += sum[(size_t)i * chunks + c];
-          fits = (level << (RB - 1)) <= (1ll << 24);
+          fits = level <= (1ll << 24);
         }
-      if (fits) break;   // at the latest with 8 chunks = 256 terms: 4 x 128 x 128 x 256 = 2^24
+      if (fits) break;   // at the latest with 8 chunks = 256 terms: (64 + 3 x 128 + 64) x 128 x 256 = 2^24
     }
   }
   return seg * kGK;
 }
 
-template <typename T>
+template <class C>
 void slice_map(Sliced& s, bool matrix) {
   const cuuint64_t pitch = (cuuint64_t)slice_pitch(s.K);
-  cuuint64_t dims[3] = {(cuuint64_t)s.K, (cuuint64_t)s.rows, (cuuint64_t)SliceCfg<T>::NS};
+  cuuint64_t dims[3] = {(cuuint64_t)s.K, (cuuint64_t)s.rows, (cuuint64_t)C::NS};
   cuuint64_t strides[2] = {pitch * 2, pitch * 2 * (cuuint64_t)s.rows};
-  cuuint32_t box[3] = {kGK, (cuuint32_t)(matrix ? GemmCfg<T>::NT : kGM), 1};
+  cuuint32_t box[3] = {kGK, (cuuint32_t)(matrix ? C::NT : kGM), 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode_fn()(&s.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, s.dig, dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
@@ -670,9 +652,9 @@ void slice_map(Sliced& s, bool matrix) {
   if (r != CUDA_SUCCESS) throw std::runtime_error("cuTensorMapEncodeTiled (slices) failed (" + std::to_string((int)r) + ")");
 }
 
-template <typename T>
-void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride, const SliceOut<T>& o,
-                cudaStream_t st, long long& nl) {
+template <class C>
+void slice_rows(const typename C::T* X, const Sliced& s, int nseg, int seg_len, long long seg_stride,
+                const SliceOut<typename C::T>& o, cudaStream_t st, long long& nl) {
   const int chunks = nseg * seg_len / 8;
   if (seg_len % 8 == 0 && chunks <= 128) {
     int group = 1;
@@ -680,10 +662,10 @@ void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long se
     const long long per_block = 256 / group;
     const int blocks = (int)std::min<long long>((s.rows + per_block - 1) / per_block, (long long)num_sms() * 32);
     const int it = (chunks + group - 1) / group;
-    launch_pdl(it == 1   ? slice8_kernel<T, 1>
-               : it == 2 ? slice8_kernel<T, 2>
-               : it == 3 ? slice8_kernel<T, 3>
-                         : slice8_kernel<T, 4>,
+    launch_pdl(it == 1   ? slice8_kernel<C, 1>
+               : it == 2 ? slice8_kernel<C, 2>
+               : it == 3 ? slice8_kernel<C, 3>
+                         : slice8_kernel<C, 4>,
                blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group, s.dig, s.ex, o);
     FCGLE_LAUNCHED(nl);
     return;
@@ -692,45 +674,51 @@ void slice_rows(const T* X, const Sliced& s, int nseg, int seg_len, long long se
   const int group = quads <= 8 ? 8 : (quads <= 16 ? 16 : 32);
   const long long per_block = 256 / group;
   const long long blocks = std::min<long long>((s.rows + per_block - 1) / per_block, (long long)num_sms() * 16);
-  launch_pdl(slice_kernel<T>, (int)blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group,
+  launch_pdl(slice_kernel<C>, (int)blocks, 256, 0, st, X, s.rows, nseg, seg_len, seg_stride, slice_pitch(s.K), group,
              s.dig, s.ex, o);
   FCGLE_LAUNCHED(nl);
 }
 
-template <typename T>
-void sliced_gemm(const Sliced& x, const Sliced& m, T* Y, long long R, long long plane, int* err, cudaStream_t st,
-                 long long& nl) {
+template <class C>
+void sliced_gemm(const Sliced& x, const Sliced& m, typename C::T* Y, long long R, long long plane, int* err,
+                 cudaStream_t st, long long& nl) {
   static std::once_flag attr;
   std::call_once(attr, [] {
-    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GemmLayout<T>::kSmem));
-    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GemmLayout<T>::kSmem));
+    for (auto* k : {sliced_gemm_kernel<C, false>, sliced_gemm_kernel<C, true>}) {
+      cudaFuncAttributes a;
+      FCGLE_CUDA(cudaFuncGetAttributes(&a, k));
+      if (a.numRegs < kGRegLaunch)
+        throw std::logic_error("sliced product built with " + std::to_string(a.numRegs) + " registers");
+    }
+    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GemmLayout<C>::kSmem));
+    FCGLE_CUDA(cudaFuncSetAttribute(sliced_gemm_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GemmLayout<C>::kSmem));
   });
   GemmParams gp;
   gp.rows = x.rows;
   gp.R = R;
   gp.plane = plane;
   gp.m = (int)m.rows;
-  gp.m_tiles = (gp.m + GemmCfg<T>::NT - 1) / GemmCfg<T>::NT;
+  gp.m_tiles = (gp.m + C::NT - 1) / C::NT;
   gp.k_chunks = (x.K + kGK - 1) / kGK;
   gp.units = (x.rows + kGM - 1) / kGM * gp.m_tiles;
   gp.seg = m.seg / kGK;
   gp.err = err;
-  launch_pdl(gp.k_chunks <= gp.seg ? sliced_gemm_kernel<T, false> : sliced_gemm_kernel<T, true>,
-             (int)std::min<long long>(gp.units, num_sms()), kGThreads, GemmLayout<T>::kSmem, st, x.tm, m.tm,
+  launch_pdl(gp.k_chunks <= gp.seg ? sliced_gemm_kernel<C, false> : sliced_gemm_kernel<C, true>,
+             (int)std::min<long long>(gp.units, num_sms()), kGThreads, GemmLayout<C>::kSmem, st, x.tm, m.tm,
              (const int*)x.ex, (const int*)m.ex, Y, gp);
   FCGLE_LAUNCHED(nl);
 }
 
-#define INST(T)                                                                                                  \
-  template int slice_segment<T>(const T*, int, int);                                                             \
-  template void slice_map<T>(Sliced&, bool);                                                                     \
-  template void slice_rows<T>(const T*, const Sliced&, int, int, long long, const SliceOut<T>&, cudaStream_t,    \
-                              long long&);                                                                       \
-  template void sliced_gemm<T>(const Sliced&, const Sliced&, T*, long long, long long, int*, cudaStream_t, long long&);
-INST(float)
-INST(double)
+#define INST(C)                                                                                                    \
+  template int slice_segment<C>(const C::T*, int, int);                                                            \
+  template void slice_map<C>(Sliced&, bool);                                                                       \
+  template void slice_rows<C>(const C::T*, const Sliced&, int, int, long long, const SliceOut<C::T>&, cudaStream_t, \
+                              long long&);                                                                         \
+  template void sliced_gemm<C>(const Sliced&, const Sliced&, C::T*, long long, long long, int*, cudaStream_t, long long&);
+INST(Slices32)
+INST(Slices64)
 #undef INST
 
 }  // namespace fcgle

@@ -47,15 +47,16 @@ def _problem(fc, n):
 @pytest.mark.parametrize("n", [1023, 1500])
 def test_digits_in_line(fc, n):
     s, p, R, product, M = _problem(fc, n)
-    # row r: digits 127 in line with those of row i = i_r of M, digit b with level
-    # 3 - b, so that all four products of level 3 have one sign; odd rows: all of one sign
+    # row r: digits as large as they come and in line with those of row i = i_r of M,
+    # digit b with level 4 - b, so that all five products of level 4 have one sign; odd
+    # rows: all of one sign
     rows = np.linspace(0, n - 1, 2 * R).astype(int)
     dig = _digits(M[rows])
     X = np.zeros((2 * R, p))
     for r in range(2 * R):
-        for b in range(4):
-            sgn = np.where(dig[3 - b, r] < 0, -1.0, 1.0) if r % 2 == 0 else np.ones(p)
-            X[r] += 127.0 * sgn * 2.0 ** (-8 * b)
+        for b in range(5):
+            sgn = np.where(dig[4 - b, r] < 0, -1.0, 1.0) if r % 2 == 0 else np.ones(p)
+            X[r] += (127.0 if b else 63.0) * sgn * 2.0 ** (-8 * b)
     X[:, n:] = 0.0
     Y = product(X)
     T = X.astype(np.longdouble) @ M.astype(np.longdouble).T
@@ -78,7 +79,7 @@ def test_exact_sums_round_once(fc, n, terms):
     ok = np.zeros((2 * R, p), bool)
     for r in range(2 * R):
         k = rng.permutation(np.flatnonzero(big[rng.integers(0, n)]))[:terms]   # one output at least qualifies
-        X[r, k] = 127.0 / 64.0 * np.where(M[rng.integers(0, n), k] < 0, -1.0, 1.0)
+        X[r, k] = 63.0 / 32.0 * np.where(M[rng.integers(0, n), k] < 0, -1.0, 1.0)
         ok[r] = big[:, k].all(axis=1)
     ok[:, n:] = False
     assert ok.any(axis=1).all()

@@ -9,25 +9,32 @@ import pytest
 
 
 def _digits(M):
-    """Balanced digits of every entry, 7 of 8 bits, one exponent per row (python integers)."""
-    out = np.zeros((7,) + M.shape, dtype=np.int64)
-    off = sum(1 << (8 * j + 7) for j in range(6))
+    """Balanced digits of every entry, 8 of 8 bits, one exponent per row (python integers)."""
+    out = np.zeros((8,) + M.shape, dtype=np.int64)
+    off = sum(1 << (8 * j + 7) for j in range(7))
     for i, row in enumerate(M):
         top = np.max(np.abs(row))
         if top == 0.0:
             w = [off] * row.size
         else:
             e = math.frexp(top)[1]
-            # 55 bits below the leading power of two, half away from zero
-            w = [int(math.copysign(math.floor(abs(math.ldexp(x, 55 - e)) + 0.5), x)) + off for x in row]
-        for a in range(7):
-            out[a, i] = [v >> 48 if a == 0 else ((v >> (8 * (6 - a))) & 255) - 128 for v in w]
+            # 62 bits below the leading power of two, half away from zero (integer arithmetic:
+            # 62 bits do not fit a double)
+            w = []
+            for x in row:
+                m, ex = math.frexp(x)
+                n, sh = int(math.ldexp(abs(m), 53)), 62 - 53 - (e - ex)
+                n = n << sh if sh >= 0 else (n + (1 << (-sh - 1))) >> -sh
+                w.append((n if x >= 0 else -n) + off)
+        for a in range(8):
+            out[a, i] = [v >> 56 if a == 0 else ((v >> (8 * (7 - a))) & 255) - 128 for v in w]
     return out
 
 
 def _level(dig, seg):
-    """The largest |P_0| .. |P_3| any data can give: all partners 128 and in line."""
-    s = 128 * np.abs(dig[:4]).sum(axis=0)
+    """The largest |P_0| .. |P_4| any data can give: all partners at their largest (128, the
+    top digit 64) and in line."""
+    s = 128 * np.abs(dig[:4]).sum(axis=0) + 64 * np.abs(dig[4])
     return max(int(s[:, k:k + seg].sum(axis=1).max()) for k in range(0, s.shape[1], seg))
 
 
