@@ -406,8 +406,8 @@ class Engine : public EngineBase {
       slice_rows<Slices64>(M, s, 1, K, 0, SliceOut<double>{}, st, nl);
     }
   };
-  // The sliced product (two launches) against the CUDA cores, us: 12.6 / 21.0 at
-  // K = 16 with 32 rows, 15.0 / 70 at 64 x 64, 18 / 150 at K = 132 with 8 rows;
+  // The sliced product (two launches) against the CUDA cores, us: 11.9 / 20.5 at
+  // K = 16 with 32 rows, 14.8 / 70 at 64 x 64, 20 / 150 at K = 132 with 8 rows;
   // shorter contractions are one k-step of the CUDA-core tile and stay there.
   static bool sliceable(int K, long long rows) { return kF64 && K >= 16 && rows < (1ll << 31); }
   // one mode product: cx = 0 with the real matrix m of order p, cx = 1 with the
